@@ -12,6 +12,7 @@
 #include "dpf_internal.h"
 #include "dpf_kernels.cuh"
 #include "dpf_dc.cuh"
+#include "dpf_resident.h"
 
 using namespace dpf;
 
@@ -110,7 +111,57 @@ static void free_device(DeviceYbus& d) {
   dfree(d.type); dfree(d.p64); dfree(d.q64); dfree(d.vmset); dfree(d.p32); dfree(d.q32);
   dfree(d.perm); dfree(d.iperm); dfree(d.br_f); dfree(d.br_t); dfree(d.br_r); dfree(d.br_x);
   dfree(d.br_bch); dfree(d.br_tap); dfree(d.br_itap); dfree(d.bridge);
+  dfree(d.res_rord); dfree(d.res_rpos); dfree(d.res_soff); dfree(d.res_col2); dfree(d.res_val32); dfree(d.res_val64);
   d.ready = false;
+}
+
+// Sliced ELL form of Y_bus for the on-chip iterations (see DeviceYbus).  Rows
+// of equal entry count follow each other, pq and pv buses apart, so that the
+// 32 rows of a slice take the same branches.
+struct SellY {
+  std::vector<int32_t> rord, rpos, soff;
+  std::vector<uint32_t> col2;
+  std::vector<float2> val32;
+  std::vector<double2> val64;
+};
+static void build_sell(const dpf_ybus* y, SellY& q) {
+  const int n = y->n;
+  const std::vector<int32_t>& rp = y->irow_ptr;
+  q.rord.resize(n);
+  q.rpos.resize(n);
+  for (int i = 0; i < n; ++i) q.rord[i] = i;
+  auto len = [&](int i) { return rp[i + 1] - rp[i]; };
+  std::stable_sort(q.rord.begin(), q.rord.end(), [&](int i, int j) {
+    if (len(i) != len(j)) return len(i) > len(j);
+    return y->bus_type[y->perm[i]] < y->bus_type[y->perm[j]];
+  });
+  for (int p = 0; p < n; ++p) q.rpos[q.rord[p]] = p;
+  const int slices = (n + 31) / 32;
+  q.soff.assign(slices + 1, 0);
+  for (int s = 0; s < slices; ++s) {
+    int mx = 0;
+    for (int p = s * 32; p < std::min(n, s * 32 + 32); ++p) mx = std::max(mx, len(q.rord[p]));
+    q.soff[s + 1] = q.soff[s] + (mx + 1) / 2;
+  }
+  const int pairs = q.soff[slices];
+  q.col2.assign((size_t)pairs * 32, 0);
+  q.val32.assign((size_t)pairs * 64, make_float2(0.f, 0.f));
+  q.val64.assign((size_t)pairs * 64, make_double2(0.0, 0.0));
+  for (int s = 0; s < slices; ++s)
+    for (int l = 0; l < 32; ++l) {
+      const int p = s * 32 + l, i = p < n ? q.rord[p] : -1;
+      for (int e = 0; e < 2 * (q.soff[s + 1] - q.soff[s]); ++e) {
+        int c = p < n ? p : 0;  // a pad: weight 0 on the row itself
+        if (i >= 0 && e < len(i)) {
+          const int t = rp[i] + e;
+          c = q.rpos[y->icol[t]];
+          const size_t at = ((size_t)(q.soff[s] + e / 2) * 32 + l) * 2 + (e & 1);
+          q.val32[at] = make_float2((float)y->ival_re[t], (float)y->ival_im[t]);
+          q.val64[at] = make_double2(y->ival_re[t], y->ival_im[t]);
+        }
+        q.col2[(size_t)(q.soff[s] + e / 2) * 32 + l] |= (uint32_t)(c * 8) << (16 * (e & 1));
+      }
+    }
 }
 
 extern "C" int dpf_ybus_upload(dpf_ybus* y, void* stream) {
@@ -175,8 +226,20 @@ extern "C" int dpf_ybus_upload(dpf_ybus* y, void* stream) {
     const double dii = dcval[y->idpos[i]];
     dcinv2[i] = pair(dii != 0.0 ? 1.0 / dii : 0.0);
   }
+  SellY sell;
+  if (n <= RES_MAX_N) build_sell(y, sell);
   int rc = DPF_OK;
   do {
+    if (n <= RES_MAX_N) {
+      if ((rc = upload(&d.res_rord, sell.rord, s))) break;
+      if ((rc = upload(&d.res_rpos, sell.rpos, s))) break;
+      if ((rc = upload(&d.res_soff, sell.soff, s))) break;
+      if ((rc = upload(&d.res_col2, sell.col2, s))) break;
+      if ((rc = upload(&d.res_val32, sell.val32, s))) break;
+      if ((rc = upload(&d.res_val64, sell.val64, s))) break;
+      d.res_slices = (int)sell.soff.size() - 1;
+      d.res_pairs = sell.soff.back();
+    }
     if ((rc = upload(&d.ent32, ent, s))) break;
     if ((rc = upload(&d.row_ptr, y->irow_ptr, s))) break;
     if ((rc = upload(&d.prow_ptr, y->iprow_ptr, s))) break;
@@ -295,6 +358,8 @@ struct dpf_workspace {
   bool direct = false;    // single-case FP32 solve: Y rows read from global memory (no staging)
   int4* pent = nullptr;   // padded Y entries of the direct view
   size_t cap_pent = 0;
+  ResShape res;            // on-chip iterations (res.ok), their launch shape
+  LossOrder res_lo;
   bool pid_ready = false;  // operating points staged by dpf_paramid_begin
   std::vector<std::pair<std::vector<long long>, std::vector<int>>> tune_cache;  // key -> (lanes, warps, rb, pairs)
   bool spec_per_case = false, has_outage = false;
@@ -729,6 +794,19 @@ static int launch_iteration(dpf_workspace* w, cudaStream_t s, bool with_check) {
   return DPF_OK;
 }
 
+// n iterations on chip (after the FP64 test, if due): one launch.
+static int launch_resident(dpf_workspace* w, cudaStream_t s, int n) {
+  const bool pdl = w->opts.pdl != 0;
+  int e;
+  if (w->precision == DPF_FP64)
+    e = res_launch<double>(w->y, make_plan<double>(w).it, w->res, w->res_lo, w->K, n, false, pdl, s);
+  else
+    e = res_launch<float>(w->y, make_plan<float>(w).it, w->res, w->res_lo, w->K, n, w->precision == DPF_FP32R, pdl, s);
+  CK((cudaError_t)e);
+  w->launches++;
+  return DPF_OK;
+}
+
 static int launch_iteration_any(dpf_workspace* w, cudaStream_t s, bool with_check) {
   return w->precision == DPF_FP64 ? launch_iteration<double>(w, s, with_check)
                                   : launch_iteration<float>(w, s, with_check);
@@ -736,6 +814,17 @@ static int launch_iteration_any(dpf_workspace* w, cudaStream_t s, bool with_chec
 static int launch_check_any(dpf_workspace* w, cudaStream_t s, bool final_pass) {
   return w->precision == DPF_FP64 ? launch_check<double>(w, s, final_pass)
                                   : launch_check<float>(w, s, final_pass);
+}
+
+// n iterations, the FP64 test first if with_check; on chip where the grid fits
+// (not while the forward and adjoint passes are timed one by one).
+static int launch_span(dpf_workspace* w, cudaStream_t s, int n, bool with_check) {
+  if (w->res.ok && !w->profile) {
+    if (with_check) TRY(launch_check_any(w, s, false));
+    return launch_resident(w, s, n);
+  }
+  for (int i = 0; i < n; ++i) TRY(launch_iteration_any(w, s, with_check && i == 0));
+  return DPF_OK;
 }
 
 // Capture one check interval (FP64 test + check_every iterations) as a graph.
@@ -747,7 +836,7 @@ static int build_graph(dpf_workspace* w) {
   w->profile = false;
   CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
   int rc = DPF_OK;
-  for (int i = 0; i < w->opts.check_every && rc == DPF_OK; ++i) rc = launch_iteration_any(w, cs, i == 0);
+  rc = launch_span(w, cs, w->opts.check_every, true);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(cs, &g);
   if (rc != DPF_OK) {
@@ -922,6 +1011,26 @@ static void choose_shape(dpf_workspace* w, const dpf_solve_opts* o, int K) {
     w->h_wlo[b] = lo;
     w->h_whi[b] = hi;
   }
+}
+
+// The on-chip form of the iterations, where the grid's per-case state fits one
+// SM (after choose_shape, whose row blocks give the order of the loss sum).
+// An explicit request for staged rows or windows (stage_y, stage_v) and the
+// plain form keep the streaming kernels.
+static void choose_resident(dpf_workspace* w, const dpf_solve_opts* o) {
+  w->res = ResShape();
+  if (o->plain || o->stage_v || o->stage_y || w->precision == DPF_MIXED) return;
+  int dev = 0, lim = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  LossOrder& lo = w->res_lo;
+  lo.gy = w->gy;
+  lo.rpb = w->rpb;
+  lo.wpb = w->warps;
+  lo.rpw = 32 / w->lanes;
+  lo.tile = w->pair_fwd ? 64 : w->lanes;
+  lo.nthr = w->warps * 32;
+  w->res = res_shape(w->y, w->K, w->precision == DPF_FP64, w->precision == DPF_FP32R, lo, (size_t)lim);
 }
 
 // Device copies of the row-block windows (after choose_shape), and zeroed
@@ -1367,6 +1476,7 @@ extern "C" int dpf_solve_begin(const dpf_ybus* y, dpf_workspace* w, const dpf_ba
   w->precision = o->precision;
   w->use_local_y = false;
   choose_shape(w, o, w->K);
+  choose_resident(w, o);
   TRY(upload_windows(w, s));
   TRY(w->precision == DPF_FP64 ? set_smem_attr<double>(std::max(w->smem, w->ysmem_b))
                                : set_smem_attr<float>(std::max(w->smem, w->ysmem_b)));
@@ -1450,9 +1560,10 @@ extern "C" int dpf_solve_iterate(dpf_workspace* w, int32_t n_iter, void* stream)
       w->t_done += ce;
       n_iter -= ce;
     } else {
-      TRY(launch_iteration_any(w, s, w->t_done % ce == 0));
-      w->t_done += 1;
-      n_iter -= 1;
+      const int n = std::min(n_iter, ce - w->t_done % ce);  // up to the next test
+      TRY(launch_span(w, s, n, w->t_done % ce == 0));
+      w->t_done += n;
+      n_iter -= n;
     }
   }
   return DPF_OK;
@@ -1794,7 +1905,19 @@ extern "C" int dpf_autotune(const dpf_ybus* y, dpf_workspace* w, const dpf_batch
   base.pair_cases = 0;
   base.stage_v = 0;
   base.stage_y = 0;
-  choose_shape(w, &base, K);
+  // a grid whose iterations run on chip has one shape (the options below only
+  // give the order of its loss sum): nothing to time
+  TRY(dpf_solve_begin(y, w, b, &base, s));
+  if (w->res.ok) {
+    w->begun = false;
+    o->lanes = auto_lanes;
+    o->warps = 8;
+    o->row_blocks = 0;
+    o->stage_v = 0;
+    o->stage_y = 0;
+    w->tune_cache.push_back({key, {auto_lanes, 8, 0, o->pair_cases, 0, 0}});
+    return DPF_OK;
+  }
   // single-case FP32 solves: global-memory or staged Y rows
   std::vector<int> sy_c = {0};
   if (auto_lanes == 1 && (o->precision == DPF_FP32 || o->precision == DPF_FP32R)) sy_c = {0, 1};

@@ -56,6 +56,15 @@ struct DeviceYbus {
   double* br_tap = nullptr;
   double* br_itap = nullptr;    // [m] 1 / tap (tap 0 read as 1): no division on the device
   uint8_t* bridge = nullptr;    // [m]
+  // Y_bus as sliced ELL for the on-chip iterations (n <= RES_MAX_N, else
+  // NULL): rows sorted by entry count, 32 rows per slice, entries in pairs
+  int32_t* res_rord = nullptr;  // [n] position -> internal row
+  int32_t* res_rpos = nullptr;  // [n] internal row -> position
+  int32_t* res_soff = nullptr;  // [slices + 1] entry pairs before a slice
+  uint32_t* res_col2 = nullptr; // [pairs][32] two columns (position * 8, 16 bits each)
+  float2* res_val32 = nullptr;  // [pairs][32][2]
+  double2* res_val64 = nullptr;
+  int res_pairs = 0, res_slices = 0;
 };
 
 }  // namespace dpf

@@ -1119,7 +1119,7 @@ __global__ void __launch_bounds__(256, DPF_ADJ_MINB) k_adj(IterArgs<R> a) {
 
 // Padded entries of the direct view: slot p of the padded rows gets its
 // CSR entry {col, re, im}, a pad {row, 0, 0} (weight 0 on its own row).
-__global__ void k_pad_entries(const int32_t* __restrict__ ppos, const int4* __restrict__ ent, int n_pad,
+static __global__ void k_pad_entries(const int32_t* __restrict__ ppos, const int4* __restrict__ ent, int n_pad,
                               int4* __restrict__ pent) {
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n_pad; p += gridDim.x * blockDim.x) {
     const int pos = ppos[p];
@@ -1142,7 +1142,7 @@ __global__ void k_pad_entries(const int32_t* __restrict__ ppos, const int4* __re
 // weights c and w = c conj(V) in FP64; it hands the FP32 adjoint w, Q_calc at
 // pv buses and the loss partials in FP32 (the gradient needs no more: near
 // convergence its error is relative to the small mismatch it is built from).
-__global__ void __launch_bounds__(256, 4) k_fwd_mixed(IterArgs<float> a) {
+static __global__ void __launch_bounds__(256, 4) k_fwd_mixed(IterArgs<float> a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const BMap mp = block_map(a.lanes, a.N, a.rpb);
   YSmem<double> ys;
@@ -1202,7 +1202,7 @@ __global__ void __launch_bounds__(256, 4) k_fwd_mixed(IterArgs<float> a) {
 }
 
 // FP64 voltages from the double-float master (mixed precision set-up).
-__global__ void k_mixed_v64(const float4* __restrict__ ms, double2* __restrict__ v, size_t n) {
+static __global__ void k_mixed_v64(const float4* __restrict__ ms, double2* __restrict__ v, size_t n) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
     const float4 s = ms[e];
     v[e] = volt64(ms_th(s), ms_vm(s));
@@ -1633,7 +1633,7 @@ struct ApplyArgs {
   int32_t* n_active;
 };
 
-__global__ void k_apply(ApplyArgs a) {
+static __global__ void k_apply(ApplyArgs a) {
   __shared__ int cnt[32];
   pdl_wait();
   pdl_release();
@@ -1673,7 +1673,7 @@ __global__ void k_apply(ApplyArgs a) {
 // V buffer holds dV = V) until the case's first FP64 test.  f_ref = -S_spec
 // (pv buses: Q_calc(V_ref) = 0).  p, q: FP32 specification, [N][Kp] if
 // per_case, else [N].
-__global__ void k_ref_init(const uint8_t* __restrict__ type, const float* __restrict__ p,
+static __global__ void k_ref_init(const uint8_t* __restrict__ type, const float* __restrict__ p,
                            const float* __restrict__ q, int per_case, int Kp, size_t n, float2* __restrict__ vref,
                            float4* __restrict__ irf) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
@@ -1686,7 +1686,7 @@ __global__ void k_ref_init(const uint8_t* __restrict__ type, const float* __rest
 }
 
 // Re-activate the first K of Kp cases (a final convergence pass deactivates all).
-__global__ void k_activate(int32_t* __restrict__ active, int K, int Kp) {
+static __global__ void k_activate(int32_t* __restrict__ active, int K, int Kp) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < Kp) active[k] = (k < K) ? 1 : 0;
 }
@@ -1694,7 +1694,7 @@ __global__ void k_activate(int32_t* __restrict__ active, int K, int Kp) {
 // ---- set-up / tear-down ----------------------------------------------------
 // Tiled transpose of a case-major [K][N] user-order FP64 array into the
 // case-minor internal layout [N][Kp] (row iperm[u] for user bus u).
-__global__ void k_to_internal(const double* __restrict__ src, double* __restrict__ dst, int K, int N,
+static __global__ void k_to_internal(const double* __restrict__ src, double* __restrict__ dst, int K, int N,
                               int Kp, const int32_t* __restrict__ iperm) {
   __shared__ double tile[32][33];
   const int u0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
@@ -1710,7 +1710,7 @@ __global__ void k_to_internal(const double* __restrict__ src, double* __restrict
 }
 
 // Inverse of k_to_internal.
-__global__ void k_to_user(const double* __restrict__ src, double* __restrict__ dst, int K, int N, int Kp,
+static __global__ void k_to_user(const double* __restrict__ src, double* __restrict__ dst, int K, int N, int Kp,
                           const int32_t* __restrict__ iperm) {
   __shared__ double tile[32][33];
   const int u0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
@@ -1895,7 +1895,7 @@ struct YValArgs {
   double2* val64;
 };
 
-__global__ void k_ybus_values(YValArgs a) {
+static __global__ void k_ybus_values(YValArgs a) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.N) return;
   double dr = 0.0, di = 0.0;

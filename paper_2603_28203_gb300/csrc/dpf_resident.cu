@@ -1,0 +1,836 @@
+// On-chip form of the DPF iterations for grids of up to RES_MAX_N buses.
+//
+// The streaming kernels (k_fwd, k_adj) pass a batch's whole state through
+// HBM / L2 twice per iteration: 128 bytes per element and iteration in the
+// refined mode.  But the cases are independent, and the state of one case of
+// such a grid fits one SM.  Here a team of threads owns one case for a whole
+// test interval: it loads the case's state once, runs the iterations with the
+// master values, the moments and the references in registers and V (or dV), w
+// and the mismatch in shared memory, and stores the state back once.  No
+// barrier spans more than the team.
+//
+//   one warp per case (N <= RES_WARP_N, RES_TEAMS cases per CTA): warp
+//   barriers only; the warp also sums the loss and steps the scheduler.
+//   one CTA per case (larger N): T compute threads with RPT rows each plus
+//   one warp that sums the loss and steps the case's scheduler while the
+//   others run the adjoint gathers.
+//
+// Y_bus is staged once per CTA as sliced ELL: rows sorted by their entry
+// count, 32 rows per slice, entry e of a slice's 32 rows adjacent, so a
+// slice's rows have (nearly) equal lengths and the value and column loads are
+// free of bank conflicts.  Shared-memory vectors are indexed by position in
+// that order.
+//
+// Measured (2,379 N-1 cases of a 2,000-bus grid, refined FP32): 123 us per
+// iteration streaming, 84 us on chip.  What bounds it now is instruction issue
+// (62% of the slots, 434 instructions per 32 rows and iteration), then the
+// shared-memory pipe (57%: two rows of 8-byte gathers at random banks).  8,192
+// cases of 30 buses: 15.9 -> 8.8 us; one case of 30 buses in FP64: 17.8 -> 9.0.
+//
+// The results are those of the streaming kernels to the bit: the same device
+// functions on the same operands, each row's products in the same order, and
+// the case's loss (which drives the plateau schedule) summed in the order of
+// the launch shape the streaming kernels would use (LossOrder).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "dpf_kernels.cuh"
+#include "dpf_resident.h"
+
+namespace dpf {
+
+// Threads of a CTA at most in the one-CTA form (FP64 needs the registers).
+template <class R> __host__ __device__ constexpr int res_threads() { return sizeof(R) == 4 ? 1024 : 512; }
+
+// Geometry of the loss sum (LossOrder with what is empty left out: adding an
+// empty chain's 0 changes nothing).  Chain (b, w, r) holds the rows b*rpb +
+// w*rpw + r + j*step of row block b.
+struct LossGeo {
+  int gy, rpb, wpb, rpw, lrpw, step, nj, nch, magic, tile, nthr;
+};
+// Shared-memory layout: X, W, the specification and (CTA form, refined mode)
+// the references by position, D = (dP, dQ) by internal row, scratch; then the
+// staged Y_bus.
+struct ResLayout {
+  unsigned w, d, s, vr, rf, scr, sc, flag, team;  // offsets inside a team's block, its size
+  unsigned val, col, soff, total;             // after the teams
+};
+template <class R> struct ValPair;
+template <class R> struct ResArgs {
+  using C = typename Prec<R>::C;
+  IterArgs<R> a;
+  int K, T, n_it;
+  const int32_t* rord;    // position -> internal row
+  const int32_t* rpos;    // internal row -> position
+  const int32_t* soff;    // [slices + 1] entry pairs before a slice
+  const uint32_t* col2;   // two column byte offsets (position * 8) per word, [pair][32]
+  const ValPair<R>* val;  // [pair][32]
+  int n_pair;             // entry pairs of all slices
+  int n_slice;
+  LossGeo lo;
+  ResLayout L;
+};
+
+// Scratch values of the loss sum.
+__host__ __device__ __forceinline__ int res_scratch(const LossGeo& g) {
+  return g.gy * g.wpb + g.gy + (g.gy + SCHED_GROUP - 1) / SCHED_GROUP + 256 + 16;
+}
+
+// One case's loss sum in the streaming kernels' order, in two parts.  Chains:
+// warp `cw` of `ncw` sums its chains' rows and the butterfly over a warp's
+// rows into part.  Tail (one warp): the warps, the row blocks and (beyond 64)
+// their groups.  FP64 solves, whose plateau decisions do not hang on the last
+// bit, take a shorter fixed order: strided rows, then a butterfly.
+template <class R, class C>
+__device__ __forceinline__ void loss_chains(const C* __restrict__ D, R* __restrict__ part, int N, const LossGeo& g,
+                                            int cw, int ncw, int lane) {
+  if constexpr (sizeof(R) == 8) {
+    R s = R(0);
+    for (int i = cw * 32 + lane; i < N; i += 32 * ncw) {
+      const C d = D[i];
+      s = fmaT(d.x, d.x, fmaT(d.y, d.y, s));
+    }
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) part[cw] = s;
+  } else {
+    for (int c0 = cw * 32; c0 < g.nch; c0 += ncw * 32) {
+      const int c = c0 + lane, bw = c >> g.lrpw;
+      const int b = (int)(((unsigned)bw * (unsigned)g.magic) >> 18);  // bw / wpb
+      int i = b * g.rpb + ((bw - b * g.wpb) << g.lrpw) + (c & (g.rpw - 1));
+      const int r1 = c < g.nch ? min(N, (b + 1) * g.rpb) : 0;
+      R acc = R(0);
+      if (g.nj == 1) {
+        if (i < r1) {
+          const C d = D[i];
+          acc = fmaT(d.x, d.x, fmaT(d.y, d.y, R(0)));
+        }
+      } else {
+        for (; i < r1; i += 4 * g.step) {  // four rows' loads in flight; a missing row adds 0
+          C d[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) d[u] = i + u * g.step < r1 ? D[i + u * g.step] : mkc(R(0), R(0));
+#pragma unroll
+          for (int u = 0; u < 4; ++u) acc = fmaT(d[u].x, d[u].x, fmaT(d[u].y, d[u].y, acc));
+        }
+        __syncwarp();
+      }
+      for (int off = g.rpw >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+      if (c < g.nch && (c & (g.rpw - 1)) == 0) part[bw] = acc;
+    }
+  }
+}
+
+template <class R>
+__device__ __forceinline__ R loss_tail(R* __restrict__ scr, const LossGeo& g, int ncw, int lane) {
+  R L = R(0);
+  if constexpr (sizeof(R) == 8) {
+    for (int c = 0; c < ncw; ++c) L += scr[c];
+  } else {
+    const int nbw = g.gy * g.wpb;
+    const R* sums = scr;
+    R* blk = scr + ((nbw + 3) & ~3);
+    R* grp = blk + ((g.gy + 3) & ~3);
+    if (g.wpb > 1) {
+      for (int b = lane; b < g.gy; b += 32) {
+        const R* pb = scr + b * g.wpb;
+        R s = R(0);
+        if (g.wpb == 8) {
+          const float4 u = *reinterpret_cast<const float4*>(pb), v = *reinterpret_cast<const float4*>(pb + 4);
+          s = ((((((((s + u.x) + u.y) + u.z) + u.w) + v.x) + v.y) + v.z) + v.w);
+        } else {
+          for (int w = 0; w < g.wpb; ++w) s += pb[w];
+        }
+        blk[b] = s;
+      }
+      __syncwarp();
+      sums = blk;
+    }
+    if (g.gy <= 64) {
+      int b = 0;
+      for (; b + 4 <= g.gy; b += 4) {
+        const float4 u = *reinterpret_cast<const float4*>(sums + b);
+        L = (((L + u.x) + u.y) + u.z) + u.w;
+      }
+      for (; b < g.gy; ++b) L += sums[b];
+    } else {
+      const int ng = (g.gy + SCHED_GROUP - 1) / SCHED_GROUP;
+      for (int q = lane; q < ng; q += 32) {
+        R s = R(0);
+        for (int u = 0; u < SCHED_GROUP; ++u) s += (q * SCHED_GROUP + u < g.gy) ? sums[q * SCHED_GROUP + u] : R(0);
+        grp[q] = s;
+      }
+      __syncwarp();
+      int tpc = 1;
+      while (2 * tpc * g.tile <= g.nthr) tpc *= 2;
+      R* tree = grp + ng;
+      for (int j = lane; j < tpc; j += 32) {
+        R s = R(0);
+        for (int q = j; q < ng; q += tpc) s += grp[q];
+        tree[j] = s;
+      }
+      __syncwarp();
+      for (int st = tpc >> 1; st > 0; st >>= 1) {
+        for (int j = lane; j < st; j += 32) tree[j] += tree[j + st];
+        __syncwarp();
+      }
+      L = tree[0];
+    }
+  }
+  __syncwarp();  // the scratch is reused by the next iteration
+  return L;
+}
+
+// The scheduler of one case, run by one warp with its state in registers (the
+// same decisions and values as sched_case).  FP64 issue is dear on GB300, so
+// in FP32 solves a step takes two FP64 operations: lane 0 carries beta1^t,
+// lane 1 beta2^t; the plateau test compares the FP32 loss sums and falls back
+// to the FP64 comparison only where they are within 1e-6 of the threshold;
+// the step schedule's power is taken when its exponent changes.
+template <class R> struct ResSched {
+  double lr, best, bt;    // bt: lane 0 beta1^t, lane 1 beta2^t
+  float bsum;             // FP32: the loss sum behind `best` (< 0: best as loaded)
+  float tsum;             // FP32: bsum (1 - threshold), approximately (< 0: not usable)
+  R lrw;                  // lr in working precision
+  int bad, cool, it;
+  R step, isb;            // of the update numbered it + 1
+  __device__ __forceinline__ void load(const SchedArgs<R>& s, int k, int lane) {
+    lr = s.lr[k];
+    lrw = (R)lr;
+    best = s.best[k];
+    bt = lane == 0 ? s.b1t[k] : s.b2t[k];
+    bad = s.bad[k];
+    cool = s.cool[k];
+    it = s.iters[k];
+    bsum = tsum = -1.f;
+    step = isb = R(1);
+  }
+  // the powers of update it + 1 and its bias corrections (independent of the loss)
+  __device__ __forceinline__ void terms(const SchedArgs<R>& s, int lane) {
+    step = lrw;
+    isb = R(1);
+    bt *= lane == 0 ? s.beta1 : s.beta2;
+    if (s.opt == OPT_ADAM) {
+      const R om = R(1) - (R)bt;
+      step = lrw / __shfl_sync(0xffffffffu, om, 0);
+      isb = R(1) / sqrtT(__shfl_sync(0xffffffffu, om, 1));
+    }
+  }
+  // the decision of sched_case on this iterate's loss
+  __device__ __forceinline__ bool improved(const SchedArgs<R>& s, R lsum) {
+    if constexpr (sizeof(R) == 4) {
+      if (tsum > 1e-30f) {
+        if (lsum < tsum * (1.f - 1e-6f)) return true;
+        if (lsum > tsum * (1.f + 1e-6f)) return false;
+      }
+      if (bsum >= 0.f) best = (double)bsum * s.inv_m;
+    }
+    return (double)lsum * s.inv_m < best * (1.0 - s.threshold);
+  }
+  __device__ __forceinline__ void feed(const SchedArgs<R>& s, R lsum) {
+    it += 1;
+    if (s.sched == SCHED_PLATEAU) {
+      if (improved(s, lsum)) {
+        if constexpr (sizeof(R) == 4) {
+          bsum = lsum;
+          const float f = 1.f - (float)s.threshold;
+          tsum = f > 1e-3f ? lsum * f : -1.f;
+        } else {
+          best = (double)lsum * s.inv_m;
+        }
+        bad = 0;
+      } else {
+        bad += 1;
+      }
+      if (cool > 0) { cool -= 1; bad = 0; }
+      if (bad > s.patience) {
+        const double nl = fmax(lr * s.factor, s.min_lr);
+        if (lr - nl > 1e-8) lr = nl;
+        lrw = (R)lr;
+        cool = s.cooldown;
+        bad = 0;
+      }
+    } else if (s.sched == SCHED_STEP && it % s.step_every == 0) {
+      double gk = 1.0, base = s.gamma;
+      for (int e = it / s.step_every; e > 0; e >>= 1) {
+        if (e & 1) gk *= base;
+        base *= base;
+      }
+      lr = s.lr0 * gk;
+      lrw = (R)lr;
+    }
+  }
+  // after the last step (bt is that step's power, step / isb its terms)
+  __device__ __forceinline__ void store(const SchedArgs<R>& s, int k, int lane) {
+    if (lane == 1) s.b2t[k] = bt;
+    if (lane) return;
+    s.lr[k] = lr;
+    s.b1t[k] = bt;
+    s.iters[k] = it;
+    s.step_size[k] = step;
+    s.isbc2[k] = isb;
+    if (s.sched == SCHED_PLATEAU) {
+      if (bsum >= 0.f) best = (double)bsum * s.inv_m;
+      s.best[k] = best;
+      s.bad[k] = bad;
+      s.cool[k] = cool;
+    }
+  }
+};
+
+// Two adjacent entries of a row: their values, one aligned access.
+template <class R> struct __align__(16) ValPair { typename Prec<R>::C a, b; };
+
+// sum_e val[e] x[col[e]] over a row's entry pairs: even entries into a0, odd
+// into a1, as row_spmv does (pads: weight 0 on the row itself).
+template <class R>
+__device__ __forceinline__ typename Prec<R>::C sell_row(const ValPair<R>* __restrict__ val,
+                                                        const uint32_t* __restrict__ col2, int p0, int p1,
+                                                        const unsigned char* __restrict__ X) {
+  using C = typename Prec<R>::C;
+  constexpr unsigned sc = sizeof(C) / 8;
+  C a0 = mkc(R(0), R(0)), a1 = a0;
+  for (int p = p0; p < p1; p += 32) {
+    const uint32_t cc = col2[p];
+    const ValPair<R> y = val[p];
+    const C x0 = *reinterpret_cast<const C*>(X + (cc & 0xffffu) * sc);
+    const C x1 = *reinterpret_cast<const C*>(X + (cc >> 16) * sc);
+    cfma(a0, y.a, x0);
+    cfma(a1, y.b, x1);
+  }
+  return mkc(a0.x + a1.x, a0.y + a1.y);
+}
+
+// One row of a case held by a thread: master values and moments.
+template <class R> struct ResRow {
+  typename Prec<R>::M th, vm;
+  R m1, v1, m2, v2;
+  __device__ __forceinline__ void load(const IterArgs<R>& a, size_t e) {
+    const typename Prec<R>::MS ms = a.ms[e];
+    th = ms_th(ms);
+    vm = ms_vm(ms);
+    const Mom<R> o = mom_load(a.os + e);
+    m1 = o.m1;
+    v1 = o.v1;
+    m2 = o.m2;
+    v2 = o.v2;
+  }
+  __device__ __forceinline__ void store(const IterArgs<R>& a, size_t e) const {
+    a.ms[e] = ms_make(th, vm);
+    mom_store(a.os + e, Mom<R>{m1, v1, m2, v2});
+  }
+};
+
+// Forward epilogue of one row (the arithmetic of fwd_body): I = Y V (refined:
+// Y dV) with the outage taken out, x the gathered vector's own value, sp the
+// specification; returns (dP, dQ), w and Q_calc.
+template <class R, bool REF>
+__device__ __forceinline__ typename Prec<R>::C res_fwd(const IterArgs<R>& a, int ty, typename Prec<R>::C x,
+                                                       typename Prec<R>::C I, typename Prec<R>::C sp, float2 vr,
+                                                       float4 rf, typename Prec<R>::C& w, R& Q, float& mx) {
+  using C = typename Prec<R>::C;
+  C v;
+  R dP, dQ;
+  if constexpr (REF) {
+    const float2 d = refined_mismatch(x, I, vr, rf, v);
+    dP = (ty != BUS_SLACK) ? d.x : R(0);
+    dQ = (ty == BUS_PQ) ? d.y : R(0);
+    Q = d.y;
+  } else {
+    v = x;
+    const C S = power_of(v, I);
+    Q = S.y;
+    dP = (ty != BUS_SLACK) ? S.x - sp.x : R(0);
+    dQ = (ty == BUS_PQ) ? Q - sp.y : R(0);
+  }
+  const R ca = a.inv_m2 * dP, cb = a.inv_m2 * dQ;
+  w = w_of(ca, cb, v);
+  const float am = fmaxf(fabsf((float)dP), fabsf((float)dQ));
+  mx = (am != am) ? __int_as_float(0x7f800000) : fmaxf(mx, am);
+  return mkc(dP, dQ);
+}
+
+// Adjoint of one row (the arithmetic of adj_finish) and the optimiser step;
+// sp.y is Q_calc at pv buses.  Returns the new value of the gathered vector.
+template <class R, bool REF, bool ADAM>
+__device__ __forceinline__ typename Prec<R>::C res_adj(const IterArgs<R>& a, int ty, ResRow<R>& r,
+                                                       typename Prec<R>::C x, typename Prec<R>::C w,
+                                                       typename Prec<R>::C z, typename Prec<R>::C sp, R step, R isb) {
+  using C = typename Prec<R>::C;
+  const int opt = ADAM ? (int)OPT_ADAM : a.opt;
+  C v = x, u;
+  if constexpr (REF) v = volt(r.th, r.vm, u);
+  const C g0 = conj_c_s(w, v, ty, sp.x, sp.y, sp.y, a.m_half);
+  const C h = adj_h(g0, v, z);
+  const R vm_old = mwork(r.vm);
+  R d_th = R(0), d_vm = R(0);
+  r.th = opt_update(opt, r.th, -h.y, r.m1, r.v1, a.beta1, a.beta2, step, isb, a.eps, a.mom, a.alpha, d_th);
+  if (ty == BUS_PQ)
+    r.vm = opt_update(opt, r.vm, div_step(h.x, vm_old), r.m2, r.v2, a.beta1, a.beta2, step, isb, a.eps, a.mom,
+                      a.alpha, d_vm);
+  if constexpr (REF) {
+    const float2 dd = volt_change(u, vm_old, -d_th, -d_vm);
+    return make_float2(x.x + dd.x, x.y + dd.y);
+  } else {
+    return volt(r.th, r.vm);
+  }
+}
+
+// The outaged branch's block out of acc at its two rows (bits of `end`: 1
+// from-bus, 2 to-bus); xo: the operand at the other end.
+template <class R, class C>
+__device__ __forceinline__ void res_outage(const IterArgs<R>& a, int k, int end, C x, C xo, C& acc) {
+  if (end & 1) {
+    cfms(acc, a.yff[k], x);
+    cfms(acc, a.yft[k], xo);
+  } else {
+    cfms(acc, a.yft[k], xo);
+    cfms(acc, a.ytt[k], x);
+  }
+}
+
+// Y_bus to shared memory (it does not change during a solve).
+template <class R>
+__device__ __forceinline__ void res_stage(const ResArgs<R>& q, unsigned char* smem) {
+  ValPair<R>* sval = reinterpret_cast<ValPair<R>*>(smem + q.L.val);
+  uint32_t* scol = reinterpret_cast<uint32_t*>(smem + q.L.col);
+  int* ssoff = reinterpret_cast<int*>(smem + q.L.soff);
+  for (int t = threadIdx.x; t < q.n_pair * 32; t += blockDim.x) {
+    sval[t] = q.val[t];
+    scol[t] = __ldg(q.col2 + t);
+  }
+  for (int t = threadIdx.x; t <= q.n_slice; t += blockDim.x) ssoff[t] = __ldg(q.soff + t) * 32;
+}
+
+// One warp per case, RES_TEAMS cases per CTA.
+template <class R, bool REF, bool ADAM, int RPT>
+__global__ void __launch_bounds__(32 * RES_TEAMS, sizeof(R) == 8 ? 3 : 5)
+    k_resident_warp(const ResArgs<R> q) {
+  using C = typename Prec<R>::C;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const IterArgs<R>& a = q.a;
+  const int N = a.N, lane = threadIdx.x & 31, team = threadIdx.x >> 5;
+  unsigned char* tb = smem + team * q.L.team;
+  unsigned char* wb = tb + q.L.w;
+  C* X = reinterpret_cast<C*>(tb);
+  C* W = reinterpret_cast<C*>(wb);
+  C* D = reinterpret_cast<C*>(tb + q.L.d);
+  R* scr = reinterpret_cast<R*>(tb + q.L.scr);
+  const ValPair<R>* val = reinterpret_cast<const ValPair<R>*>(smem + q.L.val) + lane;
+  const uint32_t* col = reinterpret_cast<const uint32_t*>(smem + q.L.col) + lane;
+  const int* soff = reinterpret_cast<const int*>(smem + q.L.soff);
+  const int k = blockIdx.x * RES_TEAMS + team;
+  res_stage(q, smem);
+  pdl_wait();
+  pdl_release();
+  __syncthreads();
+  if (k >= q.K || !a.active[k]) return;  // (no CTA barrier follows)
+  const size_t Kp = (size_t)a.Kp;
+
+  int row[RPT], ty[RPT], end[RPT];
+  ResRow<R> rw[RPT];
+  C sp[RPT];
+  float2 vr[RPT];
+  float4 rf[RPT];
+  int of = -1, ot = -1;
+  if (a.has_outage) {
+    of = a.of[k];
+    ot = a.ot[k];
+  }
+  const int pf = of >= 0 ? q.rpos[of] : 0, pt = of >= 0 ? q.rpos[ot] : 0;
+#pragma unroll
+  for (int s = 0; s < RPT; ++s) {
+    const int p = s * 32 + lane;
+    row[s] = p < N ? __ldg(q.rord + p) : -1;
+    ty[s] = BUS_SLACK;
+    end[s] = 0;
+    C x = mkc(R(0), R(0));
+    sp[s] = x;
+    rw[s] = ResRow<R>{};
+    vr[s] = make_float2(0.f, 0.f);
+    rf[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row[s] >= 0) {
+      const size_t e = (size_t)row[s] * Kp + k, si = a.spec_per_case ? e : (size_t)row[s];
+      ty[s] = __ldg(a.type + row[s]);
+      end[s] = row[s] == of ? 1 : row[s] == ot ? 2 : 0;
+      x = a.V[e];
+      sp[s] = mkc(a.pspec[si], a.qspec[si]);
+      rw[s].load(a, e);
+      if constexpr (REF) {
+        vr[s] = a.vref[e];
+        rf[s] = a.irf[e];
+      }
+    }
+    X[p] = x;
+    W[p] = mkc(R(0), R(0));
+  }
+  ResSched<R> sc;
+  sc.load(a.sc, k, lane);
+  __syncwarp();
+  bool fin = true;
+  for (int it = 0; it < q.n_it; ++it) {
+    sc.terms(a.sc, lane);
+    float mx = 0.f;
+#pragma unroll
+    for (int s = 0; s < RPT; ++s) {
+      const int p = s * 32 + lane;
+      if (s >= q.n_slice) break;
+      C I = sell_row<R>(val, col, soff[s], soff[s + 1], tb);
+      if (row[s] < 0) continue;
+      const C x = X[p];
+      if (end[s]) res_outage(a, k, end[s], x, X[end[s] & 1 ? pt : pf], I);
+      C w;
+      R Q;
+      D[row[s]] = res_fwd<R, REF>(a, ty[s], x, I, sp[s], vr[s], rf[s], w, Q, mx);
+      if (ty[s] == BUS_PV) sp[s].y = Q;
+      W[p] = w;
+    }
+    if (it == q.n_it - 1 && a.sc.mx32) {
+      const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+      if (lane == 0) a.sc.cand[k] = (a.sc.gate <= 0.0 || (double)__uint_as_float(m) <= a.sc.gate) ? 1 : 0;
+    }
+    __syncwarp();
+    loss_chains<R>(D, scr, N, q.lo, 0, 1, lane);
+    __syncwarp();
+    const R lsum = loss_tail<R>(scr, q.lo, 1, lane);
+    fin = isfinite(lsum);  // (as the loss: 1 / m <= 1)
+    if (!fin) break;       // stops as diverged before it steps
+#pragma unroll
+    for (int s = 0; s < RPT; ++s) {
+      const int p = s * 32 + lane;
+      if (s >= q.n_slice) break;
+      C z = sell_row<R>(val, col, soff[s], soff[s + 1], wb);
+      if (ty[s] == BUS_SLACK) continue;
+      const C w = W[p];
+      if (end[s]) res_outage(a, k, end[s], w, W[end[s] & 1 ? pt : pf], z);
+      X[p] = res_adj<R, REF, ADAM>(a, ty[s], rw[s], X[p], w, z, sp[s], sc.step, sc.isb);
+    }
+    sc.feed(a.sc, lsum);
+    __syncwarp();
+  }
+  if (!fin && lane == 0) {
+    a.sc.status[k] = CASE_DIVERGED;
+    a.sc.active[k] = 0;
+    atomicSub(a.sc.n_active, 1);
+  }
+#pragma unroll
+  for (int s = 0; s < RPT; ++s) {
+    if (ty[s] == BUS_SLACK) continue;  // (a slack's state does not change)
+    const size_t e = (size_t)row[s] * Kp + k;
+    rw[s].store(a, e);
+    a.V[e] = X[s * 32 + lane];
+  }
+  sc.store(a.sc, k, lane);
+}
+
+// One CTA per case.  The last warp also keeps the scheduler: it finishes an
+// iteration's loss sum and takes the scheduler's step during the next forward
+// pass, whose adjoint is the first to need the new rate.  A loss that is not
+// finite is therefore noticed one update late: the CTA then starts over from
+// the state in global memory and takes only the steps before it (what the
+// streaming kernels return for a diverged case).
+template <class R, bool REF, bool ADAM, int RPT>
+__global__ void __launch_bounds__(res_threads<R>(), 1) k_resident_cta(const ResArgs<R> q) {
+  using C = typename Prec<R>::C;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const IterArgs<R>& a = q.a;
+  const int N = a.N, T = q.T, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = (int)blockDim.x >> 5;
+  constexpr unsigned WOFF = res_threads<R>() * RPT * sizeof(C);
+  C* X = reinterpret_cast<C*>(smem) + tid;  // this thread's rows: every T-th position from tid
+  C* W = reinterpret_cast<C*>(smem + WOFF) + tid;
+  C* D = reinterpret_cast<C*>(smem + q.L.d);
+  C* S = reinterpret_cast<C*>(smem + q.L.s) + tid;
+  float2* VR = reinterpret_cast<float2*>(smem + q.L.vr) + tid;
+  float4* RF = reinterpret_cast<float4*>(smem + q.L.rf) + tid;
+  R* scr = reinterpret_cast<R*>(smem + q.L.scr);
+  int* flag = reinterpret_cast<int*>(smem + q.L.flag);      // [0] steps before a divergence, or -1
+  unsigned* mxs = reinterpret_cast<unsigned*>(flag + 1);    // [1] max mismatch of the last iterate
+  R* terms = reinterpret_cast<R*>(smem + q.L.flag + 16);    // step, isb of the coming update
+  const ValPair<R>* val = reinterpret_cast<const ValPair<R>*>(smem + q.L.val) + lane;
+  const uint32_t* col = reinterpret_cast<const uint32_t*>(smem + q.L.col) + lane;
+  const int* soff = reinterpret_cast<const int*>(smem + q.L.soff);
+  ResSched<R>* scs = reinterpret_cast<ResSched<R>*>(smem + q.L.sc) + lane;
+  const int k = blockIdx.x;
+  res_stage(q, smem);
+  pdl_wait();
+  pdl_release();
+  if (!a.active[k]) return;  // the whole CTA
+  const bool compute = tid < T, sched = warp == nw - 1;  // (T = blockDim: the last warp does both)
+  // the warps that sum the loss chains: the last ones before the scheduler's
+  const int ncw = max(1, min(nw - 1, (q.lo.nch + 31) >> 5)), cw = warp - (nw - 1 - ncw);
+  const size_t Kp = (size_t)a.Kp;
+  int n = q.n_it;
+  bool diverged = false;
+  for (;;) {
+    int info[RPT];  // internal row, bus type << 16, outage end << 20; -1: no row
+    ResRow<R> rw[RPT];
+    int ends = 0;   // positions of the outaged branch's ends: from-bus, to-bus << 16
+    if (compute) {
+      int of = -1, ot = -1;
+      if (a.has_outage) {
+        of = a.of[k];
+        ot = a.ot[k];
+        if (of >= 0) ends = q.rpos[of] | q.rpos[ot] << 16;
+      }
+#pragma unroll
+      for (int s = 0; s < RPT; ++s) {
+        const int p = s * T + tid, i = p < N ? __ldg(q.rord + p) : -1;
+        info[s] = -1;
+        C x = mkc(R(0), R(0));
+        if (i >= 0) {
+          const size_t e = (size_t)i * Kp + k, si = a.spec_per_case ? e : (size_t)i;
+          info[s] = i | (int)__ldg(a.type + i) << 16 | (i == of ? 1 : i == ot ? 2 : 0) << 20;
+          x = a.V[e];
+          S[s * T] = mkc(a.pspec[si], a.qspec[si]);
+          rw[s].load(a, e);
+          if constexpr (REF) {
+            VR[s * T] = a.vref[e];
+            RF[s * T] = a.irf[e];
+          }
+        }
+        X[s * T] = x;
+        W[s * T] = mkc(R(0), R(0));
+      }
+    }
+    if (sched) {
+      ResSched<R> sc;
+      sc.load(a.sc, k, lane);
+      *scs = sc;
+      if (lane == 0) {
+        flag[0] = -1;
+        *mxs = 0u;
+      }
+    }
+    __syncthreads();
+
+    for (int it = 0; it <= n; ++it) {
+      if (sched) {  // the previous iterate's loss, then this update's step terms
+        ResSched<R> sc = *scs;
+        bool fin = true;
+        if (it > 0) {
+          const R lsum = loss_tail<R>(scr, q.lo, ncw, lane);
+          fin = isfinite(lsum);  // (as the loss: 1 / m <= 1)
+          if (fin) sc.feed(a.sc, lsum);
+          else if (lane == 0) flag[0] = it - 1;
+        }
+        if (it < n) {
+          if (fin) sc.terms(a.sc, lane);
+          if (lane == 0) {
+            terms[0] = sc.step;
+            terms[1] = sc.isb;
+          }
+        }
+        *scs = sc;
+      }
+      if (it == n) break;
+      if (compute) {  // forward: I = Y V, mismatch, w
+        float mx = 0.f;
+#pragma unroll
+        for (int s = 0; s < RPT; ++s) {
+          const int sl = (s * T + tid) >> 5;  // (the same for the whole warp)
+          if (sl >= q.n_slice) break;
+          C I = sell_row<R>(val, col, soff[sl], soff[sl + 1], smem);
+          if (info[s] < 0) continue;
+          const C x = X[s * T];
+          const int ty = (info[s] >> 16) & 15;
+          if (info[s] >> 20)
+            res_outage(a, k, info[s] >> 20, x,
+                       reinterpret_cast<C*>(smem)[(info[s] >> 20) & 1 ? ends >> 16 : ends & 0xffff], I);
+          float2 vr = make_float2(0.f, 0.f);
+          float4 rf = make_float4(0.f, 0.f, 0.f, 0.f);
+          if constexpr (REF) {
+            vr = VR[s * T];
+            rf = RF[s * T];
+          }
+          C w, sp = mkc(R(0), R(0));
+          if constexpr (!REF) sp = S[s * T];
+          R Q;
+          D[info[s] & 0xffff] = res_fwd<R, REF>(a, ty, x, I, sp, vr, rf, w, Q, mx);
+          if (ty == BUS_PV) S[s * T].y = Q;
+          W[s * T] = w;
+        }
+        if (it == n - 1 && a.sc.mx32) {
+          const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+          if (lane == 0) atomicMax(mxs, m);
+        }
+      }
+      __syncthreads();
+      if (flag[0] >= 0) break;
+      if (cw >= 0 && !sched) loss_chains<R>(D, scr, N, q.lo, cw, ncw, lane);
+      if (compute) {  // adjoint: z = Y w, gradient, step, new V
+        const R step = terms[0], isb = terms[1];
+#pragma unroll
+        for (int s = 0; s < RPT; ++s) {
+          const int sl = (s * T + tid) >> 5;
+          if (sl >= q.n_slice) break;
+          C z = sell_row<R>(val, col, soff[sl], soff[sl + 1], smem + WOFF);
+          const int ty = (info[s] >> 16) & 15;
+          if (info[s] < 0 || ty == BUS_SLACK) continue;
+          const C w = W[s * T];
+          if (info[s] >> 20)
+            res_outage(a, k, info[s] >> 20, w,
+                       reinterpret_cast<C*>(smem + WOFF)[(info[s] >> 20) & 1 ? ends >> 16 : ends & 0xffff], z);
+          X[s * T] = res_adj<R, REF, ADAM>(a, ty, rw[s], X[s * T], w, z, S[s * T], step, isb);
+        }
+      }
+      __syncthreads();
+    }
+    __syncthreads();
+    if (flag[0] >= 0) {  // again, only the steps before the divergence
+      n = flag[0];
+      diverged = true;
+      __syncthreads();
+      continue;
+    }
+    if (compute) {
+#pragma unroll
+      for (int s = 0; s < RPT; ++s) {
+        if (info[s] < 0 || ((info[s] >> 16) & 15) == BUS_SLACK) continue;  // (a slack's state does not change)
+        const size_t e = (size_t)(info[s] & 0xffff) * Kp + k;
+        rw[s].store(a, e);
+        a.V[e] = X[s * T];
+      }
+    }
+    if (sched) {
+      scs->store(a.sc, k, lane);
+      if (lane == 0) {
+        if (a.sc.mx32)
+          a.sc.cand[k] = (a.sc.gate <= 0.0 || (double)__uint_as_float(*mxs) <= a.sc.gate) ? 1 : 0;
+        if (diverged) {
+          a.sc.status[k] = CASE_DIVERGED;
+          a.sc.active[k] = 0;
+          atomicSub(a.sc.n_active, 1);
+        }
+      }
+    }
+    return;
+  }
+}
+
+// ---- host ---------------------------------------------------------------------
+static LossGeo loss_geo(const LossOrder& lo) {
+  LossGeo g;
+  g.gy = lo.gy;
+  g.rpb = lo.rpb;
+  g.step = lo.wpb * lo.rpw;
+  g.rpw = 1;
+  g.lrpw = 0;
+  while (g.rpw < std::min(lo.rpw, lo.rpb)) {
+    g.rpw *= 2;
+    g.lrpw += 1;
+  }
+  g.wpb = std::min(lo.wpb, (lo.rpb + lo.rpw - 1) / lo.rpw);
+  g.nj = (lo.rpb + g.step - 1) / g.step;
+  g.nch = g.gy * g.wpb * g.rpw;
+  g.magic = (1 << 18) / g.wpb + 1;
+  g.tile = lo.tile;
+  g.nthr = lo.nthr;
+  return g;
+}
+
+template <class R>
+static ResLayout res_layout(const dpf_ybus* y, const ResShape& sh, bool refined, const LossOrder& lo) {
+  const unsigned cs = 2 * sizeof(R), np = (unsigned)(sh.T * sh.rpt), pairs = (unsigned)y->dev.res_pairs;
+  const bool refs = refined && !sh.warp;
+  ResLayout L;
+  L.w = (sh.warp ? np : (unsigned)(res_threads<R>() * sh.rpt)) * cs;  // (CTA form: a compile-time offset)
+  L.d = L.w + np * cs;
+  L.s = L.d + (unsigned)((y->n + 1) & ~1) * cs;
+  L.vr = L.s + np * cs;
+  L.rf = L.vr + (refs ? np * 8u : 0u);
+  L.scr = L.rf + (refs ? np * 16u : 0u);
+  L.sc = L.scr + (((unsigned)res_scratch(loss_geo(lo)) * (unsigned)sizeof(R) + 15u) & ~15u);
+  L.flag = L.sc + (sh.warp ? 0u : 32u * (unsigned)sizeof(ResSched<R>));
+  L.team = L.flag + 32u;
+  L.val = L.team * (sh.warp ? RES_TEAMS : 1);
+  L.col = L.val + pairs * 64u * cs;
+  L.soff = L.col + pairs * 32u * 4u;
+  L.total = L.soff + (((unsigned)(y->dev.res_slices + 1) * 4u + 15u) & ~15u);
+  return L;
+}
+
+ResShape res_shape(const dpf_ybus* y, int K, bool fp64, bool refined, const LossOrder& lo, size_t smem_limit) {
+  ResShape sh;
+  const DeviceYbus& d = y->dev;
+  const int n = y->n;
+  if (!d.res_rord || n > RES_MAX_N || y->m_loss <= 0) return sh;
+  // FP64 is bound by the FP64 pipe: the streaming kernels spread a case over
+  // many SMs, so the on-chip form pays only where an iteration is mostly
+  // latency.  Microseconds per 100 iterations (streaming, on chip), cases x
+  // buses: 1x30 1,920 982; 3000x30 4,256 4,017; 1x300 2,316 1,883; 150x300
+  // 3,471 1,886; but 1000x300 11,344 12,548; 1x700 2,454 3,500.  In FP32 it is
+  // faster over the whole range measured (30-2,048 buses, 1-3,000 cases):
+  // 1x30 1,169 330; 3000x30 1,330 486; 1x2000 1,234 732; 3000x2000 17,719
+  // 13,284; 3000x300 3,216 2,346; 3000x1000 8,710 6,501.
+  if (fp64 && n > RES_WARP_N && (n > 320 || K > 300)) return sh;
+  sh.warp = n <= RES_WARP_N;
+  sh.rpt = sh.warp && n <= 32 ? 1 : 2;
+  sh.T = sh.warp ? 32 : ((n + 1) / 2 + 31) / 32 * 32;
+  sh.smem = fp64 ? res_layout<double>(y, sh, refined, lo).total : res_layout<float>(y, sh, refined, lo).total;
+  sh.ok = sh.smem <= smem_limit;
+  return sh;
+}
+
+template <class R>
+static cudaError_t res_go(void (*kern)(const ResArgs<R>), const ResArgs<R>& q, const ResShape& sh, bool pdl,
+                          cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(sh.warp ? (q.K + RES_TEAMS - 1) / RES_TEAMS : q.K);
+  // a warp of its own for the scheduler, unless that would leave room for one
+  // CTA per SM instead of two
+  const int threads = sh.T <= 512 && sh.T + 32 > 512 ? sh.T : std::min(sh.T + 32, res_threads<R>());
+  cfg.blockDim = dim3(sh.warp ? 32 * RES_TEAMS : threads);
+  cfg.dynamicSmemBytes = sh.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, q);
+}
+
+template <class R, bool REF, bool ADAM>
+static cudaError_t res_pick(const ResArgs<R>& q, const ResShape& sh, bool pdl, cudaStream_t s) {
+  return res_go<R>(!sh.warp      ? k_resident_cta<R, REF, ADAM, 2>
+                   : sh.rpt == 1 ? k_resident_warp<R, REF, ADAM, 1>
+                                 : k_resident_warp<R, REF, ADAM, 2>,
+                   q, sh, pdl, s);
+}
+
+template <class R>
+int res_launch(const dpf_ybus* y, const IterArgs<R>& a, const ResShape& sh, const LossOrder& lo, int K, int n_it,
+               bool refined, bool pdl, void* stream) {
+  const DeviceYbus& d = y->dev;
+  ResArgs<R> q;
+  q.a = a;
+  q.K = K;
+  q.T = sh.T;
+  q.n_it = n_it;
+  q.rord = d.res_rord;
+  q.rpos = d.res_rpos;
+  q.soff = d.res_soff;
+  q.col2 = d.res_col2;
+  q.n_pair = d.res_pairs;
+  q.n_slice = d.res_slices;
+  q.lo = loss_geo(lo);
+  q.L = res_layout<R>(y, sh, refined, lo);
+  cudaStream_t s = (cudaStream_t)stream;
+  if constexpr (sizeof(R) == 4) {
+    q.val = reinterpret_cast<const ValPair<float>*>(d.res_val32);
+    if (a.opt == OPT_ADAM)
+      return refined ? res_pick<float, true, true>(q, sh, pdl, s) : res_pick<float, false, true>(q, sh, pdl, s);
+    return refined ? res_pick<float, true, false>(q, sh, pdl, s) : res_pick<float, false, false>(q, sh, pdl, s);
+  } else {
+    q.val = reinterpret_cast<const ValPair<double>*>(d.res_val64);
+    return res_pick<double, false, false>(q, sh, pdl, s);
+  }
+}
+template int res_launch<float>(const dpf_ybus*, const IterArgs<float>&, const ResShape&, const LossOrder&, int, int,
+                               bool, bool, void*);
+template int res_launch<double>(const dpf_ybus*, const IterArgs<double>&, const ResShape&, const LossOrder&, int, int,
+                                bool, bool, void*);
+
+}  // namespace dpf

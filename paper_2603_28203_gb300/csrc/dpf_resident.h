@@ -1,0 +1,42 @@
+// On-chip form of the iterations (dpf_resident.cu): its launch parameters,
+// shared with the host code that chooses it (dpf_api.cu).
+#pragma once
+
+#include "dpf_internal.h"
+
+namespace dpf {
+
+template <class R> struct IterArgs;
+
+// Grids up to this many buses can run the on-chip form (a case's working set
+// must fit one SM: 1,024 threads of two rows).
+constexpr int RES_MAX_N = 2048;
+constexpr int RES_WARP_N = 64;       // up to here one warp runs a case
+constexpr int RES_TEAMS = 4;         // cases (warps) per CTA of the one-warp form
+
+// Launch shape for one grid and precision.
+struct ResShape {
+  bool ok = false;
+  bool warp = false;  // one warp per case
+  int rpt = 1;        // rows per thread
+  int T = 32;         // compute threads per case
+  size_t smem = 0;
+};
+
+// The order in which the streaming kernels of the same options sum a case's
+// loss (row blocks, warps, rows per warp), which the on-chip form repeats.
+struct LossOrder {
+  int gy, rpb, wpb, rpw, tile, nthr;
+};
+
+// Whether (and how) a solve of K cases runs on chip; smem_limit: opt-in shared
+// memory per CTA.
+ResShape res_shape(const dpf_ybus* y, int K, bool fp64, bool refined, const LossOrder& lo, size_t smem_limit);
+
+// Enqueue n_it iterations of every active case (refined: DPF_FP32R); pdl:
+// programmatic dependent launch.  Returns a cudaError_t.
+template <class R>
+int res_launch(const dpf_ybus* y, const IterArgs<R>& a, const ResShape& sh, const LossOrder& lo, int K, int n_it,
+               bool refined, bool pdl, void* stream);
+
+}  // namespace dpf

@@ -1,0 +1,138 @@
+"""The on-chip form of the iterations (dpf_resident.cu) against the streaming
+kernels: same options, same bits.
+
+Timing the passes one by one (dpf_profile_enable) runs the streaming kernels,
+so one solve with it and one without compare the two forms.  FP32 and refined
+FP32 results have to agree to the bit, the plateau schedule (fed the FP32
+loss) included; the FP64 on-chip form sums the loss in another order, which
+only a schedule fed by it can see, so FP64 runs a constant rate.
+"""
+import numpy as np
+import pytest
+
+import gridgen
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2603_28203_gb300 as dpf  # noqa: E402
+
+DEV = torch.device("cuda:0")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import os
+    from paper_2603_28203_gb300.build import LIB, build
+    if not os.path.exists(LIB):
+        build()
+    dpf.lib()
+
+
+def _grid(n):
+    return gridgen.config_grid("c1_30bus_fp64") if n == 30 else gridgen.make_grid(n, 3, load_scale=0.1)
+
+
+def _run(y, ws, K, opts, streaming, **kw):
+    N = y.n_bus
+    out = dict(va=torch.zeros((K, N), dtype=torch.float64, device=DEV),
+               vm=torch.ones((K, N), dtype=torch.float64, device=DEV),
+               iters=torch.zeros(K, dtype=torch.int32, device=DEV),
+               status=torch.zeros(K, dtype=torch.int32, device=DEV),
+               max_mismatch=torch.zeros(K, dtype=torch.float64, device=DEV))
+    b = dict(n_case=K, **out, **kw)
+    dpf.dpf_profile_enable(ws, streaming)
+    dpf.dpf_solve_begin(y, ws, opts, **b)
+    dpf.dpf_solve_iterate(ws, opts.max_iter)
+    dpf.dpf_solve_end(ws, **b)
+    torch.cuda.synchronize()
+    n_fwd = dpf.dpf_kernel_times(ws)[2]
+    dpf.dpf_profile_enable(ws, False)
+    assert (n_fwd > 0) == streaming  # the two forms really ran
+    return {k: v.cpu().numpy() for k, v in out.items()}
+
+
+def _same(a, b):
+    for k in a:
+        assert np.array_equal(a[k], b[k], equal_nan=True), k
+
+
+def _inputs(g, K, seed, specs, outages):
+    rng = np.random.default_rng(seed)
+    kw = {}
+    if specs:
+        sc = 1 + 0.1 * rng.uniform(-1, 1, (K, 1))
+        kw["p_spec"] = torch.tensor(g.p_spec * sc, device=DEV)
+        kw["q_spec"] = torch.tensor(g.q_spec * sc, device=DEV)
+    if outages:
+        ok = gridgen.n1_outages(g)
+        o = np.resize(rng.permutation(ok), K).astype(np.int32)
+        o[::7] = -1
+        kw["outage"] = torch.tensor(o, device=DEV)
+    return kw
+
+
+# sizes around the edges of the forms: one row per lane (32), two (64), one
+# CTA per case above, its largest grid (2,048); cases around a CTA's four, a
+# warp's 32 and the two-case kernels' 64 (whose loss order differs)
+@pytest.mark.parametrize("n,K", [(2, 1), (30, 1), (30, 70), (32, 5), (33, 64), (64, 33), (65, 2), (129, 40), (300, 100),
+                                 (700, 1), (1000, 40), (1025, 9), (2000, 130), (2048, 3)])
+@pytest.mark.parametrize("precision", ["fp32", "fp32r"])
+def test_on_chip_equals_streaming(n, K, precision):
+    g = gridgen.two_bus(0.3, 0.1, 0.01, 0.1) if n == 2 else _grid(n)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    opts = dpf.SolveOpts(precision=getattr(dpf, precision.upper()), max_iter=63, check_every=20, lr=3e-3, patience=3,
+                         cooldown=5, gate=1e-1)
+    kw = _inputs(g, K, n + K, specs=K > 4, outages=n > 2 and K != 5)
+    _same(_run(y, ws, K, opts, False, **kw), _run(y, ws, K, opts, True, **kw))
+
+
+@pytest.mark.parametrize("n,K", [(30, 1), (64, 40), (65, 3), (300, 150)])
+def test_on_chip_equals_streaming_fp64(n, K):
+    g = _grid(n)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    opts = dpf.SolveOpts(precision=dpf.FP64, max_iter=45, check_every=20, lr=3e-3, sched=dpf.SCHED_CONST)
+    kw = _inputs(g, K, n, specs=True, outages=True)
+    _same(_run(y, ws, K, opts, False, **kw), _run(y, ws, K, opts, True, **kw))
+
+
+@pytest.mark.parametrize("opt", [dpf.OPT_SGD, dpf.OPT_RMSPROP, dpf.OPT_ADAM])
+@pytest.mark.parametrize("n", [30, 300])
+def test_on_chip_optimisers_and_step_schedule(opt, n):
+    g = _grid(n)
+    K = 6
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    opts = dpf.SolveOpts(precision=dpf.FP32, max_iter=50, check_every=16, lr=1e-3, optimizer=opt, momentum=0.5,
+                         sched=dpf.SCHED_STEP, step_size=7, gamma=0.8)
+    kw = _inputs(g, K, 1, specs=True, outages=False)
+    _same(_run(y, ws, K, opts, False, **kw), _run(y, ws, K, opts, True, **kw))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp32r"])
+@pytest.mark.parametrize("n", [30, 300])
+def test_on_chip_divergence(n, precision):
+    """A case stops as diverged before the step its loss makes impossible: at
+    once (NaN injections) or after some steps (a rate that overflows |V|);
+    the other cases go on."""
+    g = _grid(n)
+    K = 5
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    kw = _inputs(g, K, 4, specs=True, outages=False)
+    kw["p_spec"][2, n // 2] = float("nan")
+    opts = dpf.SolveOpts(precision=getattr(dpf, precision.upper()), max_iter=40, check_every=10, lr=1e-2)
+    a = _run(y, ws, K, opts, False, **kw)
+    _same(a, _run(y, ws, K, opts, True, **kw))
+    assert a["status"][2] == dpf.CASE_DIVERGED and a["iters"][2] == 0 and a["iters"][0] == 40
+    kw = _inputs(g, K, 4, specs=True, outages=False)
+    opts = dpf.SolveOpts(precision=opts.precision, max_iter=40, check_every=10, lr=3e8, sched=dpf.SCHED_STEP,
+                         step_size=1, gamma=4.0)
+    a = _run(y, ws, K, opts, False, **kw)
+    _same(a, _run(y, ws, K, opts, True, **kw))
+    assert (a["status"] == dpf.CASE_DIVERGED).all() and (a["iters"] > 0).all() and (a["iters"] < 40).all()
