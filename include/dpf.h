@@ -394,7 +394,9 @@ int dpf_loss_backward(const dpf_ybus* y, dpf_workspace* ws, int32_t n_case,
  * bridge is DPF_E_ISLANDED) as for dpf_solve_batch.  Conjugate gradients
  * with the Jacobi preconditioner on the GPU, per case until |r| <= tol |r0|
  * or max_iter iterations; the vectors are double-float pairs (~48 bits)
- * for tol < 1e-5 and FP32 for tol >= 1e-5, the per-case scalars FP64.  Outputs (caller-owned device
+ * for tol < 1e-5 and FP32 for tol >= 1e-5, the per-case scalars FP64
+ * (grids above 2,048 buses) or double-float (up to there, where one CTA runs
+ * a case's whole solve on chip).  Outputs (caller-owned device
  * arrays): va [n_case][n_bus] (required), iters [n_case] and rel_residual
  * [n_case] (|r| / |r0| at the stop; either may be NULL).  Uses (and
  * resets) the workspace like the other calls. */

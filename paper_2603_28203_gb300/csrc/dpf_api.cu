@@ -111,7 +111,7 @@ static void free_device(DeviceYbus& d) {
   dfree(d.type); dfree(d.p64); dfree(d.q64); dfree(d.vmset); dfree(d.p32); dfree(d.q32);
   dfree(d.perm); dfree(d.iperm); dfree(d.br_f); dfree(d.br_t); dfree(d.br_r); dfree(d.br_x);
   dfree(d.br_bch); dfree(d.br_tap); dfree(d.br_itap); dfree(d.bridge);
-  dfree(d.res_rord); dfree(d.res_rpos); dfree(d.res_soff); dfree(d.res_col2); dfree(d.res_val32); dfree(d.res_val64);
+  dfree(d.res_rord); dfree(d.res_rpos); dfree(d.res_soff); dfree(d.res_col2); dfree(d.res_val32); dfree(d.res_val64); dfree(d.res_bval); dfree(d.res_dinv);
   d.ready = false;
 }
 
@@ -123,8 +123,10 @@ struct SellY {
   std::vector<uint32_t> col2;
   std::vector<float2> val32;
   std::vector<double2> val64;
+  std::vector<float4> bval;
+  std::vector<float2> dinv;
 };
-static void build_sell(const dpf_ybus* y, SellY& q) {
+static void build_sell(const dpf_ybus* y, const std::vector<float2>& dcval, const std::vector<float2>& dcinv, SellY& q) {
   const int n = y->n;
   const std::vector<int32_t>& rp = y->irow_ptr;
   q.rord.resize(n);
@@ -147,6 +149,9 @@ static void build_sell(const dpf_ybus* y, SellY& q) {
   q.col2.assign((size_t)pairs * 32, 0);
   q.val32.assign((size_t)pairs * 64, make_float2(0.f, 0.f));
   q.val64.assign((size_t)pairs * 64, make_double2(0.0, 0.0));
+  q.dinv.assign((size_t)slices * 32, make_float2(0.f, 0.f));
+  for (int p = 0; p < n; ++p) q.dinv[p] = dcinv[q.rord[p]];
+  q.bval.assign((size_t)pairs * 32, make_float4(0.f, 0.f, 0.f, 0.f));
   for (int s = 0; s < slices; ++s)
     for (int l = 0; l < 32; ++l) {
       const int p = s * 32 + l, i = p < n ? q.rord[p] : -1;
@@ -158,6 +163,14 @@ static void build_sell(const dpf_ybus* y, SellY& q) {
           const size_t at = ((size_t)(q.soff[s] + e / 2) * 32 + l) * 2 + (e & 1);
           q.val32[at] = make_float2((float)y->ival_re[t], (float)y->ival_im[t]);
           q.val64[at] = make_double2(y->ival_re[t], y->ival_im[t]);
+          float4& b = q.bval[at / 2];
+          if (e & 1) {
+            b.z = dcval[t].x;
+            b.w = dcval[t].y;
+          } else {
+            b.x = dcval[t].x;
+            b.y = dcval[t].y;
+          }
         }
         q.col2[(size_t)(q.soff[s] + e / 2) * 32 + l] |= (uint32_t)(c * 8) << (16 * (e & 1));
       }
@@ -227,7 +240,7 @@ extern "C" int dpf_ybus_upload(dpf_ybus* y, void* stream) {
     dcinv2[i] = pair(dii != 0.0 ? 1.0 / dii : 0.0);
   }
   SellY sell;
-  if (n <= RES_MAX_N) build_sell(y, sell);
+  if (n <= RES_MAX_N) build_sell(y, dcval2, dcinv2, sell);
   int rc = DPF_OK;
   do {
     if (n <= RES_MAX_N) {
@@ -237,6 +250,8 @@ extern "C" int dpf_ybus_upload(dpf_ybus* y, void* stream) {
       if ((rc = upload(&d.res_col2, sell.col2, s))) break;
       if ((rc = upload(&d.res_val32, sell.val32, s))) break;
       if ((rc = upload(&d.res_val64, sell.val64, s))) break;
+      if ((rc = upload(&d.res_bval, sell.bval, s))) break;
+      if ((rc = upload(&d.res_dinv, sell.dinv, s))) break;
       d.res_slices = (int)sell.soff.size() - 1;
       d.res_pairs = sell.soff.back();
     }
@@ -1388,6 +1403,26 @@ static int dc_run_t(dpf_workspace* w, const int32_t* outage_dev, double tol, int
       k_dc_flow<double><<<cb, 256, 0, s>>>((const double2*)w->ms, a.of, a.ot, a.ob, c + 8 * (size_t)Kp, w->K, Kp);
     else
       k_dc_flow<float><<<cb, 256, 0, s>>>((const float4*)w->ms, a.of, a.ot, a.ob, c + 8 * (size_t)Kp, w->K, Kp);
+  }
+  if (d.res_rord) {  // (every grid up to RES_MAX_N buses)
+    DcRes c;
+    c.K = w->K;
+    c.Kp = Kp;
+    c.max_iter = max_iter;
+    c.spec_per_case = a.spec_per_case;
+    c.tol = tol;
+    c.va_slack = a.va_slack;
+    c.pspec = a.pspec;
+    c.of = a.of;
+    c.ot = a.ot;
+    c.ob = a.ob;
+    c.flow = a.flow;
+    c.x = w->tmp_a;
+    c.res = a.res;
+    c.iters = a.iters;
+    CK((cudaError_t)dc_res_launch(y, c, sizeof(T) == 4, s));
+    w->launches += shift ? 3 : 2;
+    return DPF_OK;
   }
   k_dc_set_count<<<1, 1, 0, s>>>(a.n_active, w->K);
   k_dc_x0<T><<<std::max(nb, 1), 256, 0, s>>>(a);

@@ -64,6 +64,8 @@ struct DeviceYbus {
   uint32_t* res_col2 = nullptr; // [pairs][32] two columns (position * 8, 16 bits each)
   float2* res_val32 = nullptr;  // [pairs][32][2]
   double2* res_val64 = nullptr;
+  float4* res_bval = nullptr;   // [pairs][32] the DC matrix in the same form, two (hi, lo) entries
+  float2* res_dinv = nullptr;   // [slices * 32] dcinv by position
   int res_pairs = 0, res_slices = 0;
 };
 

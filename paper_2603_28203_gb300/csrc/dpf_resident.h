@@ -39,4 +39,18 @@ template <class R>
 int res_launch(const dpf_ybus* y, const IterArgs<R>& a, const ResShape& sh, const LossOrder& lo, int K, int n_it,
                bool refined, bool pdl, void* stream);
 
+// On-chip form of the DC solve (dpf_dc_resident.cu): every case of the batch
+// to its tolerance in one launch.
+struct DcRes {
+  int K, Kp, max_iter, spec_per_case;
+  double tol, va_slack;
+  const double* pspec;   // [N][Kp] or [N]
+  const int32_t *of, *ot;
+  const double *ob, *flow;
+  double *x, *res;       // [N][Kp] FP64 solution; |r| / |r0| per case
+  int32_t* iters;
+};
+// f32: FP32 vectors, else double-float.  Returns a cudaError_t.
+int dc_res_launch(const dpf_ybus* y, const DcRes& c, bool f32, void* stream);
+
 }  // namespace dpf

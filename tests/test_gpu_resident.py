@@ -136,3 +136,52 @@ def test_on_chip_divergence(n, precision):
     a = _run(y, ws, K, opts, False, **kw)
     _same(a, _run(y, ws, K, opts, True, **kw))
     assert (a["status"] == dpf.CASE_DIVERGED).all() and (a["iters"] > 0).all() and (a["iters"] < 40).all()
+
+
+# ---- the DC solve on chip ------------------------------------------------------
+def _dc_true_residual(g, va, p, ell):
+    """|B' theta - P| / |P| over the non-slack rows in FP64."""
+    b = 1.0 / (g.x * np.where(g.tap == 0, 1.0, g.tap))
+    if ell >= 0:
+        b = b.copy()
+        b[ell] = 0.0
+    flow = b * (va[g.f_bus] - va[g.t_bus])
+    r = -p.copy()
+    np.add.at(r, g.f_bus, flow)
+    np.add.at(r, g.t_bus, -flow)
+    u = g.bus_type != gridgen.SLACK
+    return np.linalg.norm(r[u]) / np.linalg.norm(p[u])
+
+
+# one thread per row pair up to 1,024 threads, and (more cases than SMs) four
+# or eight rows per thread; a partial last slice, one warp, and the largest grid
+@pytest.mark.parametrize("n,K", [(2, 1), (30, 3), (65, 200), (300, 400), (1000, 2), (2047, 200), (2048, 1)])
+@pytest.mark.parametrize("tol", [1e-10, 1e-4])
+def test_dc_on_chip_residual(n, K, tol):
+    """Every case stops at the recurrence's |r| <= tol |r0|; the residual of the
+    returned angles recomputed in FP64 differs from the recurrence's by
+    rounding: a few hundred steps of 2^-47 (double-float) stay below the
+    tolerance itself, of 2^-24 (FP32 vectors) below 10 tol as
+    test_dc_fp32_vectors_at_a_loose_tolerance allows.  Equal cases give equal
+    bits whatever SM runs them."""
+    g = gridgen.two_bus(0.3, 0.1, 0.01, 0.1) if n == 2 else _grid(n)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    rng = np.random.default_rng(n)
+    P = g.p_spec * (1 + 0.1 * rng.uniform(-1, 1, (K, 1)))
+    o = np.full(K, -1, np.int32)
+    if n > 2:
+        o = np.resize(rng.permutation(gridgen.n1_outages(g)), K).astype(np.int32)
+        o[0] = -1
+    P[K // 2], o[K // 2] = P[0], o[0]
+    out = dpf.dpf_dc_solve(y, ws, K, p_spec=torch.tensor(P, device=DEV), outage=torch.tensor(o, device=DEV), tol=tol)
+    va, rr = out["va"].cpu().numpy(), out["rel_residual"].cpu().numpy()
+    it = out["iters"].cpu().numpy()
+    assert (rr <= tol).all() and (it >= 1).all()
+    assert np.array_equal(va[K // 2], va[0]) and it[K // 2] == it[0]
+    for k in range(0, K, max(1, K // 12)):
+        assert _dc_true_residual(g, va[k], P[k], int(o[k])) <= (2 if tol < 1e-5 else 10) * tol, k
+    if it.max() > 2:  # the cap stops a case where it stands
+        cap = dpf.dpf_dc_solve(y, ws, K, p_spec=torch.tensor(P, device=DEV), outage=torch.tensor(o, device=DEV),
+                               tol=tol, max_iter=2)
+        assert (cap["iters"].cpu().numpy() <= 2).all() and (cap["rel_residual"].cpu().numpy() > tol).any()
