@@ -77,13 +77,6 @@ void dfree(T*& p) {
   p = nullptr;
 }
 
-template <class T>
-int upload(T** dst, const std::vector<T>& src, cudaStream_t s) {
-  TRY(dalloc(dst, src.size()));
-  if (!src.empty()) CK(cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, s));
-  return DPF_OK;
-}
-
 int num_sms() {
   static int sms = 0;
   if (!sms) {
@@ -106,13 +99,10 @@ int pow2ceil(int v) {
 // ---------------------------------------------------------------------------
 // Y_bus upload
 // ---------------------------------------------------------------------------
+// All arrays live in one allocation (DeviceYbus::arena).
 static void free_device(DeviceYbus& d) {
-  dfree(d.ent32); dfree(d.row_ptr); dfree(d.prow_ptr); dfree(d.ppos); dfree(d.col); dfree(d.dcval); dfree(d.dcinv); dfree(d.val64); dfree(d.ebr); dfree(d.dpos);
-  dfree(d.type); dfree(d.p64); dfree(d.q64); dfree(d.vmset); dfree(d.p32); dfree(d.q32);
-  dfree(d.perm); dfree(d.iperm); dfree(d.br_f); dfree(d.br_t); dfree(d.br_r); dfree(d.br_x);
-  dfree(d.br_bch); dfree(d.br_tap); dfree(d.br_itap); dfree(d.bridge);
-  dfree(d.res_rord); dfree(d.res_rpos); dfree(d.res_soff); dfree(d.res_col2); dfree(d.res_val32); dfree(d.res_val64); dfree(d.res_bval); dfree(d.res_dinv);
-  d.ready = false;
+  dfree(d.arena);
+  d = DeviceYbus();
 }
 
 // Sliced ELL form of Y_bus for the on-chip iterations (see DeviceYbus).  Rows
@@ -125,6 +115,8 @@ struct SellY {
   std::vector<double2> val64;
   std::vector<float4> bval;
   std::vector<float2> dinv;
+  std::vector<uint16_t> upos, puser;
+  std::vector<int32_t> slot;
 };
 static void build_sell(const dpf_ybus* y, const std::vector<float2>& dcval, const std::vector<float2>& dcinv, SellY& q) {
   const int n = y->n;
@@ -138,6 +130,13 @@ static void build_sell(const dpf_ybus* y, const std::vector<float2>& dcval, cons
     return y->bus_type[y->perm[i]] < y->bus_type[y->perm[j]];
   });
   for (int p = 0; p < n; ++p) q.rpos[q.rord[p]] = p;
+  q.upos.resize(n);
+  q.puser.resize(n);
+  for (int p = 0; p < n; ++p) {
+    q.puser[p] = (uint16_t)y->perm[q.rord[p]];
+    q.upos[q.puser[p]] = (uint16_t)p;
+  }
+  q.slot.resize(y->nnz);
   const int slices = (n + 31) / 32;
   q.soff.assign(slices + 1, 0);
   for (int s = 0; s < slices; ++s) {
@@ -161,6 +160,7 @@ static void build_sell(const dpf_ybus* y, const std::vector<float2>& dcval, cons
           const int t = rp[i] + e;
           c = q.rpos[y->icol[t]];
           const size_t at = ((size_t)(q.soff[s] + e / 2) * 32 + l) * 2 + (e & 1);
+          q.slot[t] = (int32_t)at;
           q.val32[at] = make_float2((float)y->ival_re[t], (float)y->ival_im[t]);
           q.val64[at] = make_double2(y->ival_re[t], y->ival_im[t]);
           float4& b = q.bval[at / 2];
@@ -241,49 +241,63 @@ extern "C" int dpf_ybus_upload(dpf_ybus* y, void* stream) {
   }
   SellY sell;
   if (n <= RES_MAX_N) build_sell(y, dcval2, dcinv2, sell);
-  int rc = DPF_OK;
-  do {
-    if (n <= RES_MAX_N) {
-      if ((rc = upload(&d.res_rord, sell.rord, s))) break;
-      if ((rc = upload(&d.res_rpos, sell.rpos, s))) break;
-      if ((rc = upload(&d.res_soff, sell.soff, s))) break;
-      if ((rc = upload(&d.res_col2, sell.col2, s))) break;
-      if ((rc = upload(&d.res_val32, sell.val32, s))) break;
-      if ((rc = upload(&d.res_val64, sell.val64, s))) break;
-      if ((rc = upload(&d.res_bval, sell.bval, s))) break;
-      if ((rc = upload(&d.res_dinv, sell.dinv, s))) break;
-      d.res_slices = (int)sell.soff.size() - 1;
-      d.res_pairs = sell.soff.back();
-    }
-    if ((rc = upload(&d.ent32, ent, s))) break;
-    if ((rc = upload(&d.row_ptr, y->irow_ptr, s))) break;
-    if ((rc = upload(&d.prow_ptr, y->iprow_ptr, s))) break;
-    if ((rc = upload(&d.ppos, y->ippos, s))) break;
-    if ((rc = upload(&d.col, y->icol, s))) break;
-    if ((rc = upload(&d.val64, v64, s))) break;
-    if ((rc = upload(&d.dcval, dcval2, s))) break;
-    if ((rc = upload(&d.dcinv, dcinv2, s))) break;
-    if ((rc = upload(&d.ebr, y->iebr, s))) break;
-    if ((rc = upload(&d.dpos, y->idpos, s))) break;
-    if ((rc = upload(&d.type, type, s))) break;
-    if ((rc = upload(&d.p64, p64, s))) break;
-    if ((rc = upload(&d.q64, q64, s))) break;
-    if ((rc = upload(&d.vmset, vms, s))) break;
-    if ((rc = upload(&d.p32, p32, s))) break;
-    if ((rc = upload(&d.q32, q32, s))) break;
-    if ((rc = upload(&d.perm, y->perm, s))) break;
-    if ((rc = upload(&d.iperm, y->iperm, s))) break;
-    if ((rc = upload(&d.br_f, bf, s))) break;
-    if ((rc = upload(&d.br_t, bt, s))) break;
-    if ((rc = upload(&d.br_r, y->r, s))) break;
-    if ((rc = upload(&d.br_x, y->x, s))) break;
-    if ((rc = upload(&d.br_bch, y->b_ch, s))) break;
-    if ((rc = upload(&d.br_tap, y->tap, s))) break;
-    if ((rc = upload(&d.br_itap, itap, s))) break;
-    if ((rc = upload(&d.bridge, y->bridge, s))) break;
-    cudaError_t e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) { rc = fail(DPF_E_CUDA, "upload sync: %s", cudaGetErrorString(e)); break; }
-  } while (0);
+  // one allocation and one copy for all of them
+  std::vector<unsigned char> host;
+  std::vector<std::pair<void**, size_t>> at;
+  auto add = [&](auto** dst, const auto& src) {
+    const size_t o = (host.size() + 255) & ~(size_t)255, bytes = src.size() * sizeof(src[0]);
+    host.resize(o + bytes + 1);  // (an empty array gets an address too)
+    if (bytes) memcpy(host.data() + o, src.data(), bytes);
+    at.push_back({(void**)dst, o});
+  };
+  if (n <= RES_MAX_N) {
+    add(&d.res_rord, sell.rord);
+    add(&d.res_rpos, sell.rpos);
+    add(&d.res_soff, sell.soff);
+    add(&d.res_col2, sell.col2);
+    add(&d.res_val32, sell.val32);
+    add(&d.res_val64, sell.val64);
+    add(&d.res_bval, sell.bval);
+    add(&d.res_dinv, sell.dinv);
+    add(&d.res_upos, sell.upos);
+    add(&d.res_puser, sell.puser);
+    add(&d.res_slot, sell.slot);
+    d.res_slices = (int)sell.soff.size() - 1;
+    d.res_pairs = sell.soff.back();
+  }
+  add(&d.ent32, ent);
+  add(&d.row_ptr, y->irow_ptr);
+  add(&d.prow_ptr, y->iprow_ptr);
+  add(&d.ppos, y->ippos);
+  add(&d.col, y->icol);
+  add(&d.val64, v64);
+  add(&d.dcval, dcval2);
+  add(&d.dcinv, dcinv2);
+  add(&d.ebr, y->iebr);
+  add(&d.dpos, y->idpos);
+  add(&d.type, type);
+  add(&d.p64, p64);
+  add(&d.q64, q64);
+  add(&d.vmset, vms);
+  add(&d.p32, p32);
+  add(&d.q32, q32);
+  add(&d.perm, y->perm);
+  add(&d.iperm, y->iperm);
+  add(&d.br_f, bf);
+  add(&d.br_t, bt);
+  add(&d.br_r, y->r);
+  add(&d.br_x, y->x);
+  add(&d.br_bch, y->b_ch);
+  add(&d.br_tap, y->tap);
+  add(&d.br_itap, itap);
+  add(&d.bridge, y->bridge);
+  int rc = dalloc(&d.arena, host.size());
+  if (rc == DPF_OK) {
+    for (auto& p : at) *p.first = d.arena + p.second;
+    cudaError_t e = cudaMemcpyAsync(d.arena, host.data(), host.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) rc = fail(DPF_E_CUDA, "upload: %s", cudaGetErrorString(e));
+  }
   if (rc != DPF_OK) {
     free_device(d);
     return rc;
@@ -333,6 +347,8 @@ struct dpf_workspace {
   // Y values rebuilt from caller branch parameters
   int4* ent_loc = nullptr;
   double2* val_loc = nullptr;
+  float2* sell32_loc = nullptr;  // the same in the sliced form (grids that have one)
+  double2* sell64_loc = nullptr;
   // per-case buffers
   int32_t *active = nullptr, *iters = nullptr, *status = nullptr, *of = nullptr, *ot = nullptr;
   int32_t *bad = nullptr, *cool = nullptr;
@@ -396,7 +412,7 @@ static void ws_free_buffers(dpf_workspace* w) {
                    &w->sbuf, &w->cbuf, &w->step_size, &w->isbc2, &w->yff, &w->yft, &w->ytt};
   for (void** p : ptrs) dfree(*p);
   dfree(w->p64); dfree(w->q64); dfree(w->tmp_a); dfree(w->tmp_b); dfree(w->tmp_c); dfree(w->V64);
-  dfree(w->ent_loc); dfree(w->val_loc);
+  dfree(w->ent_loc); dfree(w->val_loc); dfree(w->sell32_loc); dfree(w->sell64_loc);
   dfree(w->active); dfree(w->iters); dfree(w->status); dfree(w->of); dfree(w->ot); dfree(w->bad); dfree(w->cool);
   dfree(w->lr); dfree(w->best); dfree(w->out_max); dfree(w->out_loss); dfree(w->loss64);
   dfree(w->yff64); dfree(w->yft64); dfree(w->ytt64); dfree(w->maxmis); dfree(w->outage_dev);
@@ -2014,6 +2030,26 @@ extern "C" int dpf_autotune(const dpf_ybus* y, dpf_workspace* w, const dpf_batch
 // ---------------------------------------------------------------------------
 // Evaluation entry points
 // ---------------------------------------------------------------------------
+// Argument checks of an evaluation on chip (those of eval_setup and
+// init_state), and the workspace's earlier uses ended.
+static int eval_chip_begin(const dpf_ybus* y, dpf_workspace* w, int K, int precision, const double* va,
+                           const double* vm, const double* p, const double* q, const int32_t* outage,
+                           cudaStream_t s) {
+  TRY(common_checks(y, w, K));
+  if (precision != DPF_FP32 && precision != DPF_FP64) return fail(DPF_E_INVALID, "unknown precision");
+  if (!va || !vm) return fail(DPF_E_INVALID, "va and vm are required");
+  w->begun = false;
+  w->pid_ready = false;
+  ws_drop_graph(w);
+  dpf_default_opts(&w->opts);
+  w->opts.precision = precision;
+  w->precision = precision;
+  w->K = K;
+  if ((p == nullptr) != (q == nullptr)) return fail(DPF_E_INVALID, "p_spec and q_spec must be given together");
+  if (outage) TRY(check_outages(w, outage, false, s));
+  return DPF_OK;
+}
+
 static int eval_setup(const dpf_ybus* y, dpf_workspace* w, int K, int precision, const double* va,
                       const double* vm, const double* p, const double* q, const int32_t* outage,
                       cudaStream_t s) {
@@ -2070,6 +2106,19 @@ extern "C" int dpf_power(const dpf_ybus* y, dpf_workspace* w, int32_t n_case, co
   dpf::Range nvtx_range("dpf_power");
   clear_error();
   cudaStream_t s = (cudaStream_t)stream;
+  if (y && y->dev.res_rord) {  // (every grid up to RES_MAX_N buses)
+    TRY(eval_chip_begin(y, w, n_case, precision, va, vm, nullptr, nullptr, outage, s));
+    EvalCall c = {};
+    c.K = n_case;
+    c.va = va;
+    c.vm = vm;
+    c.outage = outage;
+    c.o_p = p_calc;
+    c.o_q = q_calc;
+    CK((cudaError_t)eval_launch(y, c, precision == DPF_FP64, s));
+    w->launches++;
+    return DPF_OK;
+  }
   TRY(eval_setup(y, w, n_case, precision, va, vm, nullptr, nullptr, outage, s));
   return precision == DPF_FP64 ? power_impl<double>(w, p_calc, q_calc, s) : power_impl<float>(w, p_calc, q_calc, s);
 }
@@ -2177,6 +2226,9 @@ static void rebuild_local_y(const dpf_ybus* y, dpf_workspace* w, const double* g
   ya.itap = y->dev.br_itap;
   ya.ent32 = w->ent_loc;
   ya.val64 = w->val_loc;
+  ya.slot = w->sell32_loc && w->sell64_loc ? y->dev.res_slot : nullptr;
+  ya.sell32 = w->sell32_loc;
+  ya.sell64 = w->sell64_loc;
   k_ybus_values<<<(y->n + 127) / 128, 128, 0, s>>>(ya);
   w->use_local_y = true;
 }
@@ -2191,6 +2243,51 @@ extern "C" int dpf_loss_backward(const dpf_ybus* y, dpf_workspace* w, int32_t n_
   cudaStream_t s = (cudaStream_t)stream;
   if ((g_series == nullptr) != (b_series == nullptr))
     return fail(DPF_E_INVALID, "g_series and b_series must be given together");
+  if (y && y->dev.res_rord) {  // (every grid up to RES_MAX_N buses)
+    TRY(eval_chip_begin(y, w, n_case, precision, va, vm, p_spec, q_spec, outage, s));
+    EvalCall c = {};
+    c.K = n_case;
+    c.backward = true;
+    c.va = va;
+    c.vm = vm;
+    c.p = p_spec;
+    c.q = q_spec;
+    c.outage = outage;
+    c.loss = loss;
+    c.d_va = d_va;
+    c.d_vm = d_vm;
+    c.d_p = d_p;
+    c.d_q = d_q;
+    if (g_series) {
+      const size_t n = (size_t)y->dev.res_pairs * 64;
+      if (!w->sell32_loc) {  // (pads stay zero)
+        TRY(dalloc(&w->sell32_loc, n));
+        CK(cudaMemsetAsync(w->sell32_loc, 0, n * sizeof(float2), s));
+      }
+      if (!w->sell64_loc) {
+        TRY(dalloc(&w->sell64_loc, n));
+        CK(cudaMemsetAsync(w->sell64_loc, 0, n * sizeof(double2), s));
+      }
+      rebuild_local_y(y, w, g_series, b_series, s);
+      CKLAUNCH();
+      w->use_local_y = false;
+      c.val32 = w->sell32_loc;
+      c.val64 = w->sell64_loc;
+    }
+    const bool branch = d_g || d_b || d_bch;
+    if (branch) {  // V and w in the layout of the branch adjoint
+      choose_shape(w, nullptr, n_case);
+      TRY(ws_reserve(w, w->Kp, 0));
+      c.Kp = w->Kp;
+      c.Vout = w->V;
+      c.Wout = w->W;
+    }
+    CK((cudaError_t)eval_launch(y, c, precision == DPF_FP64, s));
+    w->launches++;
+    if (!branch) return DPF_OK;
+    return precision == DPF_FP64 ? launch_edge_grad<double>(w, d_g, d_b, d_bch, s)
+                                 : launch_edge_grad<float>(w, d_g, d_b, d_bch, s);
+  }
   TRY(eval_setup(y, w, n_case, precision, va, vm, p_spec, q_spec, outage, s));
   if (g_series) {
     rebuild_local_y(y, w, g_series, b_series, s);

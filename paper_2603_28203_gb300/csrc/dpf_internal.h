@@ -29,6 +29,7 @@ void clear_error();
 struct DeviceYbus {
   bool ready = false;
   int device = -1;
+  unsigned char* arena = nullptr;  // the allocation that holds every array below
   int4* ent32 = nullptr;        // [nnz] {col, re bits, im bits, 0}: one 16-byte load per nonzero
   int32_t* row_ptr = nullptr;   // [n+1]
   int32_t* prow_ptr = nullptr;  // [n+1] rows padded to multiples of 4 entries
@@ -66,6 +67,9 @@ struct DeviceYbus {
   double2* res_val64 = nullptr;
   float4* res_bval = nullptr;   // [pairs][32] the DC matrix in the same form, two (hi, lo) entries
   float2* res_dinv = nullptr;   // [slices * 32] dcinv by position
+  uint16_t* res_upos = nullptr; // [n] user bus -> position
+  uint16_t* res_puser = nullptr;
+  int32_t* res_slot = nullptr;  // [nnz] CSR entry -> its value's index in res_val32 / res_val64
   int res_pairs = 0, res_slices = 0;
 };
 

@@ -1893,6 +1893,9 @@ struct YValArgs {
   const double* itap;   // 1 / tap per branch
   int4* ent32;
   double2* val64;
+  const int32_t* slot;  // entry -> index in the sliced form's values, NULL: none
+  float2* sell32;
+  double2* sell64;
 };
 
 static __global__ void k_ybus_values(YValArgs a) {
@@ -1908,12 +1911,20 @@ static __global__ void k_ybus_values(YValArgs a) {
     const double vr = -gs * it, vi = -bs * it;
     a.val64[p] = make_double2(vr, vi);
     a.ent32[p] = make_int4(a.col[p], __float_as_int((float)vr), __float_as_int((float)vi), 0);
+    if (a.slot) {
+      a.sell32[a.slot[p]] = make_float2((float)vr, (float)vi);
+      a.sell64[a.slot[p]] = make_double2(vr, vi);
+    }
     if (a.br_f[ell] == i) { dr += gs * it2; di += (bs + sh) * it2; }
     else { dr += gs; di += bs + sh; }
   }
   if (pd >= 0) {
     a.val64[pd] = make_double2(dr, di);
     a.ent32[pd] = make_int4(i, __float_as_int((float)dr), __float_as_int((float)di), 0);
+    if (a.slot) {
+      a.sell32[a.slot[pd]] = make_float2((float)dr, (float)di);
+      a.sell64[a.slot[pd]] = make_double2(dr, di);
+    }
   }
 }
 

@@ -37,6 +37,7 @@
 
 #include "dpf_kernels.cuh"
 #include "dpf_resident.h"
+#include "dpf_sell.cuh"
 
 namespace dpf {
 
@@ -56,7 +57,6 @@ struct ResLayout {
   unsigned w, d, s, vr, rf, scr, sc, flag, team;  // offsets inside a team's block, its size
   unsigned val, col, soff, total;             // after the teams
 };
-template <class R> struct ValPair;
 template <class R> struct ResArgs {
   using C = typename Prec<R>::C;
   IterArgs<R> a;
@@ -277,29 +277,6 @@ template <class R> struct ResSched {
     }
   }
 };
-
-// Two adjacent entries of a row: their values, one aligned access.
-template <class R> struct __align__(16) ValPair { typename Prec<R>::C a, b; };
-
-// sum_e val[e] x[col[e]] over a row's entry pairs: even entries into a0, odd
-// into a1, as row_spmv does (pads: weight 0 on the row itself).
-template <class R>
-__device__ __forceinline__ typename Prec<R>::C sell_row(const ValPair<R>* __restrict__ val,
-                                                        const uint32_t* __restrict__ col2, int p0, int p1,
-                                                        const unsigned char* __restrict__ X) {
-  using C = typename Prec<R>::C;
-  constexpr unsigned sc = sizeof(C) / 8;
-  C a0 = mkc(R(0), R(0)), a1 = a0;
-  for (int p = p0; p < p1; p += 32) {
-    const uint32_t cc = col2[p];
-    const ValPair<R> y = val[p];
-    const C x0 = *reinterpret_cast<const C*>(X + (cc & 0xffffu) * sc);
-    const C x1 = *reinterpret_cast<const C*>(X + (cc >> 16) * sc);
-    cfma(a0, y.a, x0);
-    cfma(a1, y.b, x1);
-  }
-  return mkc(a0.x + a1.x, a0.y + a1.y);
-}
 
 // One row of a case held by a thread: master values and moments.
 template <class R> struct ResRow {

@@ -53,4 +53,19 @@ struct DcRes {
 // f32: FP32 vectors, else double-float.  Returns a cudaError_t.
 int dc_res_launch(const dpf_ybus* y, const DcRes& c, bool f32, void* stream);
 
+// Evaluation of whole cases on chip (dpf_eval.cu), one CTA per case: S_calc,
+// or the loss and its adjoint.  Inputs and outputs are the caller's case-major
+// arrays; outputs may be NULL.
+struct EvalCall {
+  int K, Kp;
+  bool backward;
+  const double *va, *vm, *p, *q;  // p, q NULL: the grid's
+  const int32_t* outage;
+  const void *val32, *val64;      // Y_bus values in the sliced form, NULL: as built
+  double *o_p, *o_q;              // backward = false
+  double *loss, *d_va, *d_vm, *d_p, *d_q;
+  void *Vout, *Wout;              // V and w in the layout [N][Kp], or NULL
+};
+int eval_launch(const dpf_ybus* y, const EvalCall& c, bool fp64, void* stream);
+
 }  // namespace dpf

@@ -185,3 +185,66 @@ def test_dc_on_chip_residual(n, K, tol):
         cap = dpf.dpf_dc_solve(y, ws, K, p_spec=torch.tensor(P, device=DEV), outage=torch.tensor(o, device=DEV),
                                tol=tol, max_iter=2)
         assert (cap["iters"].cpu().numpy() <= 2).all() and (cap["rel_residual"].cpu().numpy() > tol).any()
+
+
+# ---- evaluation on chip --------------------------------------------------------
+@pytest.mark.parametrize("n,K", [(2, 3), (31, 1), (33, 200), (513, 5), (1025, 160), (2048, 2)])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_evaluation_on_chip_against_oracle(n, K, precision):
+    """S_calc, loss and gradients at the edges of the slices and CTA sizes
+    (one row per thread up to 1,024 threads; 512 where cases outnumber SMs).
+    FP32 bars: a row's current carries |Y_ii| |V| 2^-24 times a few terms
+    (|Y_ii| up to ~200), 1e-4; gradients 1e-4 of their largest entry."""
+    import oracle
+    from oracle.ybus import grid_ybus
+    g = gridgen.two_bus(0.3, 0.1, 0.01, 0.1) if n == 2 else gridgen.make_grid(n, 3, load_scale=0.1)
+    Y = grid_ybus(g)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, 1)  # (an evaluation on chip needs no room in the workspace)
+    rng = np.random.default_rng(n)
+    va, vm = 0.1 * rng.standard_normal((K, n)), 1 + 0.03 * rng.standard_normal((K, n))
+    P, Q = g.p_spec * rng.uniform(0.9, 1.1, (K, 1)), g.q_spec * rng.uniform(0.9, 1.1, (K, 1))
+    t = lambda a: torch.tensor(a, device=DEV)  # noqa: E731
+    prec = dict(fp32=dpf.FP32, fp64=dpf.FP64)[precision]
+    tol = 1e-4 if precision == "fp32" else 1e-11
+    p, q = dpf.dpf_power(y, ws, t(va), t(vm), precision=prec)
+    out = dpf.dpf_loss_backward(y, ws, t(va), t(vm), t(P), t(Q), precision=prec,
+                                want=("loss", "d_va", "d_vm", "d_p", "d_q"))
+    for k in range(0, K, max(1, K // 5)):
+        V = vm[k] * np.exp(1j * va[k])
+        S = V * np.conj(Y @ V)
+        assert np.abs(p[k].cpu().numpy() - S.real).max() <= tol * max(1, np.abs(S).max())
+        assert np.abs(q[k].cpu().numpy() - S.imag).max() <= tol * max(1, np.abs(S).max())
+        L, ga, gm = oracle.loss_grad(Y, va[k], vm[k], P[k], Q[k], g.bus_type)
+        assert abs(out["loss"][k].item() - L) <= 1e-11 * L
+        scale = max(np.abs(ga).max(), np.abs(gm).max())
+        assert np.abs(out["d_va"][k].cpu().numpy() - ga).max() <= tol * scale
+        assert np.abs(out["d_vm"][k].cpu().numpy() - gm).max() <= tol * scale
+        act, rea, m = g.bus_type != gridgen.SLACK, g.bus_type == gridgen.PQ, (g.bus_type != 2).sum() + (g.bus_type == 0).sum()
+        c = 2.0 / m * (np.where(act, S.real - P[k], 0) + 1j * np.where(rea, S.imag - Q[k], 0))
+        assert np.abs(out["d_p"][k].cpu().numpy() + c.real).max() <= tol * np.abs(c).max()
+        assert np.abs(out["d_q"][k].cpu().numpy() + c.imag).max() <= tol * np.abs(c).max()
+
+
+def test_evaluation_on_chip_extreme_values():
+    """The integer FP64 <-> FP32 conversions hand what they do not cover (zeros,
+    subnormals, infinities, NaN, very small and large values) to the CUDA
+    ones: |V| at bus 0 of a two-bus grid scales P there quadratically."""
+    g = gridgen.two_bus(0.3, 0.1, 0.01, 0.1)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, 1)
+    ys = 1 / (g.r[0] + 1j * g.x[0])
+    m = np.array([0.0, -0.0, 1e-310, 1e-45, 1e-30, 1e-19, -1.5, 3.0, 1e10, 1e18, np.inf, np.nan])
+    va = np.zeros((m.size, 2))
+    vm = np.stack([m, np.zeros(m.size)], 1)  # bus 1 at 0: P_0 = g |V_0|^2
+    p, _ = dpf.dpf_power(y, ws, torch.tensor(va, device=DEV), torch.tensor(vm, device=DEV), precision=dpf.FP32)
+    p = p.cpu().numpy()[:, 0]
+    with np.errstate(all="ignore"):
+        want = ys.real * m.astype(np.float32).astype(np.float64) ** 2
+    for a, b in zip(p, want):
+        if not np.isfinite(b):
+            assert not np.isfinite(a)
+        elif abs(b) < 1e-36:  # below FP32's normal range
+            assert abs(a) <= 1e-36
+        elif abs(b) < 3e38:
+            assert abs(a - b) <= 1e-5 * abs(b)
