@@ -900,12 +900,11 @@ static int build_graph(dpf_workspace* w) {
 }
 
 // ---------------------------------------------------------------------------
-// State set-up shared by the solve and the evaluation entry points
+// State set-up of the solves
 // ---------------------------------------------------------------------------
 struct StateIn {
   int K;
   bool host_io;
-  bool enforce_fixed;  // solve: set-points override the given state; evaluation: state as given
   const double *va, *vm, *vmset, *p, *q;  // user layout [K][N] or NULL
   const double *va0, *vm0;                 // one start [N] shared by every case, or NULL
   const int32_t* outage;
@@ -1164,6 +1163,54 @@ static int check_outages(dpf_workspace* w, const int32_t* outage, bool host_io, 
   return DPF_OK;
 }
 
+// Per-case state and N-1 corrections of the w->K cases.
+template <class R>
+static int case_init(dpf_workspace* w, const int32_t* outage_dev, cudaStream_t s) {
+  const DeviceYbus& d = w->y->dev;
+  CaseInitArgs<R> ca;
+  memset(&ca, 0, sizeof ca);
+  ca.K = w->K;
+  ca.Kp = w->Kp;
+  ca.outage = outage_dev;
+  ca.br_f = d.br_f;
+  ca.br_t = d.br_t;
+  ca.br_r = d.br_r;
+  ca.br_x = d.br_x;
+  ca.br_bch = d.br_bch;
+  ca.br_tap = d.br_tap;
+  ca.of = w->of;
+  ca.ot = w->ot;
+  ca.yff = (typename Prec<R>::C*)w->yff;
+  ca.yft = (typename Prec<R>::C*)w->yft;
+  ca.ytt = (typename Prec<R>::C*)w->ytt;
+  ca.yff64 = w->yff64;
+  ca.yft64 = w->yft64;
+  ca.ytt64 = w->ytt64;
+  ca.active = w->active;
+  ca.iters = w->iters;
+  ca.status = w->status;
+  ca.lr = w->lr;
+  ca.best = w->best;
+  ca.bad = w->bad;
+  ca.cool = w->cool;
+  ca.step_size = (R*)w->step_size;
+  ca.isbc2 = (R*)w->isbc2;
+  ca.b1t = w->b1t;
+  ca.b2t = w->b2t;
+  ca.cand = w->cand;
+  ca.mx32 = w->mx32;
+  ca.maxmis = w->maxmis;
+  ca.loss64 = w->loss64;
+  ca.lr0 = w->opts.lr;
+  ca.beta1 = w->opts.beta1;
+  ca.beta2 = w->opts.beta2;
+  ca.opt = w->opts.optimizer;
+  k_case_init<R><<<(w->Kp + 255) / 256, 256, 0, s>>>(ca);
+  CKLAUNCH();
+  w->launches++;
+  return DPF_OK;
+}
+
 template <class R>
 static int init_state(dpf_workspace* w, const StateIn& in, cudaStream_t s) {
   const dpf_ybus* y = w->y;
@@ -1213,7 +1260,6 @@ static int init_state(dpf_workspace* w, const StateIn& in, cudaStream_t s) {
   ia.N = y->n;
   ia.K = w->K;
   ia.Kp = w->Kp;
-  ia.enforce_fixed = in.enforce_fixed ? 1 : 0;
   ia.type = d.type;
   ia.vmset_grid = d.vmset;
   ia.vms_t = vms_t;
@@ -1253,47 +1299,7 @@ static int init_state(dpf_workspace* w, const StateIn& in, cudaStream_t s) {
       outage_dev = in.outage;
     }
   }
-  CaseInitArgs<R> ca;
-  memset(&ca, 0, sizeof ca);
-  ca.K = w->K;
-  ca.Kp = w->Kp;
-  ca.outage = outage_dev;
-  ca.br_f = d.br_f;
-  ca.br_t = d.br_t;
-  ca.br_r = d.br_r;
-  ca.br_x = d.br_x;
-  ca.br_bch = d.br_bch;
-  ca.br_tap = d.br_tap;
-  ca.of = w->of;
-  ca.ot = w->ot;
-  ca.yff = (typename Prec<R>::C*)w->yff;
-  ca.yft = (typename Prec<R>::C*)w->yft;
-  ca.ytt = (typename Prec<R>::C*)w->ytt;
-  ca.yff64 = w->yff64;
-  ca.yft64 = w->yft64;
-  ca.ytt64 = w->ytt64;
-  ca.active = w->active;
-  ca.iters = w->iters;
-  ca.status = w->status;
-  ca.lr = w->lr;
-  ca.best = w->best;
-  ca.bad = w->bad;
-  ca.cool = w->cool;
-  ca.step_size = (R*)w->step_size;
-  ca.isbc2 = (R*)w->isbc2;
-  ca.b1t = w->b1t;
-  ca.b2t = w->b2t;
-  ca.cand = w->cand;
-  ca.mx32 = w->mx32;
-  ca.maxmis = w->maxmis;
-  ca.loss64 = w->loss64;
-  ca.lr0 = w->opts.lr;
-  ca.beta1 = w->opts.beta1;
-  ca.beta2 = w->opts.beta2;
-  ca.opt = w->opts.optimizer;
-  k_case_init<R><<<(w->Kp + 255) / 256, 256, 0, s>>>(ca);
-  CKLAUNCH();
-  w->launches++;
+  TRY(case_init<R>(w, outage_dev, s));
   CK(cudaMemcpyAsync(w->n_active, &w->K, 4, cudaMemcpyHostToDevice, s));
   CK(cudaStreamSynchronize(s));  // &w->K is host memory that may change later
   return DPF_OK;
@@ -1492,7 +1498,6 @@ extern "C" int dpf_dc_solve(const dpf_ybus* y, dpf_workspace* w, int32_t n_case,
   StateIn in;
   memset(&in, 0, sizeof in);
   in.K = n_case;
-  in.enforce_fixed = true;
   in.p = p_spec;
   in.q = p_spec;  // (the DC model reads only P)
   in.outage = outage;
@@ -1536,7 +1541,6 @@ extern "C" int dpf_solve_begin(const dpf_ybus* y, dpf_workspace* w, const dpf_ba
   memset(&in, 0, sizeof in);
   in.K = w->K;
   in.host_io = b->host_io != 0;
-  in.enforce_fixed = true;
   if (!o->flat_start) {
     in.va = b->va;
     in.vm = b->vm;
@@ -1891,7 +1895,7 @@ extern "C" int dpf_solve_batch(const dpf_ybus* y, dpf_workspace* ws, const dpf_b
 // ---------------------------------------------------------------------------
 __global__ void k_adam_params(int n, double* __restrict__ x, const double* __restrict__ g, double* __restrict__ m,
                               double* __restrict__ v, const double* __restrict__ lr_scale, double lr, double b1,
-                              double b2, double eps, double bc1, double bc2) {
+                              double b2, double eps, double ibc1, double ibc2) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double gi = g[i];
@@ -1900,7 +1904,7 @@ __global__ void k_adam_params(int n, double* __restrict__ x, const double* __res
   m[i] = mi;
   v[i] = vi;
   const double step = lr * (lr_scale ? lr_scale[i] : 1.0);
-  x[i] -= step * (mi / bc1) / (sqrt(vi / bc2) + eps);
+  x[i] -= step * (mi * ibc1) / (sqrt(vi * ibc2) + eps);  // (an FP64 division costs tens of its multiplications)
 }
 
 extern "C" int dpf_adam_update(int32_t n, double* x, const double* grad, double* m, double* v,
@@ -1913,8 +1917,8 @@ extern "C" int dpf_adam_update(int32_t n, double* x, const double* grad, double*
   if (n == 0) return DPF_OK;
   double b1t = 1.0, b2t = 1.0;  // host powers: one scalar each per call
   for (int k = 0; k < t; ++k) { b1t *= beta1; b2t *= beta2; }
-  k_adam_params<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(n, x, grad, m, v, lr_scale, lr, beta1, beta2,
-                                                                    eps, 1.0 - b1t, 1.0 - b2t);
+  k_adam_params<<<(n + 63) / 64, 64, 0, (cudaStream_t)stream>>>(n, x, grad, m, v, lr_scale, lr, beta1, beta2,
+                                                                    eps, 1.0 / (1.0 - b1t), 1.0 / (1.0 - b2t));
   CKLAUNCH();
   return DPF_OK;
 }
@@ -2050,6 +2054,37 @@ static int eval_chip_begin(const dpf_ybus* y, dpf_workspace* w, int K, int preci
   return DPF_OK;
 }
 
+// State of an evaluation of grids above RES_MAX_N buses: the caller's state and
+// injections into the workspace layout (one kernel), outages and the case
+// flags.  No host synchronisation (but for an outage list's check).
+template <class R>
+static int eval_state(dpf_workspace* w, const double* va, const double* vm, const double* p, const double* q,
+                      const int32_t* outage, cudaStream_t s) {
+  const dpf_ybus* y = w->y;
+  w->spec_per_case = p != nullptr;
+  EvalInArgs<R> ia;
+  ia.N = y->n;
+  ia.K = w->K;
+  ia.Kp = w->Kp;
+  ia.iperm = y->dev.iperm;
+  ia.va = va;
+  ia.vm = vm;
+  ia.p = p;
+  ia.q = q;
+  ia.ms = (typename Prec<R>::MS*)w->ms;
+  ia.V = (typename Prec<R>::C*)w->V;
+  ia.p64 = w->p64;
+  ia.q64 = w->q64;
+  ia.pw = (R*)w->p;
+  ia.qw = (R*)w->q;
+  k_eval_in<R><<<dim3((y->n + 31) / 32, (w->Kp + 31) / 32), dim3(32, 8), 0, s>>>(ia);
+  CKLAUNCH();
+  w->launches++;
+  w->has_outage = outage != nullptr;
+  if (outage) TRY(check_outages(w, outage, false, s));
+  return case_init<R>(w, outage, s);
+}
+
 static int eval_setup(const dpf_ybus* y, dpf_workspace* w, int K, int precision, const double* va,
                       const double* vm, const double* p, const double* q, const int32_t* outage,
                       cudaStream_t s) {
@@ -2064,19 +2099,42 @@ static int eval_setup(const dpf_ybus* y, dpf_workspace* w, int K, int precision,
   w->precision = precision;
   w->K = K;
   choose_shape(w, nullptr, K);
-  TRY(upload_windows(w, s));
   TRY(precision == DPF_FP64 ? set_smem_attr<double>(std::max(w->smem, w->ysmem_b))
                             : set_smem_attr<float>(std::max(w->smem, w->ysmem_b)));
   TRY(ws_reserve(w, w->Kp, 0));
-  StateIn in;
-  memset(&in, 0, sizeof in);
-  in.K = K;
-  in.va = va;
-  in.vm = vm;
-  in.p = p;
-  in.q = q;
-  in.outage = outage;
-  return precision == DPF_FP64 ? init_state<double>(w, in, s) : init_state<float>(w, in, s);
+  if ((p == nullptr) != (q == nullptr)) return fail(DPF_E_INVALID, "p_spec and q_spec must be given together");
+  return precision == DPF_FP64 ? eval_state<double>(w, va, vm, p, q, outage, s)
+                               : eval_state<float>(w, va, vm, p, q, outage, s);
+}
+
+// Working-precision results to the caller's arrays.
+template <class R>
+static int eval_out(dpf_workspace* w, const R* s0, const R* s1, size_t stride, double sign, double* d0, double* d1,
+                    cudaStream_t s) {
+  if (!d0 && !d1) return DPF_OK;
+  const dpf_ybus* y = w->y;
+  k_eval_out<R><<<dim3((y->n + 31) / 32, (w->K + 31) / 32), dim3(32, 8), 0, s>>>(s0, s1, stride, sign, w->K, y->n,
+                                                                                w->Kp, y->dev.iperm, d0, d1);
+  CKLAUNCH();
+  w->launches++;
+  return DPF_OK;
+}
+
+// FP64 loss per case of the staged state.
+template <class R>
+static int eval_loss(dpf_workspace* w, double* loss, cudaStream_t s) {
+  Plan<R> P = make_plan<R>(w);
+  P.ck.all_cases = 1;
+  using M = typename Prec<R>::M;
+  if (P.need_volt64) {
+    k_volt64<M><<<P.cgrid, P.block, 0, s>>>(P.ck);
+    w->launches++;
+  }
+  k_check64<M><<<P.cgrid, P.block, 0, s>>>(P.ck);
+  k_eval_loss<<<(w->K + 255) / 256, 256, 0, s>>>(w->loss64, P.ap.inv_m, w->K, loss);
+  CKLAUNCH();
+  w->launches += 2;
+  return DPF_OK;
 }
 
 template <class R>
@@ -2088,16 +2146,8 @@ static int power_impl(dpf_workspace* w, double* p_calc, double* q_calc, cudaStre
   P.it.tile_cnt = nullptr;
   k_fwd<R><<<P.grid, P.block, P.smem, s>>>(P.it);
   w->launches++;
-  const size_t E = (size_t)w->y->n * w->Kp;
-  const int nb = (int)std::min<size_t>((E + 255) / 256, (size_t)num_sms() * 16);
-  k_widen<R><<<nb, 256, 0, s>>>((const R*)w->sbuf, w->tmp_a, E, 2, 1.0);
-  w->launches++;
-  k_widen<R><<<nb, 256, 0, s>>>((const R*)w->sbuf + 1, w->tmp_b, E, 2, 1.0);
-  w->launches++;
   CKLAUNCH();
-  if (p_calc) TRY(to_user(w, w->tmp_a, false, nullptr, p_calc, s));
-  if (q_calc) TRY(to_user(w, w->tmp_b, false, nullptr, q_calc, s));
-  return DPF_OK;
+  return eval_out<R>(w, (const R*)w->sbuf, (const R*)w->sbuf + 1, 2, 1.0, p_calc, q_calc, s);
 }
 
 extern "C" int dpf_power(const dpf_ybus* y, dpf_workspace* w, int32_t n_case, const double* va,
@@ -2129,9 +2179,10 @@ template <class R>
 static int launch_edge_grad(dpf_workspace* w, double* d_g, double* d_b, double* d_bch, cudaStream_t s) {
   using C = typename Prec<R>::C;
   const dpf_ybus* y = w->y;
-  if (d_g) CK(cudaMemsetAsync(d_g, 0, (size_t)y->m * 8, s));
-  if (d_b) CK(cudaMemsetAsync(d_b, 0, (size_t)y->m * 8, s));
-  if (d_bch) CK(cudaMemsetAsync(d_bch, 0, (size_t)y->m * 8, s));
+  const bool add = w->gx > 1;  // (one case tile stores its sums)
+  if (add && d_g) CK(cudaMemsetAsync(d_g, 0, (size_t)y->m * 8, s));
+  if (add && d_b) CK(cudaMemsetAsync(d_b, 0, (size_t)y->m * 8, s));
+  if (add && d_bch) CK(cudaMemsetAsync(d_bch, 0, (size_t)y->m * 8, s));
   EdgeArgs<R> ea;
   memset(&ea, 0, sizeof ea);
   ea.M = y->m;
@@ -2146,6 +2197,7 @@ static int launch_edge_grad(dpf_workspace* w, double* d_g, double* d_b, double* 
   ea.d_g = d_g;
   ea.d_b = d_b;
   ea.d_bch = d_bch;
+  ea.add = add ? 1 : 0;
   const int rpw = 32 / w->lanes;
   const int gy = std::max(1, std::min((y->m + w->warps * rpw - 1) / (w->warps * rpw), 65535));
   k_edge_grad<R><<<dim3(w->gx, gy), dim3(w->warps * 32), 0, s>>>(ea);
@@ -2158,7 +2210,6 @@ template <class R>
 static int loss_backward_impl(dpf_workspace* w, double* loss, double* d_va, double* d_vm, double* d_p,
                               double* d_q, double* d_g, double* d_b, double* d_bch, cudaStream_t s) {
   using C = typename Prec<R>::C;
-  const dpf_ybus* y = w->y;
   Plan<R> P = make_plan<R>(w);
   P.it.cbuf = (d_p || d_q) ? (C*)w->cbuf : nullptr;
   P.it.loss_part = nullptr;  // (the loss is the FP64 pass's)
@@ -2168,8 +2219,6 @@ static int loss_backward_impl(dpf_workspace* w, double* loss, double* d_va, doub
   k_fwd<R><<<P.grid, P.block, P.smem, s>>>(P.it);
   w->launches++;
   CKLAUNCH();
-  const size_t E = (size_t)y->n * w->Kp;
-  const int nb = (int)std::min<size_t>((E + 255) / 256, (size_t)num_sms() * 16);
   if (d_va || d_vm) {  // the voltage adjoint (the branch adjoint needs only w and V)
     P.it.gva = (R*)w->tmp_c;  // gradient scratch: [N][Kp] R each
     P.it.gvm = (R*)w->sbuf;
@@ -2179,36 +2228,10 @@ static int loss_backward_impl(dpf_workspace* w, double* loss, double* d_va, doub
     w->launches++;
     CKLAUNCH();
   }
-  if (d_va) {
-    k_widen<R><<<nb, 256, 0, s>>>((const R*)w->tmp_c, w->tmp_a, E, 1, 1.0);
-    w->launches++;
-    CKLAUNCH();
-    TRY(to_user(w, w->tmp_a, false, nullptr, d_va, s));
-  }
-  if (d_vm) {
-    k_widen<R><<<nb, 256, 0, s>>>((const R*)w->sbuf, w->tmp_a, E, 1, 1.0);
-    w->launches++;
-    CKLAUNCH();
-    TRY(to_user(w, w->tmp_a, false, nullptr, d_vm, s));
-  }
-  if (d_p) {
-    k_widen<R><<<nb, 256, 0, s>>>((const R*)w->cbuf, w->tmp_a, E, 2, -1.0);
-    w->launches++;
-    CKLAUNCH();
-    TRY(to_user(w, w->tmp_a, false, nullptr, d_p, s));
-  }
-  if (d_q) {
-    k_widen<R><<<nb, 256, 0, s>>>((const R*)w->cbuf + 1, w->tmp_a, E, 2, -1.0);
-    w->launches++;
-    CKLAUNCH();
-    TRY(to_user(w, w->tmp_a, false, nullptr, d_q, s));
-  }
+  TRY(eval_out<R>(w, (const R*)w->tmp_c, (const R*)w->sbuf, 1, 1.0, d_va, d_vm, s));
+  TRY(eval_out<R>(w, (const R*)w->cbuf, (const R*)w->cbuf + 1, 2, -1.0, d_p, d_q, s));
   if (d_g || d_b || d_bch) TRY(launch_edge_grad<R>(w, d_g, d_b, d_bch, s));
-  if (loss) {
-    TRY(launch_check<R>(w, s, true));
-    CK(cudaMemcpyAsync(loss, w->out_loss, (size_t)w->K * 8, cudaMemcpyDeviceToDevice, s));
-  }
-  return DPF_OK;
+  return loss ? eval_loss<R>(w, loss, s) : DPF_OK;
 }
 
 // Y_bus values from caller series admittances (the workspace's local copy).
@@ -2229,7 +2252,7 @@ static void rebuild_local_y(const dpf_ybus* y, dpf_workspace* w, const double* g
   ya.slot = w->sell32_loc && w->sell64_loc ? y->dev.res_slot : nullptr;
   ya.sell32 = w->sell32_loc;
   ya.sell64 = w->sell64_loc;
-  k_ybus_values<<<(y->n + 127) / 128, 128, 0, s>>>(ya);
+  k_ybus_values<<<(y->n + 63) / 64, 64, 0, s>>>(ya);
   w->use_local_y = true;
 }
 
@@ -2317,8 +2340,6 @@ extern "C" int dpf_paramid_begin(const dpf_ybus* y, dpf_workspace* w, int32_t n_
 
 template <class R>
 static int paramid_impl(dpf_workspace* w, double* d_g, double* d_b, double* d_bch, double* loss, cudaStream_t s) {
-  k_activate<<<(w->Kp + 255) / 256, 256, 0, s>>>(w->active, w->K, w->Kp);
-  w->launches++;
   Plan<R> P = make_plan<R>(w);
   P.it.cbuf = nullptr;
   P.it.loss_part = nullptr;
@@ -2329,11 +2350,9 @@ static int paramid_impl(dpf_workspace* w, double* d_g, double* d_b, double* d_bc
   w->launches++;
   CKLAUNCH();
   if (d_g || d_b || d_bch) TRY(launch_edge_grad<R>(w, d_g, d_b, d_bch, s));
-  if (loss) {
-    TRY(launch_check<R>(w, s, true));
-    CK(cudaMemcpyAsync(loss, w->out_loss, (size_t)w->K * 8, cudaMemcpyDeviceToDevice, s));
-  }
-  return DPF_OK;
+  if (!loss) return DPF_OK;
+  CK(cudaMemsetAsync(w->loss64, 0, (size_t)w->Kp * 8, s));  // the sums of an earlier step
+  return eval_loss<R>(w, loss, s);
 }
 
 extern "C" int dpf_paramid_step(const dpf_ybus* y, dpf_workspace* w, const double* g_series,

@@ -56,33 +56,6 @@ template <class R> struct EvalArgs {
   unsigned w, s, c, m, v64;
 };
 
-// FP64 -> (hi, lo) as mfrom<float2>: hi = v rounded to FP32, lo = v - hi
-// rounded to FP32.  Integer arithmetic where neither word is subnormal.
-__device__ __forceinline__ float2 split_df(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const int e = (int)((b >> 52) & 0x7ff) - 1023;
-  if (e >= -60 && e <= 60) {
-    const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
-    unsigned top = (unsigned)(m >> 29);
-    const unsigned rem = (unsigned)m & 0x1fffffffu;
-    const unsigned up = (rem > 0x10000000u || (rem == 0x10000000u && (top & 1u))) ? 1u : 0u;
-    top += up;
-    int r = (int)rem - (int)(up << 29);
-    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
-    if (sign) r = -r;
-    const float hi = __uint_as_float(sign | (((unsigned)(e + 127) << 23) + (top - 0x800000u)));
-    return make_float2(hi, (float)r * __uint_as_float((unsigned)(e - 52 + 127) << 23));
-  }
-  return mfrom<float2>(v);
-}
-// FP32 -> FP64 (exact)
-__device__ __forceinline__ double widen(float f) {
-  const unsigned u = __float_as_uint(f), ex = (u >> 23) & 0xff;
-  if (ex == 0 || ex == 255) return (u << 1) == 0 ? __hiloint2double((int)u, 0) : (double)f;
-  return __hiloint2double((int)((u & 0x80000000u) | (((ex + 896u) << 20) | ((u & 0x7fffffu) >> 3))), (int)(u << 29));
-}
-__device__ __forceinline__ double widen(double f) { return f; }
-
 // Working-precision state of one bus from the caller's FP64 (theta, |V|).
 __device__ __forceinline__ void eval_volt(double va, double vm, float2& v, float& m, double2* v64) {
   const float2 th = split_df(va), mg = split_df(vm);
@@ -90,8 +63,8 @@ __device__ __forceinline__ void eval_volt(double va, double vm, float2& v, float
   m = mwork(mg);
   if (v64) {  // the master value, 48 bits, as the streaming FP64 pass sees it
     double s, c;
-    sincos(widen(th.x) + widen(th.y), &s, &c);
-    const double w = widen(mg.x) + widen(mg.y);
+    sincos(mval(th), &s, &c);
+    const double w = mval(mg);
     *v64 = make_double2(w * c, w * s);
   }
 }
@@ -99,9 +72,6 @@ __device__ __forceinline__ void eval_volt(double va, double vm, double2& v, doub
   v = volt(va, vm);
   m = vm;
 }
-__device__ __forceinline__ float to_work(double v, float) { return split_df(v).x; }
-__device__ __forceinline__ double to_work(double v, double) { return v; }
-
 // BWD: the adjoint pass; LOSS: the FP64 loss (in FP32 from an FP64 pass over
 // the same state).
 template <class R, bool BWD, bool LOSS>

@@ -148,7 +148,52 @@ __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.lau
 // FP32 mode keeps theta and |V| as an unevaluated sum hi + lo of two floats
 // (~48 significant bits) and updates them with an error-free two-sum, so the
 // per-iteration path needs no FP64 instruction.
-__device__ __forceinline__ double mval(float2 m) { return (double)m.x + (double)m.y; }
+//
+// Conversions between FP64 and FP32 are written as integer arithmetic: GB300
+// issues an FP64 instruction, conversions included, in about 16 cycles per
+// warp and SM, these take a handful of single-cycle ones.  Same values; what
+// they do not cover goes to the CUDA conversion.
+// FP32 -> FP64 (exact)
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), ex = (u >> 23) & 0xff;
+  if (ex == 0 || ex == 255) return (u << 1) == 0 ? __hiloint2double((int)u, 0) : (double)f;
+  return __hiloint2double((int)((u & 0x80000000u) | (((ex + 896u) << 20) | ((u & 0x7fffffu) >> 3))), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+// FP64 -> (hi, lo): hi = v rounded to FP32, lo = v - hi rounded to FP32
+// (integers where neither word is subnormal).
+__device__ __forceinline__ float2 split_df(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int e = (int)((b >> 52) & 0x7ff) - 1023;
+  if (e >= -60 && e <= 60) {
+    const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    unsigned top = (unsigned)(m >> 29);
+    const unsigned rem = (unsigned)m & 0x1fffffffu;
+    const unsigned up = (rem > 0x10000000u || (rem == 0x10000000u && (top & 1u))) ? 1u : 0u;
+    top += up;
+    int r = (int)rem - (int)(up << 29);
+    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+    if (sign) r = -r;
+    const float hi = __uint_as_float(sign | (((unsigned)(e + 127) << 23) + (top - 0x800000u)));
+    return make_float2(hi, (float)r * __uint_as_float((unsigned)(e - 52 + 127) << 23));
+  }
+  const float hi = (float)v;
+  return make_float2(hi, (float)(v - (double)hi));
+}
+// FP64 -> FP32, rounded to nearest even
+__device__ __forceinline__ float narrow(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned e = (hi >> 20) & 0x7ff;
+  if (e > 1023 - 126 && e < 1023 + 127) {  // a normal result, no overflow by rounding
+    const unsigned top = (((e - 896u) << 23) | ((hi & 0xfffffu) << 3)) + (lo >> 29), rem = lo & 0x1fffffffu;
+    const unsigned up = (rem > 0x10000000u || (rem == 0x10000000u && (top & 1u))) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (top + up));
+  }
+  return (float)v;
+}
+__device__ __forceinline__ float to_work(double v, float) { return narrow(v); }
+__device__ __forceinline__ double to_work(double v, double) { return v; }
+__device__ __forceinline__ double mval(float2 m) { return widen(m.x) + widen(m.y); }
 __device__ __forceinline__ double mval(double m) { return m; }
 __device__ __forceinline__ float mwork(float2 m) { return m.x + m.y; }
 __device__ __forceinline__ double mwork(double m) { return m; }
@@ -165,10 +210,7 @@ __device__ __forceinline__ float2 msub(float2 a, float d) {
 __device__ __forceinline__ double msub(double a, double d) { return a - d; }
 
 template <class M> __device__ __forceinline__ M mfrom(double v);
-template <> __device__ __forceinline__ float2 mfrom<float2>(double v) {
-  const float hi = (float)v;
-  return make_float2(hi, (float)(v - (double)hi));
-}
+template <> __device__ __forceinline__ float2 mfrom<float2>(double v) { return split_df(v); }
 template <> __device__ __forceinline__ double mfrom<double>(double v) { return v; }
 
 // (theta, |V|) master pair of one element
@@ -1569,7 +1611,10 @@ __global__ void __launch_bounds__(1024) k_check64(Check64Args<M> a) {
   const Map mp = thread_map(a.lanes);
   const int k = mp.k;
   const bool on = (k < a.Kp) && (a.all_cases || (a.active[k] && examined(a.cand, a.iters, a.full_every, k)));
-  double mx = 0.0, sq = 0.0;
+  // max |f| on the bit patterns (a magnitude's order is its bits' order; a NaN
+  // is above infinity): an FP64 comparison costs as much as a product
+  unsigned long long mxb = 0;
+  double sq = 0.0;
   if (on) {
     int of = -1, ot = -1;
     double2 yff = make_double2(0, 0), yft = yff, ytt = yff;
@@ -1600,18 +1645,19 @@ __global__ void __launch_bounds__(1024) k_check64(Check64Args<M> a) {
       const size_t si = a.spec_per_case ? e : (size_t)i;
       const double dP = (ty != BUS_SLACK) ? P - a.pspec[si] : 0.0;
       const double dQ = (ty == BUS_PQ) ? Q - a.qspec[si] : 0.0;
-      // a NaN mismatch is recorded as +inf so that it survives the max reduction
-      const double am = (isnan(dP) || isnan(dQ)) ? __longlong_as_double(0x7ff0000000000000LL)
-                                                 : fmax(fabs(dP), fabs(dQ));
-      mx = fmax(mx, am);
+      const unsigned long long bp = (unsigned long long)__double_as_longlong(dP) & 0x7fffffffffffffffull;
+      const unsigned long long bq = (unsigned long long)__double_as_longlong(dQ) & 0x7fffffffffffffffull;
+      mxb = max(mxb, max(bp, bq));
       sq += dP * dP + dQ * dQ;
       if (a.refresh) {
-        a.vref[e] = make_float2((float)vi.x, (float)vi.y);
-        a.irf[e] = make_float4((float)I.x, (float)I.y, (float)dP, (float)((ty == BUS_PV) ? Q : dQ));
+        a.vref[e] = make_float2(narrow(vi.x), narrow(vi.y));
+        a.irf[e] = make_float4(narrow(I.x), narrow(I.y), narrow(dP), narrow((ty == BUS_PV) ? Q : dQ));
         a.dv[e] = make_float2(0.f, 0.f);
       }
     }
   }
+  // a NaN mismatch is recorded as +inf so that it survives the max reduction
+  const double mx = __longlong_as_double((long long)min(mxb, 0x7ff0000000000000ull));
   case_max_sum_atomic(mx, sq, a.lanes, a.maxmis, a.loss64, a.Kp);
 }
 
@@ -1685,12 +1731,6 @@ static __global__ void k_ref_init(const uint8_t* __restrict__ type, const float*
   }
 }
 
-// Re-activate the first K of Kp cases (a final convergence pass deactivates all).
-static __global__ void k_activate(int32_t* __restrict__ active, int K, int Kp) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < Kp) active[k] = (k < K) ? 1 : 0;
-}
-
 // ---- set-up / tear-down ----------------------------------------------------
 // Tiled transpose of a case-major [K][N] user-order FP64 array into the
 // case-minor internal layout [N][Kp] (row iperm[u] for user bus u).
@@ -1731,7 +1771,6 @@ template <class R> struct InitArgs {
   using C = typename Prec<R>::C;
   using M = typename Prec<R>::M;
   int N, K, Kp;
-  int enforce_fixed;         // 1: slack angle and pv/slack |V| set from the specification
   const uint8_t* type;
   const double* vmset_grid;  // [N]
   const double* vms_t;       // [N][Kp] or NULL
@@ -1762,19 +1801,17 @@ __global__ void k_init(InitArgs<R> a) {
         th = a.va_t[si];
         vm = a.vm_t[si];
       }
-      if (a.enforce_fixed || !a.va_t) {
-        const double set = a.vms_t ? a.vms_t[e] : a.vmset_grid[i];
-        if (ty != BUS_PQ) vm = set;
-        if (ty == BUS_SLACK) th = a.va_slack;
-      }
+      // slack angle and pv/slack |V| from the specification
+      if (ty != BUS_PQ) vm = a.vms_t ? a.vms_t[e] : a.vmset_grid[i];
+      if (ty == BUS_SLACK) th = a.va_slack;
     }
     const M mth = mfrom<M>(th), mvm = mfrom<M>(vm);
     a.ms[e] = ms_make(mth, mvm);
     a.V[e] = volt(mth, mvm);
     a.os[e] = Mom<R>{R(0), R(0), R(0), R(0)};
     if (a.p64) {
-      a.p[e] = (R)a.p64[e];
-      a.q[e] = (R)a.q64[e];
+      a.p[e] = to_work(a.p64[e], R(0));
+      a.q[e] = to_work(a.q64[e], R(0));
     }
   }
 }
@@ -1871,13 +1908,6 @@ __global__ void k_master64(const MS* __restrict__ src, double* __restrict__ th, 
   }
 }
 
-// working precision -> FP64, optional scale (outputs of the evaluation calls)
-template <class R>
-__global__ void k_widen(const R* __restrict__ src, double* __restrict__ dst, size_t n, size_t stride, double scale) {
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
-    dst[e] = scale * (double)src[e * stride];
-}
-
 // Y_bus values from per-branch series admittance (g + jb), charging and taps,
 // one thread per internal row: off-diagonal entries -y_s/tau, diagonal the
 // sum of the incident branches' end contributions.
@@ -1903,20 +1933,39 @@ static __global__ void k_ybus_values(YValArgs a) {
   if (i >= a.N) return;
   double dr = 0.0, di = 0.0;
   int pd = -1;
-  for (int p = a.rp[i]; p < a.rp[i + 1]; ++p) {
-    const int ell = a.ebr[p];
-    if (ell < 0) { pd = p; continue; }
-    const double it = a.itap[ell], it2 = it * it;
-    const double gs = a.g[ell], bs = a.b[ell], sh = 0.5 * a.bch[ell];
-    const double vr = -gs * it, vi = -bs * it;
-    a.val64[p] = make_double2(vr, vi);
-    a.ent32[p] = make_int4(a.col[p], __float_as_int((float)vr), __float_as_int((float)vi), 0);
-    if (a.slot) {
-      a.sell32[a.slot[p]] = make_float2((float)vr, (float)vi);
-      a.sell64[a.slot[p]] = make_double2(vr, vi);
+  const int p1 = a.rp[i + 1];
+  for (int p0 = a.rp[i]; p0 < p1; p0 += 4) {  // four entries' loads in flight
+    int ell[4], bf[4], cl[4], sl[4];
+    double it[4], g[4], b[4], bc[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) ell[u] = p0 + u < p1 ? __ldg(a.ebr + p0 + u) : -2;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (ell[u] < 0) continue;
+      it[u] = __ldg(a.itap + ell[u]);
+      g[u] = __ldg(a.g + ell[u]);
+      b[u] = __ldg(a.b + ell[u]);
+      bc[u] = __ldg(a.bch + ell[u]);
+      bf[u] = __ldg(a.br_f + ell[u]);
+      cl[u] = __ldg(a.col + p0 + u);
+      sl[u] = a.slot ? __ldg(a.slot + p0 + u) : 0;
     }
-    if (a.br_f[ell] == i) { dr += gs * it2; di += (bs + sh) * it2; }
-    else { dr += gs; di += bs + sh; }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int p = p0 + u;
+      if (ell[u] == -1) pd = p;
+      if (ell[u] < 0) continue;
+      const double it1 = it[u], it2 = it1 * it1, gs = g[u], bs = b[u], sh = 0.5 * bc[u];
+      const double vr = -gs * it1, vi = -bs * it1;
+      a.val64[p] = make_double2(vr, vi);
+      a.ent32[p] = make_int4(cl[u], __float_as_int(narrow(vr)), __float_as_int(narrow(vi)), 0);
+      if (a.slot) {
+        a.sell32[sl[u]] = make_float2(narrow(vr), narrow(vi));
+        a.sell64[sl[u]] = make_double2(vr, vi);
+      }
+      if (bf[u] == i) { dr += gs * it2; di += (bs + sh) * it2; }
+      else { dr += gs; di += bs + sh; }
+    }
   }
   if (pd >= 0) {
     a.val64[pd] = make_double2(dr, di);
@@ -1943,6 +1992,7 @@ template <class R> struct EdgeArgs {
   double* d_g;
   double* d_b;
   double* d_bch;
+  int add;  // 1: several case tiles add into zeroed outputs; 0: one tile stores
 };
 
 template <class R>
@@ -1974,12 +2024,95 @@ __global__ void __launch_bounds__(1024) k_edge_grad(EdgeArgs<R> a) {
       eb += __shfl_xor_sync(0xffffffffu, eb, off);
       ec += __shfl_xor_sync(0xffffffffu, ec, off);
     }
-    if (mp.kl == 0 && ell < a.M) {
+    if (mp.kl == 0 && ell < a.M && !a.add) {
+      if (a.d_g) a.d_g[ell] = widen(eg);
+      if (a.d_b) a.d_b[ell] = widen(eb);
+      if (a.d_bch) a.d_bch[ell] = widen(ec);
+    } else if (mp.kl == 0 && ell < a.M) {
       if (a.d_g) atomicAdd(a.d_g + ell, (double)eg);
       if (a.d_b) atomicAdd(a.d_b + ell, (double)eb);
       if (a.d_bch) atomicAdd(a.d_bch + ell, (double)ec);
     }
   }
+}
+
+// ---- inputs and outputs of the evaluation calls ------------------------------
+// One tiled transpose from the caller's case-major FP64 state (and, if given,
+// injections) to the working arrays: master pairs, V, injections in FP64 and in
+// working precision.
+template <class R> struct EvalInArgs {
+  int N, K, Kp;
+  const int32_t* iperm;
+  const double *va, *vm, *p, *q;
+  typename Prec<R>::MS* ms;
+  typename Prec<R>::C* V;
+  double *p64, *q64;
+  R *pw, *qw;
+};
+template <class R>
+__global__ void k_eval_in(EvalInArgs<R> a) {
+  using M = typename Prec<R>::M;
+  __shared__ double t0[32][33], t1[32][33];
+  const int u0 = blockIdx.x * 32, k0 = blockIdx.y * 32, tx = threadIdx.x;
+  for (int half = 0; half < (a.p ? 2 : 1); ++half) {
+    const double *s0 = half ? a.p : a.va, *s1 = half ? a.q : a.vm;
+    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+      const int k = k0 + r, u = u0 + tx;
+      const bool in = k < a.K && u < a.N;
+      t0[r][tx] = in ? __ldcs(s0 + (size_t)k * a.N + u) : 0.0;
+      t1[r][tx] = in ? __ldcs(s1 + (size_t)k * a.N + u) : (half ? 0.0 : 1.0);  // (a padded case: V = 1)
+    }
+    __syncthreads();
+    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+      const int u = u0 + r, k = k0 + tx;
+      if (u >= a.N || k >= a.Kp) continue;
+      const size_t e = (size_t)a.iperm[u] * a.Kp + k;
+      const double x = t0[tx][r], y = t1[tx][r];
+      if (half) {
+        if (k < a.K) {
+          a.p64[e] = x;
+          a.q64[e] = y;
+        }
+        a.pw[e] = to_work(x, R(0));
+        a.qw[e] = to_work(y, R(0));
+      } else {
+        const M th = mfrom<M>(x), vm = mfrom<M>(y);
+        a.ms[e] = ms_make(th, vm);
+        a.V[e] = volt(th, vm);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// One tiled transpose of two working-precision arrays (each element `stride`
+// values apart) to the caller's case-major FP64 outputs (either may be NULL).
+template <class R>
+__global__ void k_eval_out(const R* __restrict__ s0, const R* __restrict__ s1, size_t stride, double sign, int K, int N,
+                           int Kp, const int32_t* __restrict__ iperm, double* __restrict__ d0, double* __restrict__ d1) {
+  __shared__ R t0[32][33], t1[32][33];
+  const int u0 = blockIdx.x * 32, k0 = blockIdx.y * 32, tx = threadIdx.x;
+  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+    const int u = u0 + r, k = k0 + tx;
+    if (u < N && k < K) {
+      const size_t e = ((size_t)iperm[u] * Kp + k) * stride;
+      if (d0) t0[tx][r] = s0[e];
+      if (d1) t1[tx][r] = s1[e];
+    }
+  }
+  __syncthreads();
+  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+    const int k = k0 + r, u = u0 + tx;
+    if (u >= N || k >= K) continue;
+    if (d0) __stcs(d0 + (size_t)k * N + u, sign * widen(t0[r][tx]));
+    if (d1) __stcs(d1 + (size_t)k * N + u, sign * widen(t1[r][tx]));
+  }
+}
+
+// FP64 loss of the evaluation calls from the check's sums.
+static __global__ void k_eval_loss(const double* __restrict__ sum, double inv_m, int K, double* __restrict__ loss) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < K) loss[k] = sum[k] * inv_m;
 }
 
 }  // namespace dpf
