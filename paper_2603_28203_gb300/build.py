@@ -34,7 +34,7 @@ def build(verbose: bool = False, ptxas_info: bool = False) -> str:
     cuda = _cuda_home()
     nvcc = os.path.join(cuda, "bin", "nvcc")
     objs, cmds = [], []
-    for src in ("dpf_api.cu", "dpf_noalloc.cu", "dpf_nr.cu", "dpf_resident.cu", "dpf_dc_resident.cu", "dpf_eval.cu"):
+    for src in ("dpf_api.cu", "dpf_noalloc.cu", "dpf_nr.cu", "dpf_resident.cu", "dpf_dc_resident.cu", "dpf_eval.cu", "dpf_grid.cu"):
         obj = os.path.join(OUT_DIR, src.replace(".cu", ".o"))
         cu = [nvcc, *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
               "-I" + INCLUDE, *os.environ.get("DPF_NVCC_FLAGS", "").split(), "-c", os.path.join(CSRC, src),

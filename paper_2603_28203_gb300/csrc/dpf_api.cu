@@ -391,6 +391,10 @@ struct dpf_workspace {
   size_t cap_pent = 0;
   ResShape res;            // on-chip iterations (res.ok), their launch shape
   LossOrder res_lo;
+  GridShape grid;           // whole-GPU iterations (grid.ok)
+  float* grid_terms = nullptr;
+  unsigned* grid_sus = nullptr;
+  unsigned* grid_bar = nullptr;
   bool pid_ready = false;  // operating points staged by dpf_paramid_begin
   std::vector<std::pair<std::vector<long long>, std::vector<int>>> tune_cache;  // key -> (lanes, warps, rb, pairs)
   bool spec_per_case = false, has_outage = false;
@@ -417,7 +421,7 @@ static void ws_free_buffers(dpf_workspace* w) {
   dfree(w->lr); dfree(w->best); dfree(w->out_max); dfree(w->out_loss); dfree(w->loss64);
   dfree(w->yff64); dfree(w->yft64); dfree(w->ytt64); dfree(w->maxmis); dfree(w->outage_dev);
   dfree(w->b1t); dfree(w->b2t); dfree(w->cand); dfree(w->mx32);
-  dfree(w->dcs); dfree(w->dci);
+  dfree(w->dcs); dfree(w->dci); dfree(w->grid_terms); dfree(w->grid_sus);
   dfree(w->st_a); dfree(w->st_b); dfree(w->st_c);
   dfree(w->d_wlo); dfree(w->d_whi);
   dfree(w->pent);
@@ -462,7 +466,7 @@ static int ws_reserve(dpf_workspace* w, int Kp, size_t stage) {
     dfree(w->cool); dfree(w->lr); dfree(w->best); dfree(w->out_max); dfree(w->out_loss); dfree(w->loss64);
     dfree(w->yff64); dfree(w->yft64); dfree(w->ytt64); dfree(w->maxmis); dfree(w->outage_dev);
     dfree(w->b1t); dfree(w->b2t); dfree(w->cand); dfree(w->mx32);
-    dfree(w->dcs); dfree(w->dci);
+    dfree(w->dcs); dfree(w->dci); dfree(w->grid_terms); dfree(w->grid_sus);
     w->cap_elems = 0;
     w->cap_cases = 0;
     char** bufs16[] = {(char**)&w->V, (char**)&w->W, (char**)&w->G0, (char**)&w->V64, (char**)&w->sbuf,
@@ -485,6 +489,8 @@ static int ws_reserve(dpf_workspace* w, int Kp, size_t stage) {
     TRY(dalloc(&w->maxmis, Kp)); TRY(dalloc(&w->outage_dev, Kp));
     TRY(dalloc(&w->b1t, Kp)); TRY(dalloc(&w->b2t, Kp)); TRY(dalloc(&w->cand, Kp)); TRY(dalloc(&w->mx32, Kp));
     TRY(dalloc(&w->dcs, (size_t)9 * Kp)); TRY(dalloc(&w->dci, (size_t)2 * Kp + 1));
+    TRY(dalloc(&w->grid_terms, (size_t)4 * Kp)); TRY(dalloc(&w->grid_sus, (size_t)Kp + 2));
+    w->grid_bar = w->grid_sus + Kp;
     CK(cudaMemset(w->p64, 0, E * 8));
     CK(cudaMemset(w->q64, 0, E * 8));
     w->cap_elems = E;
@@ -516,8 +522,8 @@ extern "C" int dpf_workspace_create(const dpf_ybus* y, int32_t max_case, dpf_wor
   dpf_default_opts(&w->opts);
   int rc = DPF_OK;
   do {
-    if ((rc = dalloc(&w->n_active, 1))) break;
-    cudaError_t e = cudaMallocHost((void**)&w->h_n_active, sizeof(int32_t));
+    if ((rc = dalloc(&w->n_active, 2))) break;  // [1]: a grid barrier gave up
+    cudaError_t e = cudaMallocHost((void**)&w->h_n_active, 2 * sizeof(int32_t));
     if (e != cudaSuccess) { rc = fail(DPF_E_OOM, "cudaMallocHost: %s", cudaGetErrorString(e)); break; }
     e = cudaMallocHost((void**)&w->h_dc_nact, sizeof(int32_t));
     if (e != cudaSuccess) { rc = fail(DPF_E_OOM, "cudaMallocHost: %s", cudaGetErrorString(e)); break; }
@@ -854,6 +860,14 @@ static int launch_span(dpf_workspace* w, cudaStream_t s, int n, bool with_check)
     if (with_check) TRY(launch_check_any(w, s, false));
     return launch_resident(w, s, n);
   }
+  if (w->grid.ok && !w->profile) {
+    if (with_check) TRY(launch_check_any(w, s, false));
+    CK((cudaError_t)grid_launch(make_plan<float>(w).it, w->grid, w->res_lo, w->lanes, w->K, n,
+                                w->precision == DPF_FP32R, w->grid_terms, w->grid_sus, w->grid_bar, w->n_active + 1,
+                                s));
+    w->launches++;
+    return DPF_OK;
+  }
   for (int i = 0; i < n; ++i) TRY(launch_iteration_any(w, s, with_check && i == 0));
   return DPF_OK;
 }
@@ -1049,6 +1063,7 @@ static void choose_shape(dpf_workspace* w, const dpf_solve_opts* o, int K) {
 // plain form keep the streaming kernels.
 static void choose_resident(dpf_workspace* w, const dpf_solve_opts* o) {
   w->res = ResShape();
+  w->grid = GridShape();
   if (o->plain || o->stage_v || o->stage_y || w->precision == DPF_MIXED) return;
   int dev = 0, lim = 0;
   cudaGetDevice(&dev);
@@ -1061,6 +1076,7 @@ static void choose_resident(dpf_workspace* w, const dpf_solve_opts* o) {
   lo.tile = w->pair_fwd ? 64 : w->lanes;
   lo.nthr = w->warps * 32;
   w->res = res_shape(w->y, w->K, w->precision == DPF_FP64, w->precision == DPF_FP32R, lo, (size_t)lim);
+  if (!w->res.ok && w->precision != DPF_FP64) w->grid = grid_shape(w->y, w->K, lo, w->lanes, (size_t)lim);
 }
 
 // Device copies of the row-block windows (after choose_shape), and zeroed
@@ -1300,8 +1316,9 @@ static int init_state(dpf_workspace* w, const StateIn& in, cudaStream_t s) {
     }
   }
   TRY(case_init<R>(w, outage_dev, s));
-  CK(cudaMemcpyAsync(w->n_active, &w->K, 4, cudaMemcpyHostToDevice, s));
-  CK(cudaStreamSynchronize(s));  // &w->K is host memory that may change later
+  const int32_t count[2] = {w->K, 0};
+  CK(cudaMemcpyAsync(w->n_active, count, 8, cudaMemcpyHostToDevice, s));
+  CK(cudaStreamSynchronize(s));  // (host memory of this frame)
   return DPF_OK;
 }
 
@@ -1571,7 +1588,8 @@ extern "C" int dpf_solve_begin(const dpf_ybus* y, dpf_workspace* w, const dpf_ba
     CKLAUNCH();
     w->launches += (w->precision == DPF_MIXED) ? 2 : 1;
   }
-  if (w->direct) {  // padded entries of the direct view
+  if (w->grid.ok) CK(cudaMemsetAsync(w->grid_sus, 0, (size_t)w->cap_cases * sizeof(unsigned), s));
+  if (w->direct || w->grid.ok) {  // padded entries of the direct view
     const size_t np = (size_t)y->iprow_ptr[y->n];
     if (np > w->cap_pent) {
       dfree(w->pent);
@@ -1608,7 +1626,7 @@ extern "C" int dpf_solve_iterate(dpf_workspace* w, int32_t n_iter, void* stream)
   n_iter = std::min(n_iter, w->opts.max_iter - w->t_done);
   const int ce = w->opts.check_every;
   while (n_iter > 0) {
-    if (w->opts.use_graph && !w->profile && w->t_done % ce == 0 && n_iter >= ce) {
+    if (w->opts.use_graph && !w->profile && !w->grid.ok && w->t_done % ce == 0 && n_iter >= ce) {
       if (!w->gexec) TRY(build_graph(w));
       CK(cudaGraphLaunch(w->gexec, s));
       w->launches += w->graph_kernels;
@@ -1624,13 +1642,18 @@ extern "C" int dpf_solve_iterate(dpf_workspace* w, int32_t n_iter, void* stream)
   return DPF_OK;
 }
 
+// The error flag of the whole-GPU iterations, as last read with the count.
+static int barrier_error(const dpf_workspace* w) {
+  return w->h_n_active[1] ? fail(DPF_E_CUDA, "a grid barrier of the iterations gave up waiting") : DPF_OK;
+}
+
 extern "C" int dpf_active_count(dpf_workspace* w, int32_t* n_active, void* stream) {
   if (!w || !n_active) return fail(DPF_E_INVALID, "dpf_active_count: NULL argument");
   cudaStream_t s = (cudaStream_t)stream;
-  CK(cudaMemcpyAsync(w->h_n_active, w->n_active, 4, cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(w->h_n_active, w->n_active, 8, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   *n_active = *w->h_n_active;
-  return DPF_OK;
+  return barrier_error(w);
 }
 
 extern "C" int dpf_profile_enable(dpf_workspace* w, int32_t on) {
@@ -1824,13 +1847,17 @@ static int solve_batched(const dpf_ybus* y, dpf_workspace* w, const dpf_batch* b
       if (*w->h_n_active == 0) break;
     }
     if (!pending) {
-      cudaMemcpyAsync(w->h_n_active, w->n_active, 4, cudaMemcpyDeviceToHost, s);
+      cudaMemcpyAsync(w->h_n_active, w->n_active, 8, cudaMemcpyDeviceToHost, s);
       cudaEventRecord(ev, s);
       pending = true;
     }
   }
   if (pending) cudaEventSynchronize(ev);
   cudaEventDestroy(ev);
+  if (rc == DPF_OK && w->grid.ok) {
+    int32_t act;
+    rc = dpf_active_count(w, &act, s);
+  }
   if (rc != DPF_OK) return rc;
   return dpf_solve_end(w, b, s);
 }

@@ -39,6 +39,21 @@ template <class R>
 int res_launch(const dpf_ybus* y, const IterArgs<R>& a, const ResShape& sh, const LossOrder& lo, int K, int n_it,
                bool refined, bool pdl, void* stream);
 
+// Whole-GPU form of the FP32 iterations (dpf_grid.cu): one persistent launch
+// per test interval for larger grids whose batch fits the SMs together.
+struct GridShape {
+  bool ok = false;
+  int ctas = 0, warps = 0, workers = 0;
+  int gx = 0;   // case tiles that hold cases
+  int vb = 0;   // virtual blocks (case tile x row block) per CTA
+  size_t smem = 0;
+};
+GridShape grid_shape(const dpf_ybus* y, int K, const LossOrder& lo, int lanes, size_t smem_limit);
+// terms: 4 Kp floats; suspect: Kp words, zero between launches; bar: two words;
+// err: set to 1 if a barrier gave up.  Returns a cudaError_t.
+int grid_launch(const IterArgs<float>& a, const GridShape& g, const LossOrder& lo, int lanes, int K, int n_it,
+                bool refined, float* terms, unsigned* suspect, unsigned* bar, int32_t* err, void* stream);
+
 // On-chip form of the DC solve (dpf_dc_resident.cu): every case of the batch
 // to its tolerance in one launch.
 struct DcRes {

@@ -91,6 +91,23 @@ def test_on_chip_equals_streaming(n, K, precision):
     _same(_run(y, ws, K, opts, False, **kw), _run(y, ws, K, opts, True, **kw))
 
 
+# larger grids with about one element per thread of the GPU: fewer row blocks
+# than SMs (one case), one and two tiles, two-case tiles with a padded half,
+# lanes < 32, more row blocks than 64 (two-level loss sum), two rounds of tasks
+# per warp; the last is just above the range
+@pytest.mark.parametrize("n,K", [(2049, 1), (2500, 33), (2500, 65), (5000, 3), (9001, 17), (40000, 1), (40000, 4),
+                                 (160001, 1), (10000, 20)])
+@pytest.mark.parametrize("precision", ["fp32", "fp32r"])
+def test_whole_gpu_equals_streaming(n, K, precision):
+    g = _grid(n)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    opts = dpf.SolveOpts(precision=getattr(dpf, precision.upper()), max_iter=63, check_every=20, lr=3e-3, patience=3,
+                         cooldown=5, gate=1e-1)
+    kw = _inputs(g, K, n + K, specs=K > 4, outages=K != 5)
+    _same(_run(y, ws, K, opts, False, **kw), _run(y, ws, K, opts, True, **kw))
+
+
 @pytest.mark.parametrize("n,K", [(30, 1), (64, 40), (65, 3), (300, 150)])
 def test_on_chip_equals_streaming_fp64(n, K):
     g = _grid(n)
@@ -102,7 +119,7 @@ def test_on_chip_equals_streaming_fp64(n, K):
 
 
 @pytest.mark.parametrize("opt", [dpf.OPT_SGD, dpf.OPT_RMSPROP, dpf.OPT_ADAM])
-@pytest.mark.parametrize("n", [30, 300])
+@pytest.mark.parametrize("n", [30, 300, 3000])
 def test_on_chip_optimisers_and_step_schedule(opt, n):
     g = _grid(n)
     K = 6
@@ -115,7 +132,7 @@ def test_on_chip_optimisers_and_step_schedule(opt, n):
 
 
 @pytest.mark.parametrize("precision", ["fp32", "fp32r"])
-@pytest.mark.parametrize("n", [30, 300])
+@pytest.mark.parametrize("n", [30, 300, 3000])
 def test_on_chip_divergence(n, precision):
     """A case stops as diverged before the step its loss makes impossible: at
     once (NaN injections) or after some steps (a rate that overflows |V|);
