@@ -14,10 +14,12 @@ step is a relative change of about `lr`.
 """
 from __future__ import annotations
 
+import ctypes as C
+
 import torch
 
 from . import _abi
-from .dpf import Workspace, Ybus, dpf_adam_update, dpf_paramid_begin, dpf_paramid_step
+from .dpf import Workspace, Ybus, _check, _ptr, _stream, dpf_paramid_begin, lib
 
 
 def identify_branches(y: Ybus, ws: Workspace, va, vm, p, q, g0, b0, iters: int, lr: float = 3e-3,
@@ -29,13 +31,23 @@ def identify_branches(y: Ybus, ws: Workspace, va, vm, p, q, g0, b0, iters: int, 
     sg, sb = g0.abs(), b0.abs()
     hist = []
     dpf_paramid_begin(y, ws, va, vm, p, q, precision=precision, stream=stream)
-    bufs = {}
+    # The loop's buffers do not change, so its calls (dpf_paramid_step, then
+    # dpf_adam_update on g and on b) take arguments marshalled once: a step is
+    # some 20 us of kernels, less than marshalling three calls afresh.
+    L, h = lib(), _stream(stream)
+    dg, db = (torch.empty(y.n_branch, dtype=torch.float64, device=g0.device) for _ in range(2))
+    loss = torch.empty(int(va.shape[0]) if record_every else 0, dtype=torch.float64, device=g0.device)
+    ptr = lambda t: C.c_void_p(_ptr(t))  # noqa: E731
+    n, h = C.c_int32(int(g0.numel())), C.c_void_p(h)
+    step = (y.handle, ws.handle, ptr(g), ptr(b), ptr(dg), ptr(db), None)
+    adam = [(n, ptr(x), ptr(d), ptr(m), ptr(v), ptr(sc)) for x, d, m, v, sc in
+            ((g, dg, mg, vg, sg), (b, db, mb, vb, sb))]
+    rate = (C.c_double(lr), C.c_double(betas[0]), C.c_double(betas[1]), C.c_double(1e-8), h)
     for t in range(1, iters + 1):
-        want = ("d_g", "d_b", "loss") if (record_every and t % record_every == 0) else ("d_g", "d_b")
-        out = dpf_paramid_step(y, ws, g, b, want=want, out=bufs, stream=stream)
-        bufs.update(out)
-        if "loss" in out:
-            hist.append((t, float(out["loss"].sum().item())))
-        dpf_adam_update(g, out["d_g"], mg, vg, t, lr, betas[0], betas[1], lr_scale=sg, stream=stream)
-        dpf_adam_update(b, out["d_b"], mb, vb, t, lr, betas[0], betas[1], lr_scale=sb, stream=stream)
+        record = bool(record_every) and t % record_every == 0
+        _check(L.dpf_paramid_step(*step, ptr(loss) if record else None, h))
+        if record:
+            hist.append((t, float(loss.sum().item())))
+        for a in adam:
+            _check(L.dpf_adam_update(*a, t, *rate))
     return g, b, hist
