@@ -59,7 +59,7 @@ using namespace dpf;
 namespace {
 
 constexpr uint8_t NR_PQ = 0, NR_SLACK = 2;  // bus types (pv = 1)
-constexpr int NR_THREADS = 256;
+constexpr int NR_THREADS = 512;  // of k_nr_lu in FP32; half in FP64
 constexpr int NR_SMEM_THREADS = 1024;
 constexpr int NR_CHUNKS = 16;  // row chunks of the per-case reduction
 
@@ -797,7 +797,7 @@ static int nr_iterate_linear(dpf_nr* h, const NrArgs& a, bool smem, cudaStream_t
     return DPF_OK;
   }
   k_nr_assemble<T><<<grid_for((size_t)a.N * a.Kp), 256, 0, s>>>(a);
-  k_nr_lu<T><<<a.Kp / a.C, NR_THREADS, 0, s>>>(a);
+  k_nr_lu<T><<<a.Kp / a.C, sizeof(T) == 8 ? NR_THREADS / 2 : NR_THREADS, 0, s>>>(a);
   CKLAUNCH();
   h->launches += 2;
   return DPF_OK;
@@ -858,13 +858,15 @@ extern "C" int dpf_nr_solve(dpf_nr* h, const dpf_batch* b, const dpf_nr_opts* o,
   a.K = K;
   a.Kp = (K + 31) / 32 * 32;
   // cases per CTA: the C lanes of a slot share its schedule loads and read
-  // C consecutive blocks; few enough cases per CTA that every CTA of the
-  // batch is resident at once (each walks the whole tree: a second wave
-  // would double the time)
+  // C consecutive blocks (a 128-byte line: 8 in FP32, 4 in FP64); few enough cases per CTA
+  // that every CTA of the batch is resident at once (each walks the whole tree:
+  // a second wave would double the time).  ms for 2,379 cases of 2,000 buses
+  // by threads and C: 512, 8 12.9; 256, 4 13.5; 128, 2 14.6; 256, 8 15.0;
+  // 512, 4 15.7; 256, 2 16.4; 128, 4 16.5.
   const int C_fixed = o->lanes;
   auto lanes_for = [&](int n_active) {
     if (C_fixed) return C_fixed;
-    int C = 4;
+    int C = precision == DPF_FP64 ? 4 : 8;
     while (C > 1 && n_active / C < num_sms_nr()) C >>= 1;
     return C;
   };
