@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(GRID_WARPS * 32, 1) k_grid_resident(const Grid
           if (i == of) res_outage(a, x.k, 1, xi, __ldcg(a.V + (unsigned)ot * Kp + x.k), I);
           else if (i == ot) res_outage(a, x.k, 2, xi, __ldcg(a.V + (unsigned)of * Kp + x.k), I);
           float Q;
-          const float2 d = res_fwd<float, REF>(a, ty, xi, I, sp, vr, rf, w, Q, mx);
+          const float2 d = res_fwd<float, REF>(a, ty, xi, I, sp, vr, rf, w, Q, mx, last);
           __stcg(a.W + e, w);
           if (ty == BUS_PV) __stcg(a.qpv + e, Q);
           acc = fmaf(d.x, d.x, fmaf(d.y, d.y, acc));

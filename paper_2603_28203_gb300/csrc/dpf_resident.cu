@@ -56,7 +56,7 @@ struct LossGeo {
 // staged Y_bus.
 struct ResLayout {
   unsigned w, d, s, vr, rf, scr, sc, flag, team;  // offsets inside a team's block, its size
-  unsigned val, col, soff, total;             // after the teams
+  unsigned val, col, total;                   // after the teams
 };
 template <class R> struct ResArgs {
   using C = typename Prec<R>::C;
@@ -187,12 +187,10 @@ template <class R>
 __device__ __forceinline__ void res_stage(const ResArgs<R>& q, unsigned char* smem) {
   ValPair<R>* sval = reinterpret_cast<ValPair<R>*>(smem + q.L.val);
   uint32_t* scol = reinterpret_cast<uint32_t*>(smem + q.L.col);
-  int* ssoff = reinterpret_cast<int*>(smem + q.L.soff);
   for (int t = threadIdx.x; t < q.n_pair * 32; t += blockDim.x) {
     sval[t] = q.val[t];
     scol[t] = __ldg(q.col2 + t);
   }
-  for (int t = threadIdx.x; t <= q.n_slice; t += blockDim.x) ssoff[t] = __ldg(q.soff + t) * 32;
 }
 
 // One warp per case, RES_TEAMS cases per CTA.
@@ -211,7 +209,6 @@ __global__ void __launch_bounds__(32 * RES_TEAMS, sizeof(R) == 8 ? 3 : 5)
   R* scr = reinterpret_cast<R*>(tb + q.L.scr);
   const ValPair<R>* val = reinterpret_cast<const ValPair<R>*>(smem + q.L.val) + lane;
   const uint32_t* col = reinterpret_cast<const uint32_t*>(smem + q.L.col) + lane;
-  const int* soff = reinterpret_cast<const int*>(smem + q.L.soff);
   const int k = blockIdx.x * RES_TEAMS + team;
   res_stage(q, smem);
   pdl_wait();
@@ -220,7 +217,7 @@ __global__ void __launch_bounds__(32 * RES_TEAMS, sizeof(R) == 8 ? 3 : 5)
   if (k >= q.K || !a.active[k]) return;  // (no CTA barrier follows)
   const size_t Kp = (size_t)a.Kp;
 
-  int row[RPT], ty[RPT], end[RPT];
+  int row[RPT], ty[RPT], end[RPT], sl[RPT];
   ResRow<R> rw[RPT];
   C sp[RPT];
   float2 vr[RPT];
@@ -237,6 +234,11 @@ __global__ void __launch_bounds__(32 * RES_TEAMS, sizeof(R) == 8 ? 3 : 5)
     row[s] = p < N ? __ldg(q.rord + p) : -1;
     ty[s] = BUS_SLACK;
     end[s] = 0;
+    sl[s] = 0;
+    if (s < q.n_slice) {
+      const int p0 = __ldg(q.soff + s);
+      sl[s] = p0 * 32 | (__ldg(q.soff + s + 1) - p0) << 20;
+    }
     C x = mkc(R(0), R(0));
     sp[s] = x;
     rw[s] = ResRow<R>{};
@@ -264,21 +266,21 @@ __global__ void __launch_bounds__(32 * RES_TEAMS, sizeof(R) == 8 ? 3 : 5)
   for (int it = 0; it < q.n_it; ++it) {
     sc.terms(a.sc, lane);
     float mx = 0.f;
+    const bool track = it == q.n_it - 1 && a.sc.mx32;
 #pragma unroll
     for (int s = 0; s < RPT; ++s) {
       const int p = s * 32 + lane;
-      if (s >= q.n_slice) break;
-      C I = sell_row<R>(val, col, soff[s], soff[s + 1], tb);
+      C I = sell_row<R>(val, col, sl[s], tb);
       if (row[s] < 0) continue;
       const C x = X[p];
       if (end[s]) res_outage(a, k, end[s], x, X[end[s] & 1 ? pt : pf], I);
       C w;
       R Q;
-      D[row[s]] = res_fwd<R, REF>(a, ty[s], x, I, sp[s], vr[s], rf[s], w, Q, mx);
+      D[row[s]] = res_fwd<R, REF>(a, ty[s], x, I, sp[s], vr[s], rf[s], w, Q, mx, track);
       if (ty[s] == BUS_PV) sp[s].y = Q;
       W[p] = w;
     }
-    if (it == q.n_it - 1 && a.sc.mx32) {
+    if (track) {
       const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
       if (lane == 0) a.sc.cand[k] = (a.sc.gate <= 0.0 || (double)__uint_as_float(m) <= a.sc.gate) ? 1 : 0;
     }
@@ -291,8 +293,7 @@ __global__ void __launch_bounds__(32 * RES_TEAMS, sizeof(R) == 8 ? 3 : 5)
 #pragma unroll
     for (int s = 0; s < RPT; ++s) {
       const int p = s * 32 + lane;
-      if (s >= q.n_slice) break;
-      C z = sell_row<R>(val, col, soff[s], soff[s + 1], wb);
+      C z = sell_row<R>(val, col, sl[s], wb);
       if (ty[s] == BUS_SLACK) continue;
       const C w = W[p];
       if (end[s]) res_outage(a, k, end[s], w, W[end[s] & 1 ? pt : pf], z);
@@ -341,7 +342,6 @@ __global__ void __launch_bounds__(res_threads<R>(), 1) k_resident_cta(const ResA
   R* terms = reinterpret_cast<R*>(smem + q.L.flag + 16);    // step, isb of the coming update
   const ValPair<R>* val = reinterpret_cast<const ValPair<R>*>(smem + q.L.val) + lane;
   const uint32_t* col = reinterpret_cast<const uint32_t*>(smem + q.L.col) + lane;
-  const int* soff = reinterpret_cast<const int*>(smem + q.L.soff);
   ResSched<R>* scs = reinterpret_cast<ResSched<R>*>(smem + q.L.sc) + lane;
   const int k = blockIdx.x;
   res_stage(q, smem);
@@ -356,6 +356,7 @@ __global__ void __launch_bounds__(res_threads<R>(), 1) k_resident_cta(const ResA
   bool diverged = false;
   for (;;) {
     int info[RPT];  // internal row, bus type << 16, outage end << 20; -1: no row
+    int sl[RPT];    // entry pairs of the row's slice: first * 32, count << 20
     ResRow<R> rw[RPT];
     int ends = 0;   // positions of the outaged branch's ends: from-bus, to-bus << 16
     if (compute) {
@@ -369,6 +370,11 @@ __global__ void __launch_bounds__(res_threads<R>(), 1) k_resident_cta(const ResA
       for (int s = 0; s < RPT; ++s) {
         const int p = s * T + tid, i = p < N ? __ldg(q.rord + p) : -1;
         info[s] = -1;
+        sl[s] = 0;
+        if ((p >> 5) < q.n_slice) {
+          const int p0 = __ldg(q.soff + (p >> 5));
+          sl[s] = p0 * 32 | (__ldg(q.soff + (p >> 5) + 1) - p0) << 20;
+        }
         C x = mkc(R(0), R(0));
         if (i >= 0) {
           const size_t e = (size_t)i * Kp + k, si = a.spec_per_case ? e : (size_t)i;
@@ -418,11 +424,10 @@ __global__ void __launch_bounds__(res_threads<R>(), 1) k_resident_cta(const ResA
       if (it == n) break;
       if (compute) {  // forward: I = Y V, mismatch, w
         float mx = 0.f;
+        const bool track = it == n - 1 && a.mx32;
 #pragma unroll
         for (int s = 0; s < RPT; ++s) {
-          const int sl = (s * T + tid) >> 5;  // (the same for the whole warp)
-          if (sl >= q.n_slice) break;
-          C I = sell_row<R>(val, col, soff[sl], soff[sl + 1], smem);
+          C I = sell_row<R>(val, col, sl[s], smem);  // (no entries past the last slice)
           if (info[s] < 0) continue;
           const C x = X[s * T];
           const int ty = (info[s] >> 16) & 15;
@@ -438,7 +443,7 @@ __global__ void __launch_bounds__(res_threads<R>(), 1) k_resident_cta(const ResA
           C w, sp = mkc(R(0), R(0));
           if constexpr (!REF) sp = S[s * T];
           R Q;
-          D[info[s] & 0xffff] = res_fwd<R, REF>(a, ty, x, I, sp, vr, rf, w, Q, mx);
+          D[info[s] & 0xffff] = res_fwd<R, REF>(a, ty, x, I, sp, vr, rf, w, Q, mx, track);
           if (ty == BUS_PV) S[s * T].y = Q;
           W[s * T] = w;
         }
@@ -454,9 +459,7 @@ __global__ void __launch_bounds__(res_threads<R>(), 1) k_resident_cta(const ResA
         const R step = terms[0], isb = terms[1];
 #pragma unroll
         for (int s = 0; s < RPT; ++s) {
-          const int sl = (s * T + tid) >> 5;
-          if (sl >= q.n_slice) break;
-          C z = sell_row<R>(val, col, soff[sl], soff[sl + 1], smem + WOFF);
+          C z = sell_row<R>(val, col, sl[s], smem + WOFF);
           const int ty = (info[s] >> 16) & 15;
           if (info[s] < 0 || ty == BUS_SLACK) continue;
           const C w = W[s * T];
@@ -537,8 +540,7 @@ static ResLayout res_layout(const dpf_ybus* y, const ResShape& sh, bool refined,
   L.team = L.flag + 32u;
   L.val = L.team * (sh.warp ? RES_TEAMS : 1);
   L.col = L.val + pairs * 64u * cs;
-  L.soff = L.col + pairs * 32u * 4u;
-  L.total = L.soff + (((unsigned)(y->dev.res_slices + 1) * 4u + 15u) & ~15u);
+  L.total = L.col + pairs * 32u * 4u;
   return L;
 }
 

@@ -155,7 +155,7 @@ __device__ __forceinline__ typename Prec<R>::C res_adj(const IterArgs<R>& a, int
 template <class R, bool REF>
 __device__ __forceinline__ typename Prec<R>::C res_fwd(const IterArgs<R>& a, int ty, typename Prec<R>::C x,
                                                        typename Prec<R>::C I, typename Prec<R>::C sp, float2 vr,
-                                                       float4 rf, typename Prec<R>::C& w, R& Q, float& mx) {
+                                                       float4 rf, typename Prec<R>::C& w, R& Q, float& mx, bool track) {
   using C = typename Prec<R>::C;
   C v;
   R dP, dQ;
@@ -173,8 +173,10 @@ __device__ __forceinline__ typename Prec<R>::C res_fwd(const IterArgs<R>& a, int
   }
   const R ca = a.inv_m2 * dP, cb = a.inv_m2 * dQ;
   w = w_of(ca, cb, v);
-  const float am = fmaxf(fabsf((float)dP), fabsf((float)dQ));
-  mx = (am != am) ? __int_as_float(0x7f800000) : fmaxf(mx, am);
+  if (track) {  // max |f| (a NaN counts as infinity): only the last iteration before a test needs it
+    const float am = fmaxf(fabsf((float)dP), fabsf((float)dQ));
+    mx = (am != am) ? __int_as_float(0x7f800000) : fmaxf(mx, am);
+  }
   return mkc(dP, dQ);
 }
 

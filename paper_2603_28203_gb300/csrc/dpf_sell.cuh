@@ -11,16 +11,21 @@ template <class R> struct __align__(16) ValPair { typename Prec<R>::C a, b; };
 
 // sum_e val[e] x[col[e]] over a row's entry pairs: even entries into a0, odd
 // into a1, as row_spmv does (pads: weight 0 on the row itself).
+// slice: the first pair's index | the number of pairs << 20; val and col2
+// point at this lane's entries.
 template <class R>
 __device__ __forceinline__ typename Prec<R>::C sell_row(const ValPair<R>* __restrict__ val,
-                                                        const uint32_t* __restrict__ col2, int p0, int p1,
+                                                        const uint32_t* __restrict__ col2, int slice,
                                                         const unsigned char* __restrict__ X) {
   using C = typename Prec<R>::C;
   constexpr unsigned sc = sizeof(C) / 8;
   C a0 = mkc(R(0), R(0)), a1 = a0;
-  for (int p = p0; p < p1; p += 32) {
-    const uint32_t cc = col2[p];
-    const ValPair<R> y = val[p];
+  val += slice & 0xfffff;
+  col2 += slice & 0xfffff;
+#pragma unroll 2
+  for (int n = slice >> 20; n > 0; --n, val += 32, col2 += 32) {
+    const uint32_t cc = *col2;
+    const ValPair<R> y = *val;
     const C x0 = *reinterpret_cast<const C*>(X + (cc & 0xffffu) * sc);
     const C x1 = *reinterpret_cast<const C*>(X + (cc >> 16) * sc);
     cfma(a0, y.a, x0);
