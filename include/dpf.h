@@ -272,6 +272,12 @@ int dpf_solve_batch(const dpf_ybus* y, dpf_workspace* ws, const dpf_batch* b,
 int dpf_solve_begin(const dpf_ybus* y, dpf_workspace* ws, const dpf_batch* b,
                     const dpf_solve_opts* o, void* stream);
 int dpf_solve_iterate(dpf_workspace* ws, int32_t n_iter, void* stream);
+/* Grids of up to 2,048 buses iterate on chip (a case's state stays in one SM
+ * for a whole check interval), a few cases of a larger grid in one kernel over
+ * the whole GPU, unless plain, stage_v or stage_y is set or the precision is
+ * DPF_MIXED; FP64 only up to 64 buses, or 320 buses and 300 cases.  Results
+ * are those of the two-pass kernels (FP32, FP32R: to the bit; lanes, warps,
+ * row_blocks and pair_cases then only set the order of the loss sum). */
 int dpf_solve_end(dpf_workspace* ws, const dpf_batch* b, void* stream);
 /* Autotuner.  Times candidate launch shapes of the solve loop on this batch
  * -- cases per row group (`lanes`, i.e. rows per warp = 32/lanes), warps per
@@ -282,7 +288,8 @@ int dpf_solve_end(dpf_workspace* ws, const dpf_batch* b, void* stream);
  * inputs are read (as in dpf_solve_begin) but no output is written; a later
  * dpf_solve_begin starts from scratch.  Results are cached in the workspace
  * per (n_case, precision, grid, outage/injection layout).  Synchronises
- * `stream`. */
+ * `stream`.  Returns at once, options unchanged, for batches that iterate on
+ * chip (see dpf_solve_iterate): the two passes' launch shape isn't used. */
 int dpf_autotune(const dpf_ybus* y, dpf_workspace* ws, const dpf_batch* b, dpf_solve_opts* o,
                  int32_t iters, void* stream);
 
@@ -294,7 +301,8 @@ int dpf_iterations_done(const dpf_workspace* ws, int32_t* n_iter);
 /* ---- measurement ----------------------------------------------------------
  * dpf_profile_enable(ws, 1): from now on dpf_solve_iterate launches without a
  * CUDA graph and brackets every forward (k_fwd) and adjoint (k_adj) launch
- * with CUDA events on the caller's stream; 0 switches back to graph replay.
+ * with CUDA events on the caller's stream (the two-pass kernels, also where a
+ * solve would run on chip); 0 switches back to graph replay.
  * dpf_kernel_times: summed durations (ms) and launch counts of the
  * bracketed launches since the last enable (synchronises `stream`).
  * dpf_kernel_launches: number of kernels the workspace has enqueued since it
@@ -449,7 +457,8 @@ typedef struct {
   int32_t max_iter;          /* Newton steps per case                           */
   int32_t flat_start;        /* 1: ignore va/vm inputs, start flat              */
   int32_t lanes;             /* cases per CTA of the factor and solve kernels
-                                (power of 2 up to 32; 0 = auto)               */
+                                (power of 2 up to 32; 0 = auto, or one case
+                                per CTA in shared memory where few iterate)   */
   int32_t fallback;          /* 1 (with flat_start = 0): a case Newton does not
                                 converge keeps the start passed in va/vm and
                                 reports the start's max |f| and loss (its

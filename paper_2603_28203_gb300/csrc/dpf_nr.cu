@@ -16,6 +16,8 @@
 //                  CTA per tile of cases, which syncs only its own threads:
 //                  the cases are independent, so no CTA waits for another
 //   k_nr_update    theta += dx_theta (pv, pq), |V| += dx_|V| (pq)
+// or, where few cases iterate and a case's factor fits in shared memory,
+// k_nr_lu_smem in the place of the last three.
 // The factor and the triangular solves run in the factor precision (FP64, or
 // FP32: GB300 issues FP32 FMA at many times its FP64 rate, and a Newton step
 // solved to FP32 accuracy still converges, linearly at a rate of about
@@ -60,7 +62,7 @@ namespace {
 
 constexpr uint8_t NR_PQ = 0, NR_SLACK = 2;  // bus types (pv = 1)
 constexpr int NR_THREADS = 512;  // of k_nr_lu in FP32; half in FP64
-constexpr int NR_SMEM_THREADS = 1024;
+constexpr int NR_SMEM_THREADS = 512;
 constexpr int NR_CHUNKS = 16;  // row chunks of the per-case reduction
 
 // 2x2 block: rows (P, Q), columns (theta, |V|), row-major.
@@ -143,6 +145,11 @@ struct NrArgs {
   const int32_t* rlvl_ptr;
   const int4* rows;
   int64_t npos;
+  const uint4* sstream;  // schedule of the shared-memory form (k_nr_lu_smem)
+  const int2* schunk;
+  const uint4* sent;
+  const uint4* sdiag;
+  int n_ent, n_chunk, chunk_units, ring_bytes;
   // state [N][Kp]
   double* th;
   double* vm;
@@ -277,36 +284,44 @@ __global__ void k_nr_eval(NrArgs a) {
 
 // Per case and chunk of rows (32 cases x 8 row groups per CTA, fixed
 // summation order): partial max |f| (NaN if any entry is NaN) and partial
-// ||f||^2 from the right-hand side -f.
+// ||f||^2 from the right-hand side -f.  The maximum is taken on the bits of
+// |f|, which order as the values do and put NaN above infinity: an FP64
+// comparison holds the FP64 pipe as long as an FMA.
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffULL;
+}
+__device__ __forceinline__ double max_of_bits(unsigned long long m) {
+  return __longlong_as_double(m > 0x7ff0000000000000ULL ? 0x7ff8000000000000LL : (long long)m);
+}
 __global__ void __launch_bounds__(256) k_nr_partial(NrArgs a) {
-  __shared__ double smax[8][32], ssum[8][32];
+  __shared__ unsigned long long smax[8][32];
+  __shared__ double ssum[8][32];
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int k = blockIdx.x * 32 + lane;
   const bool on = k < a.K && a.active[k];
   const int rpc = (a.N + NR_CHUNKS - 1) / NR_CHUNKS;
   const int r0 = blockIdx.y * rpc, r1 = min(a.N, r0 + rpc);
-  double mx = 0.0, sm = 0.0;
-  bool nan = false;
-  if (on)
+  unsigned long long mx = 0;
+  double sm = 0.0;
+  if (on) {
+#pragma unroll 4
     for (int r = r0 + g; r < r1; r += 8) {
       const double2 x = a.X[(size_t)r * a.Kp + k];
-      nan = nan || !(x.x == x.x) || !(x.y == x.y);
-      mx = fmax(mx, fmax(fabs(x.x), fabs(x.y)));
+      mx = max(mx, max(abs_bits(x.x), abs_bits(x.y)));
       sm = fma(x.x, x.x, fma(x.y, x.y, sm));
     }
-  smax[g][lane] = nan ? __longlong_as_double(0x7ff8000000000000LL) : mx;
+  }
+  smax[g][lane] = mx;
   ssum[g][lane] = sm;
   __syncthreads();
   if (g != 0 || !on) return;
-  mx = 0.0;
+  mx = 0;
   sm = 0.0;
   for (int q = 0; q < 8; ++q) {
-    const double m = smax[q][lane];
-    nan = nan || !(m == m);
-    mx = fmax(mx, m);
+    mx = max(mx, smax[q][lane]);
     sm += ssum[q][lane];
   }
-  a.pmax[(size_t)blockIdx.y * a.Kp + k] = nan ? __longlong_as_double(0x7ff8000000000000LL) : mx;
+  a.pmax[(size_t)blockIdx.y * a.Kp + k] = max_of_bits(mx);
   a.psum[(size_t)blockIdx.y * a.Kp + k] = sm;
 }
 
@@ -372,6 +387,44 @@ __device__ __forceinline__ Cx<T> mul(Cx<T> a, Cx<T> b) {
   return Cx<T>{fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x)};
 }
 
+// The block of bus pair (i, j) of case k with Y_bus value y: vi = V_i,
+// uj = e^{j theta_j}, vmj = |V|_j, ii = I_i (read where i == j), bus types.
+template <class T>
+__device__ __forceinline__ Blk<T> jac_block(const NrArgs& a, int i, int j, double2 y, int k, int of, int ot, Cx<T> vi,
+                                            Cx<T> uj, T vmj, Cx<T> ii, int ti, int tj) {
+  if (of >= 0) {
+    if (i == of && j == of) y = csub(y, a.yff[k]);
+    else if (i == ot && j == ot) y = csub(y, a.ytt[k]);
+    else if ((i == of && j == ot) || (i == ot && j == of)) y = csub(y, a.yft[k]);
+  }
+  const Cx<T> w = mulc(vi, mul(cx<T>(y), uj));
+  T ba, bb, bc, bd;
+  if (i != j) {
+    ba = vmj * w.y;
+    bc = -vmj * w.x;
+    bb = w.x;
+    bd = w.y;
+  } else {
+    const Cx<T> si = mulc(vi, ii);   // S_i
+    const Cx<T> sdi = mulc(uj, ii);  // S_i / |V|_i
+    ba = fma(vmj, w.y, -si.y);
+    bc = fma(-vmj, w.x, si.x);
+    bb = sdi.x + w.x;
+    bd = sdi.y + w.y;
+  }
+  const bool rp = ti != NR_SLACK, rq = ti == NR_PQ, ct = tj != NR_SLACK, cv = tj == NR_PQ;
+  Blk<T> b;
+  b.a = (rp && ct) ? ba : T(0);
+  b.b = (rp && cv) ? bb : T(0);
+  b.c = (rq && ct) ? bc : T(0);
+  b.d = (rq && cv) ? bd : T(0);
+  if (i == j) {
+    if (!rp) b.a = T(1);
+    if (!rq) b.d = T(1);
+  }
+  return b;
+}
+
 // One block row of case k: its positions' blocks to dst[q * stride].
 template <class T>
 __device__ __forceinline__ void assemble_row(const NrArgs& a, int r, int k, Blk<T>* __restrict__ dst, size_t stride) {
@@ -379,50 +432,16 @@ __device__ __forceinline__ void assemble_row(const NrArgs& a, int r, int k, Blk<
   const double2* __restrict__ U = a.U;
   const double* __restrict__ VM = a.vm;
   const int i = __ldg(a.order + r);
-  const size_t ei = (size_t)i * Kp + k;
-  const Cx<T> vi = cx<T>(a.V[ei]), ii = cx<T>(a.I[ei]);
-  const Cx<T> si = mulc(vi, ii);             // S_i
-  const Cx<T> sdi = mulc(cx<T>(U[ei]), ii);  // S_i / |V|_i
-  const uint8_t ti = __ldg(a.type + i);
-  const bool rp = ti != NR_SLACK, rq = ti == NR_PQ;
-  const int of = a.of[k], ot = a.ot[k];
+  const Cx<T> vi = cx<T>(a.V[(size_t)i * Kp + k]), ii = cx<T>(a.I[(size_t)i * Kp + k]);
+  const int of = a.of[k], ot = a.ot[k], ti = __ldg(a.type + i);
   const int q1 = __ldg(a.frp + r + 1);
   for (int q = __ldg(a.frp + r); q < q1; ++q) {
-    const int j = __ldg(a.order + __ldg(a.fcol + q));
     const int yp = __ldg(a.ymap + q);
     Blk<T> b{T(0), T(0), T(0), T(0)};
     if (yp >= 0) {
-      double2 y = __ldg(a.yval + yp);
-      if (of >= 0) {
-        if (i == of && j == of) y = csub(y, a.yff[k]);
-        else if (i == ot && j == ot) y = csub(y, a.ytt[k]);
-        else if ((i == of && j == ot) || (i == ot && j == of)) y = csub(y, a.yft[k]);
-      }
+      const int j = __ldg(a.order + __ldg(a.fcol + q));
       const size_t ej = (size_t)j * Kp + k;
-      const Cx<T> w = mulc(vi, mul(cx<T>(y), cx<T>(U[ej])));
-      const T vmj = (T)VM[ej];
-      T ba, bb, bc, bd;
-      if (i != j) {
-        ba = vmj * w.y;
-        bc = -vmj * w.x;
-        bb = w.x;
-        bd = w.y;
-      } else {
-        ba = fma(vmj, w.y, -si.y);
-        bc = fma(-vmj, w.x, si.x);
-        bb = sdi.x + w.x;
-        bd = sdi.y + w.y;
-      }
-      const uint8_t tj = __ldg(a.type + j);
-      const bool ct = tj != NR_SLACK, cv = tj == NR_PQ;
-      b.a = (rp && ct) ? ba : T(0);
-      b.b = (rp && cv) ? bb : T(0);
-      b.c = (rq && ct) ? bc : T(0);
-      b.d = (rq && cv) ? bd : T(0);
-      if (i == j) {
-        if (!rp) b.a = T(1);
-        if (!rq) b.d = T(1);
-      }
+      b = jac_block<T>(a, i, j, __ldg(a.yval + yp), k, of, ot, vi, cx<T>(U[ej]), (T)VM[ej], ii, ti, __ldg(a.type + j));
     }
     stb(dst + (size_t)q * stride, b);
   }
@@ -571,31 +590,282 @@ __global__ void __launch_bounds__(NR_THREADS) k_nr_lu(NrArgs a) {
             a.bad + k);
 }
 
-// Shared-memory form, for grids whose factor of one case fits: one CTA per
-// case assembles its Jacobian straight into shared memory (the factor never
-// goes to HBM), factorises and solves there, and writes dx back.
-template <class T>
-__global__ void __launch_bounds__(NR_SMEM_THREADS) k_nr_lu_smem(NrArgs a) {
-  extern __shared__ __align__(16) unsigned char nr_smem[];
-  const int k = blockIdx.x;
-  if (!a.active[k]) return;  // the same for the whole CTA
-  Blk<T>* Fs = reinterpret_cast<Blk<T>*>(nr_smem);
-  Blk<T>* Ds = Fs + a.npos;
-  Cx<T>* Xs = reinterpret_cast<Cx<T>*>(Ds + a.N);
-  const size_t Kp = a.Kp;
-  for (int r = threadIdx.x; r < a.N; r += blockDim.x) {
-    Xs[r] = ldx<T>(a.X + (size_t)r * Kp + k);
-    assemble_row(a, r, k, Fs, 1);
-  }
-  __syncthreads();
-  lu_levels(a, Fs, 1, Ds, 1, Xs, 1, (int)threadIdx.x, (int)blockDim.x, true, a.bad + k);
-  for (int r = threadIdx.x; r < a.N; r += blockDim.x) stx(a.X + (size_t)r * Kp + k, Xs[r]);
+// Schedule of the shared-memory form: one stream of chunks, in 16-byte units.
+// A chunk is a set of targets of one level, one per thread at most: first a
+// record per target, then their lists in groups of 4 entries, filled up with
+// the zero block (position npos) and the zero solution entry (row N), which
+// change no bit of a sum.  Positions and rows are 16-bit fields (what fits in
+// shared memory has fewer).
+//   record {pos | x2 << 16, offset of its list in the chunk, groups, kind}
+//   NR_U, NR_DIAG, NR_L: updates {L(i,k) | U(k,j) << 16} of position pos; an L
+//     target is multiplied by its pivot's inverse at x2 after a barrier
+//   NR_FWD: row x2's forward substitution {L position | column << 16}
+//   NR_BACK: row x2's back substitution {U position | column << 16}, its
+//     inverse diagonal at pos
+//   chunk {first unit, targets | units to stage << 10, has L targets: bit 31};
+//     no units: larger than a stage, read in place (a pivot with long lists)
+// Block and vector targets don't share a warp.  A U target without updates has
+// no record.  The pivots of a chunk are whole; one larger than a stage is
+// split with its diagonal first.
+//   entry {position, i | j << 16, types, Y_bus entry}: blocks off the diagonal
+//   by Y_bus entry, diag {position, Y_bus entry, type} by bus
+enum { NR_FWD = 3, NR_BACK = 4, NR_NONE = 5 };
+constexpr int NR_STAGES = 4;  // chunks in shared memory: this one, the next ones on their way
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Shared memory the shared-memory form needs for one case.
 template <class T>
-size_t lu_smem_bytes(int64_t npos, int n) {
-  return (size_t)(npos + n) * sizeof(Blk<T>) + (size_t)n * sizeof(Cx<T>);
+__device__ __forceinline__ void upd_group(Blk<T>& acc, const Blk<T>* F, uint4 g) {
+  const Blk<T> l0 = ldb(F + (g.x & 0xffffu)), u0 = ldb(F + (g.x >> 16));
+  const Blk<T> l1 = ldb(F + (g.y & 0xffffu)), u1 = ldb(F + (g.y >> 16));
+  const Blk<T> l2 = ldb(F + (g.z & 0xffffu)), u2 = ldb(F + (g.z >> 16));
+  const Blk<T> l3 = ldb(F + (g.w & 0xffffu)), u3 = ldb(F + (g.w >> 16));
+  msub(acc, l0, u0);
+  msub(acc, l1, u1);
+  msub(acc, l2, u2);
+  msub(acc, l3, u3);
+}
+template <class T>
+__device__ __forceinline__ void sub_x(Cx<T>& y, const Blk<T>& m, const Cx<T>& x) {
+  y.x = fma(-m.a, x.x, fma(-m.b, x.y, y.x));
+  y.y = fma(-m.c, x.x, fma(-m.d, x.y, y.y));
+}
+template <class T>
+__device__ __forceinline__ void sub_group(Cx<T>& y, const Blk<T>* F, const Cx<T>* X, uint4 g) {
+  const Blk<T> m0 = ldb(F + (g.x & 0xffffu)), m1 = ldb(F + (g.y & 0xffffu));
+  const Blk<T> m2 = ldb(F + (g.z & 0xffffu)), m3 = ldb(F + (g.w & 0xffffu));
+  const Cx<T> x0 = X[g.x >> 16], x1 = X[g.y >> 16], x2 = X[g.z >> 16], x3 = X[g.w >> 16];
+  sub_x(y, m0, x0);
+  sub_x(y, m1, x1);
+  sub_x(y, m2, x2);
+  sub_x(y, m3, x3);
+}
+
+// One target (see the schedule above); true: `acc` is an L target's, to be
+// multiplied by the inverse at position `x2`.
+template <class T>
+__device__ __forceinline__ bool smem_target(const uint4* __restrict__ p, uint4 r, uint4 g, Blk<T>* F, Cx<T>* X,
+                                            Blk<T>& acc, int& pos, int& x2, int* bad) {
+  const int n = (int)r.z, kind = (int)r.w;
+  pos = r.x & 0xffffu;
+  x2 = r.x >> 16;
+  if (kind <= NR_L) {
+    acc = ldb(F + pos);
+    for (int i = 0; i < n; ++i) {
+      const uint4 c = g;
+      if (i + 1 < n) g = p[i + 1];
+      upd_group(acc, F, c);
+    }
+    if (kind == NR_L) return true;
+    if (kind == NR_DIAG) {
+      Blk<T> di;
+      if (!inv2(acc, di)) *bad = 1;
+      acc = di;
+    }
+    stb(F + pos, acc);
+  } else {
+    Cx<T> y = X[x2];
+    for (int i = 0; i < n; ++i) {
+      const uint4 c = g;
+      if (i + 1 < n) g = p[i + 1];
+      sub_group(y, F, X, c);
+    }
+    if (kind == NR_BACK) {
+      const Blk<T> d = ldb(F + pos);
+      y = Cx<T>{fma(d.a, y.x, d.b * y.y), fma(d.c, y.x, d.d * y.y)};
+    }
+    X[x2] = y;
+  }
+  return false;
+}
+
+// Shared-memory form, for grids whose factor of one case fits: one CTA per
+// case assembles its Jacobian straight into shared memory (the factor never
+// goes to HBM), factorises and solves there by the levels of lu_levels (same
+// sums in the same order: same bits), and updates theta and |V|.
+//
+// What bounds it is latency: a chain of 143 chunks for a 2,000-bus grid, most
+// of the upper ones a warp's worth of targets, 1,440 cycles each (a target's
+// loads from shared memory, the pivot's inverse, two barriers).  So the
+// schedule arrives by cp.async some chunks ahead and never costs a trip to
+// L2; a pivot's diagonal is updated and inverted once, not in each of its L
+// targets; block and vector targets sit in different warps and don't take
+// turns.  One case of 2,000 buses: 390 us with the schedule read from L2 by
+// each thread and the diagonal updated per L target, 135 us so (assembly 29).
+// 384 threads take 2% longer, 256 8%, 768 6%; 8 stages of 256 units 11%.
+template <class T>
+__global__ void __launch_bounds__(NR_SMEM_THREADS, 1) k_nr_lu_smem(NrArgs a) {
+  extern __shared__ __align__(16) unsigned char nr_smem[];
+  __shared__ int s_bad;
+  const int k = blockIdx.x, tid = threadIdx.x, S = blockDim.x, N = a.N, C = a.n_chunk;
+  if (!a.active[k]) return;  // the same for the whole CTA
+  const int npos = (int)a.npos;
+  Blk<T>* F = reinterpret_cast<Blk<T>*>(nr_smem);
+  unsigned char* ring = reinterpret_cast<unsigned char*>(F + npos + 1);
+  Cx<T>* X = reinterpret_cast<Cx<T>*>(ring + a.ring_bytes);
+  int2* chunk = reinterpret_cast<int2*>(X + N + 1);
+  const size_t Kp = a.Kp;
+
+  // V in the place of X, e^{j theta} and |V| in that of the stages; four
+  // buses' loads in flight
+  Cx<T>* Us = reinterpret_cast<Cx<T>*>(ring);
+  T* Ms = reinterpret_cast<T*>(Us + N);
+  for (int i0 = tid; i0 < N; i0 += 4 * S) {
+    double2 u[4], v[4];
+    double m[4];
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      const size_t e = (size_t)min(i0 + z * S, N - 1) * Kp + k;
+      u[z] = a.U[e];
+      v[z] = a.V[e];
+      m[z] = a.vm[e];
+    }
+#pragma unroll
+    for (int z = 0; z < 4; ++z)
+      if (i0 + z * S < N) {
+        Us[i0 + z * S] = cx<T>(u[z]);
+        X[i0 + z * S] = cx<T>(v[z]);
+        Ms[i0 + z * S] = (T)m[z];
+      }
+  }
+  for (int q = tid; q <= npos; q += S) stb(F + q, Blk<T>{T(0), T(0), T(0), T(0)});
+  for (int c = tid; c < C; c += S) chunk[c] = __ldg(a.schunk + c);
+  if (tid == 0) {
+    X[N] = Cx<T>{T(0), T(0)};
+    s_bad = 0;
+  }
+  __syncthreads();
+  {
+    const int of = a.of[k], ot = a.ot[k];
+    for (int q0 = tid; q0 < a.n_ent; q0 += 4 * S) {
+      uint4 en[4];
+      double2 y[4];
+#pragma unroll
+      for (int z = 0; z < 4; ++z) en[z] = __ldg(a.sent + min(q0 + z * S, a.n_ent - 1));
+#pragma unroll
+      for (int z = 0; z < 4; ++z) y[z] = __ldg(a.yval + en[z].w);
+#pragma unroll
+      for (int z = 0; z < 4; ++z)
+        if (q0 + z * S < a.n_ent) {
+          const int i = en[z].y & 0xffffu, j = en[z].y >> 16;
+          stb(F + en[z].x, jac_block<T>(a, i, j, y[z], k, of, ot, X[i], Us[j], Ms[j], Cx<T>{T(0), T(0)}, en[z].z & 3,
+                                        en[z].z >> 2));
+        }
+    }
+    for (int i0 = tid; i0 < N; i0 += 4 * S) {
+      uint4 dg[4];
+      double2 ii[4], y[4];
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        const int i = min(i0 + z * S, N - 1);
+        dg[z] = __ldg(a.sdiag + i);
+        ii[z] = a.I[(size_t)i * Kp + k];
+      }
+#pragma unroll
+      for (int z = 0; z < 4; ++z) y[z] = __ldg(a.yval + dg[z].y);
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        const int i = i0 + z * S;
+        if (i < N)
+          stb(F + dg[z].x, jac_block<T>(a, i, i, y[z], k, of, ot, X[i], Us[i], Ms[i], cx<T>(ii[z]), dg[z].z, dg[z].z));
+      }
+    }
+  }
+  __syncthreads();
+  for (int r0 = tid; r0 < N; r0 += 4 * S) {
+    double2 x[4];
+#pragma unroll
+    for (int z = 0; z < 4; ++z) x[z] = a.X[(size_t)min(r0 + z * S, N - 1) * Kp + k];
+#pragma unroll
+    for (int z = 0; z < 4; ++z)
+      if (r0 + z * S < N) X[r0 + z * S] = cx<T>(x[z]);
+  }
+  uint4* stage = reinterpret_cast<uint4*>(ring);
+  const int units = a.chunk_units;
+  auto fetch = [&](int c, int at) {
+    if (c < C) {
+      const int2 ch = chunk[c];
+      for (int u = tid; u < ((ch.y >> 10) & 0xffff); u += S) cp_async16(stage + at * units + u, a.sstream + ch.x + u);
+    }
+    cp_commit();
+  };
+#pragma unroll
+  for (int c = 0; c < NR_STAGES - 1; ++c) fetch(c, c);
+  // This thread's record of the next chunk and its list's first group are
+  // read a chunk ahead: they don't depend on this chunk's results.
+  const uint4 none = make_uint4(0, 0, 0, NR_NONE);
+  uint4 rec = none, grp = none;
+  const uint4* list = nullptr;
+  auto look = [&](int2 ch, int at) {
+    rec = none;
+    if (tid < (ch.y & 1023)) {
+      const uint4* base = ((ch.y >> 10) & 0xffff) ? stage + at * units : a.sstream + ch.x;
+      rec = base[tid];
+      list = base + rec.y;
+      if (rec.z) grp = list[0];
+    }
+  };
+  cp_wait<NR_STAGES - 2>();
+  __syncthreads();
+  int2 ch = chunk[0];
+  look(ch, 0);
+  int at = 0;
+  for (int c = 0; c < C; ++c) {
+    cp_wait<NR_STAGES - 3>();
+    __syncthreads();  // chunk c + 1 has arrived; what the chunks before this one wrote is there
+    int prev = at - 1, next = at + 1;
+    if (prev < 0) prev = NR_STAGES - 1;
+    if (next == NR_STAGES) next = 0;
+    fetch(c + NR_STAGES - 1, prev);
+    const uint4 r = rec, g = grp;
+    const uint4* p = list;
+    const int y = ch.y;
+    if (c + 1 < C) {
+      ch = chunk[c + 1];
+      look(ch, next);
+    }
+    Blk<T> acc;
+    int pos, x2;
+    bool lower = false;
+    if (r.w != NR_NONE) lower = smem_target(p, r, g, F, X, acc, pos, x2, &s_bad);
+    if (y < 0) {
+      __syncthreads();  // the pivots' inverses
+      if (lower) stb(F + pos, mul(acc, ldb(F + x2)));
+    }
+    at = next;
+  }
+  __syncthreads();
+  if (s_bad) {
+    if (tid == 0) a.bad[k] = 1;
+    return;
+  }
+  for (int r = tid; r < N; r += S) {
+    const int i = __ldg(a.order + r);
+    const uint8_t ty = __ldg(a.type + i);
+    const size_t e = (size_t)i * Kp + k;
+    if (ty != NR_SLACK) a.th[e] += (double)X[r].x;
+    if (ty == NR_PQ) a.vm[e] += (double)X[r].y;
+  }
+}
+
+// Shared memory the shared-memory form needs for one case: the factor, the
+// stages (before the factorisation: e^{j theta} and |V|), X, the chunks.
+template <class T>
+size_t lu_ring_bytes(int n, int units) {
+  return std::max((size_t)NR_STAGES * units * 16, ((size_t)n * 3 * sizeof(T) + 15) / 16 * 16);
+}
+template <class T>
+size_t lu_smem_bytes(int64_t npos, int n, int units, int n_chunk) {
+  return (size_t)(npos + 1) * sizeof(Blk<T>) + lu_ring_bytes<T>(n, units) + (size_t)(n + 1) * sizeof(Cx<T>) +
+         (size_t)n_chunk * 8 + 64;  // 64: the static part
 }
 
 __global__ void k_nr_update(NrArgs a) {
@@ -685,6 +955,10 @@ struct dpf_nr {
   int4* rows = nullptr;
   int4* targets = nullptr;
   int2* pairs = nullptr;
+  // shared-memory form, if the grid has one
+  uint4 *sstream = nullptr, *sent = nullptr, *sdiag = nullptr;  // in one allocation, sstream's
+  int2* schunk = nullptr;
+  int n_ent = 0, n_chunk = 0, smem_threads = 0, chunk_units = 0;
   // state
   double *th = nullptr, *vm = nullptr, *Ps = nullptr, *Qs = nullptr;
   double2 *V = nullptr, *U = nullptr, *I = nullptr, *X = nullptr;
@@ -701,12 +975,172 @@ struct dpf_nr {
 static void nr_release(dpf_nr* h) {
   dfree(h->order); dfree(h->rank); dfree(h->frp); dfree(h->fcol); dfree(h->fdiag);
   dfree(h->ymap); dfree(h->lvl_ptr); dfree(h->rlvl_ptr); dfree(h->rows); dfree(h->targets); dfree(h->pairs);
+  dfree(h->sstream);
   dfree(h->th); dfree(h->vm); dfree(h->Ps); dfree(h->Qs); dfree(h->V); dfree(h->U); dfree(h->I); dfree(h->X);
   dfree(h->F); dfree(h->Dinv);
   dfree(h->of); dfree(h->ot); dfree(h->active); dfree(h->status); dfree(h->iters); dfree(h->bad);
   dfree(h->n_active); dfree(h->yff); dfree(h->yft); dfree(h->ytt); dfree(h->maxmis); dfree(h->loss); dfree(h->pmax); dfree(h->psum); dfree(h->maxmis0); dfree(h->loss0);
   if (h->h_nact) cudaFreeHost(h->h_nact);
   h->h_nact = nullptr;
+}
+
+static size_t smem_optin() {
+  int dev = 0, v = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return (size_t)v;
+}
+
+// The shared-memory form's schedule (above upd_group) from the analysis.  The
+// order is free within a level: long lists come first, so that the lanes of a
+// warp walk lists of like length.
+static int nr_setup_smem(dpf_nr* h) {
+  const NrSymbolic& s = h->sym;
+  const dpf_ybus* y = h->y;
+  const int n = s.n, npos = s.row_ptr[(size_t)n];
+  const int S = n <= 64 ? 64 : n <= 256 ? 128 : n <= 1000 ? 256 : NR_SMEM_THREADS;
+  const int units = std::min(4 * S, 512);
+  const uint32_t pad_f = (uint32_t)npos | (uint32_t)npos << 16, pad_x = (uint32_t)npos | (uint32_t)n << 16;
+  struct Item {
+    uint32_t pos, x2, kind;
+    std::vector<uint32_t> list;
+  };
+  auto pad = [](std::vector<uint32_t>& v, uint32_t p) {
+    while (v.size() % 4) v.push_back(p);
+  };
+  std::vector<uint32_t> stream;
+  std::vector<int2> chunks;
+  auto vec = [](const Item* i) { return i->kind == NR_FWD || i->kind == NR_BACK; };
+  // one chunk: block targets from the first thread on, vector targets from the next warp on
+  auto emit = [&](std::vector<const Item*> its, bool staged) {
+    std::stable_sort(its.begin(), its.end(), [&](const Item* a, const Item* b) {
+      if (vec(a) != vec(b)) return vec(b);
+      return a->list.size() > b->list.size();
+    });
+    static const Item none{0, 0, NR_NONE, {}};
+    size_t nb = 0;
+    bool lower = false;
+    for (const Item* i : its) {
+      nb += !vec(i);
+      lower = lower || i->kind == NR_L;
+    }
+    if (nb < its.size()) its.insert(its.begin() + (long)nb, (32 - nb % 32) % 32, &none);
+    const size_t base = stream.size();
+    size_t at = its.size();
+    for (const Item* i : its) {
+      const uint32_t r[4] = {i->pos | i->x2 << 16, (uint32_t)at, (uint32_t)(i->list.size() / 4), i->kind};
+      stream.insert(stream.end(), r, r + 4);
+      at += r[2];
+    }
+    for (const Item* i : its) stream.insert(stream.end(), i->list.begin(), i->list.end());
+    const uint32_t y = (uint32_t)its.size() | (staged ? (uint32_t)at << 10 : 0) | (lower ? 0x80000000u : 0);
+    chunks.push_back(make_int2((int)(base / 4), (int)y));
+  };
+  // chunks of a level from its pivots (whole where they fit a stage)
+  std::vector<std::vector<Item>> pivots;
+  auto pack = [&] {
+    std::vector<std::pair<size_t, size_t>> by_length;  // ~longest list, pivot
+    for (size_t i = 0; i < pivots.size(); ++i) {
+      size_t x = 0;
+      for (const Item& it : pivots[i]) x = std::max(x, it.list.size());
+      by_length.emplace_back(~x, i);
+    }
+    std::sort(by_length.begin(), by_length.end());
+    const size_t most = (size_t)S - 32;  // 32: the fill between block and vector targets
+    std::vector<const Item*> cur;
+    size_t size = 0;
+    auto flush = [&] {
+      if (!cur.empty()) emit(cur, true);
+      cur.clear();
+      size = 0;
+    };
+    for (const auto& ip : by_length) {
+      const std::vector<Item>& pv = pivots[ip.second];
+      size_t u = pv.size();
+      for (const Item& it : pv) u += it.list.size() / 4;
+      if (u + 32 > (size_t)units || pv.size() > most) {
+        flush();
+        std::vector<const Item*> big;
+        for (const Item& it : pv) big.push_back(&it);
+        std::stable_sort(big.begin(), big.end(), [](const Item* a, const Item* b) {
+          return (a->kind == NR_DIAG) > (b->kind == NR_DIAG);
+        });
+        for (size_t i = 0; i < big.size(); i += most)
+          emit(std::vector<const Item*>(big.begin() + (long)i, big.begin() + (long)std::min(big.size(), i + most)), false);
+        continue;
+      }
+      if (size + u + 32 > (size_t)units || cur.size() + pv.size() > most) flush();
+      for (const Item& it : pv) cur.push_back(&it);
+      size += u;
+    }
+    flush();
+  };
+  std::vector<int32_t> row_of((size_t)npos), slot((size_t)n, -1);
+  for (int r = 0; r < n; ++r)
+    for (int q = s.row_ptr[(size_t)r]; q < s.row_ptr[(size_t)r + 1]; ++q) row_of[(size_t)q] = r;
+  for (int l = 0; l < s.n_levels; ++l) {
+    pivots.clear();
+    for (int t = s.lvl_ptr[(size_t)l]; t < s.lvl_ptr[(size_t)l + 1]; ++t) {
+      const int32_t* w = &s.targets[(size_t)8 * t];
+      Item it{(uint32_t)w[0], w[3] == NR_L ? (uint32_t)w[4] : 0, (uint32_t)w[3], {}};
+      for (int p = w[1]; p < w[2]; ++p)
+        it.list.push_back((uint32_t)s.pairs[2 * (size_t)p] | (uint32_t)s.pairs[2 * (size_t)p + 1] << 16);
+      pad(it.list, pad_f);
+      if (w[3] == NR_U && it.list.empty()) continue;
+      const int p = std::min(row_of[(size_t)w[0]], s.col[(size_t)w[0]]);
+      if (slot[(size_t)p] < 0) {
+        slot[(size_t)p] = (int)pivots.size();
+        pivots.emplace_back();
+      }
+      auto& pv = pivots[(size_t)slot[(size_t)p]];
+      pv.push_back(std::move(it));
+      if (w[3] != NR_DIAG || w[4] == w[0]) continue;
+      Item fw{0, (uint32_t)w[7], NR_FWD, {}};
+      for (int q = w[4]; q < w[0]; ++q) fw.list.push_back((uint32_t)q | (uint32_t)s.col[(size_t)q] << 16);
+      pad(fw.list, pad_x);
+      pv.push_back(std::move(fw));
+    }
+    pack();
+  }
+  for (int l = s.n_levels - 1; l >= 0; --l) {
+    pivots.clear();
+    for (int t = s.rlvl_ptr[(size_t)l]; t < s.rlvl_ptr[(size_t)l + 1]; ++t) {
+      const int32_t* w = &s.rows[(size_t)4 * t];
+      Item it{(uint32_t)s.diag[(size_t)w[0]], (uint32_t)w[0], NR_BACK, {}};
+      for (int q = w[1]; q < w[2]; ++q) it.list.push_back((uint32_t)q | (uint32_t)s.col[(size_t)q] << 16);
+      pad(it.list, pad_x);
+      pivots.emplace_back(1, std::move(it));
+    }
+    pack();
+  }
+  if (stream.size() / 4 > 0x7fffffffu) return DPF_OK;
+  // blocks by Y_bus entry, and the diagonal by bus
+  std::vector<uint4> ent, dg((size_t)n);
+  for (int r = 0; r < n; ++r)
+    for (int q = s.row_ptr[(size_t)r]; q < s.row_ptr[(size_t)r + 1]; ++q) {
+      const int yp = s.ymap[(size_t)q], i = s.order[(size_t)r], j = s.order[(size_t)s.col[(size_t)q]];
+      const uint32_t ti = y->bus_type[(size_t)y->perm[(size_t)i]], tj = y->bus_type[(size_t)y->perm[(size_t)j]];
+      if (yp < 0) continue;
+      if (i == j) dg[(size_t)i] = make_uint4((uint32_t)q, (uint32_t)yp, ti, 0);
+      else ent.push_back(make_uint4((uint32_t)q, (uint32_t)i | (uint32_t)j << 16, ti | tj << 2, (uint32_t)yp));
+    }
+  std::sort(ent.begin(), ent.end(), [](const uint4& a, const uint4& b) { return a.w < b.w; });
+  // one allocation: the stream, entries and diagonal (16-byte units), the chunks
+  const size_t ns = stream.size() / 4, ne = ent.size(), nc = chunks.size();
+  std::vector<uint4> all(ns + ne + (size_t)n + (nc + 1) / 2);
+  memcpy(all.data(), stream.data(), ns * 16);
+  std::copy(ent.begin(), ent.end(), all.begin() + (long)ns);
+  std::copy(dg.begin(), dg.end(), all.begin() + (long)(ns + ne));
+  memcpy(all.data() + ns + ne + (size_t)n, chunks.data(), nc * 8);
+  TRY(upload(&h->sstream, all));
+  h->sent = h->sstream + ns;
+  h->sdiag = h->sent + ne;
+  h->schunk = reinterpret_cast<int2*>(h->sdiag + n);
+  h->n_ent = (int)ent.size();
+  h->n_chunk = (int)chunks.size();
+  h->smem_threads = S;
+  h->chunk_units = units;
+  return DPF_OK;
 }
 
 static int nr_setup(dpf_nr* h) {
@@ -727,6 +1161,7 @@ static int nr_setup(dpf_nr* h) {
   CK(cudaMemcpy(h->targets, s.targets.data(), s.targets.size() * 4, cudaMemcpyHostToDevice));
   TRY(dalloc(&h->pairs, s.pairs.size() / 2));
   if (!s.pairs.empty()) CK(cudaMemcpy(h->pairs, s.pairs.data(), s.pairs.size() * 4, cudaMemcpyHostToDevice));
+  if (lu_smem_bytes<float>((int64_t)npos, n, 0, 0) <= smem_optin()) TRY(nr_setup_smem(h));
   const int Kp = h->Kp;
   const size_t E = (size_t)n * Kp;
   TRY(dalloc(&h->th, E)); TRY(dalloc(&h->vm, E));
@@ -786,28 +1221,29 @@ extern "C" int dpf_nr_stats(const dpf_nr* h, int64_t* n_pos, int64_t* n_pairs, i
   return DPF_OK;
 }
 
+// CTAs of the shared-memory form an SM holds.
+template <class T>
+static int smem_ctas(int threads, size_t bytes, int* n) {
+  CK(cudaFuncSetAttribute(k_nr_lu_smem<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_nr_lu_smem<T>, threads, bytes));
+  return DPF_OK;
+}
+
 template <class T>
 static int nr_iterate_linear(dpf_nr* h, const NrArgs& a, bool smem, cudaStream_t s) {
   if (smem) {
-    const size_t bytes = lu_smem_bytes<T>(a.npos, a.N);
-    CK(cudaFuncSetAttribute(k_nr_lu_smem<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    k_nr_lu_smem<T><<<a.K, NR_SMEM_THREADS, bytes, s>>>(a);
+    const size_t bytes = lu_smem_bytes<T>(a.npos, a.N, a.chunk_units, a.n_chunk);
+    k_nr_lu_smem<T><<<a.K, h->smem_threads, bytes, s>>>(a);
     CKLAUNCH();
     h->launches += 1;
     return DPF_OK;
   }
   k_nr_assemble<T><<<grid_for((size_t)a.N * a.Kp), 256, 0, s>>>(a);
   k_nr_lu<T><<<a.Kp / a.C, sizeof(T) == 8 ? NR_THREADS / 2 : NR_THREADS, 0, s>>>(a);
+  k_nr_update<<<grid_for((size_t)a.N * a.Kp), 256, 0, s>>>(a);
   CKLAUNCH();
-  h->launches += 2;
+  h->launches += 3;
   return DPF_OK;
-}
-
-static size_t smem_optin() {
-  int dev = 0, v = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  return (size_t)v;
 }
 
 extern "C" void dpf_nr_default_opts(dpf_nr_opts* o) {
@@ -872,13 +1308,26 @@ extern "C" int dpf_nr_solve(dpf_nr* h, const dpf_batch* b, const dpf_nr_opts* o,
   };
   a.C = lanes_for(K);
   // The shared-memory form where one case's factor fits and the cases still
-  // iterating fit in one wave of one CTA per SM (its walk down the tree is
-  // shorter, but a second wave would double it); else the global-memory
-  // form.  Both give the same bits.  o->lanes > 0 forces the global form.
-  const size_t need = precision == DPF_FP64 ? lu_smem_bytes<double>(sym.row_ptr[sym.n], y->n)
-                                            : lu_smem_bytes<float>(sym.row_ptr[sym.n], y->n);
-  const bool fits = o->lanes == 0 && need <= smem_optin();
-  bool smem = false;
+  // iterating are few: it takes a case in the least time, the global form the
+  // most cases at a time (it hides one case's latency behind others).  Both
+  // give the same bits; o->lanes > 0 forces the global form.  Whole solve in
+  // ms by waves of CTAs, shared-memory and global form: FP32, 2,000 buses, 1
+  // case 1.0 / 1.9, 300 (2 waves) 2.3 / 4.3, 850 (6) 6.2 / 7.5, 2,379 (16)
+  // 17.1 / 12.8; 1,000 buses, 300 (2) 1.6 / 3.1, 2,000 (14) 8.8 / 7.0; 300
+  // buses, 300 (1) 1.1 / 2.0, 3,000 (7) 4.0 / 4.0; 118, 3,000 (4) 1.35 /
+  // 1.52.  FP64, one wave: 30 buses, 1 case 1.2 / 1.4; 118, 500 1.0 / 1.3; 300,
+  // 300 2.3 / 3.7; 1,000, 120 2.9 / 5.0; but 30 buses, 1,500 (10 CTAs an SM) 2.1
+  // / 1.7 and 118, 3,000 3.5 / 2.7: a few CTAs keep the FP64 pipe busy.
+  const size_t need = precision == DPF_FP64 ? lu_smem_bytes<double>(sym.row_ptr[sym.n], y->n, h->chunk_units, h->n_chunk)
+                                            : lu_smem_bytes<float>(sym.row_ptr[sym.n], y->n, h->chunk_units, h->n_chunk);
+  const bool fits = o->lanes == 0 && h->sstream && need <= smem_optin();
+  int smem_cases = 0;  // most cases the shared-memory form takes
+  if (fits) {
+    int per_sm = 0;
+    if (precision == DPF_FP64) TRY(smem_ctas<double>(h->smem_threads, need, &per_sm));
+    else TRY(smem_ctas<float>(h->smem_threads, need, &per_sm));
+    smem_cases = num_sms_nr() * (precision == DPF_FP64 ? std::min(per_sm, 4) : per_sm * 6);
+  }
   a.va_slack = y->va_slack;
   a.tol = tol;
   a.inv_m = y->m_loss > 0 ? 1.0 / y->m_loss : 0.0;
@@ -903,6 +1352,15 @@ extern "C" int dpf_nr_solve(dpf_nr* h, const dpf_batch* b, const dpf_nr_opts* o,
   a.pairs = h->pairs;
   a.rlvl_ptr = h->rlvl_ptr;
   a.rows = h->rows;
+  a.sstream = h->sstream;
+  a.schunk = h->schunk;
+  a.sent = h->sent;
+  a.sdiag = h->sdiag;
+  a.n_ent = h->n_ent;
+  a.n_chunk = h->n_chunk;
+  a.chunk_units = h->chunk_units;
+  a.ring_bytes = (int)(precision == DPF_FP64 ? lu_ring_bytes<double>(y->n, h->chunk_units)
+                                             : lu_ring_bytes<float>(y->n, h->chunk_units));
   a.npos = sym.row_ptr[sym.n];
   a.th = h->th;
   a.vm = h->vm;
@@ -951,12 +1409,9 @@ extern "C" int dpf_nr_solve(dpf_nr* h, const dpf_batch* b, const dpf_nr_opts* o,
     // few cases left: fewer cases per CTA, more slots per case (a shorter
     // walk for each; CTAs whose cases have all stopped return at once)
     a.C = lanes_for(*h->h_nact);
-    smem = fits && *h->h_nact <= num_sms_nr();
+    const bool smem = *h->h_nact <= smem_cases;
     if (precision == DPF_FP64) TRY(nr_iterate_linear<double>(h, a, smem, s));
     else TRY(nr_iterate_linear<float>(h, a, smem, s));
-    k_nr_update<<<grid_for(E), 256, 0, s>>>(a);
-    CKLAUNCH();
-    h->launches += 1;
   }
   const int fb = o->fallback && !flat_start;
   k_nr_out<<<grid_for(E), 256, 0, s>>>(a, b->va, b->vm, fb);

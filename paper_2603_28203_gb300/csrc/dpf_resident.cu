@@ -22,10 +22,10 @@
 // that order.
 //
 // Measured (2,379 N-1 cases of a 2,000-bus grid, refined FP32): 123 us per
-// iteration streaming, 84 us on chip.  What bounds it now is instruction issue
+// iteration streaming, 80 us on chip.  What bounds it now is instruction issue
 // (62% of the slots, 434 instructions per 32 rows and iteration), then the
 // shared-memory pipe (57%: two rows of 8-byte gathers at random banks).  8,192
-// cases of 30 buses: 15.9 -> 8.8 us; one case of 30 buses in FP64: 17.8 -> 9.0.
+// cases of 30 buses: 15.9 -> 8.2 us; one case of 30 buses in FP64: 17.8 -> 8.7.
 //
 // The results are those of the streaming kernels to the bit: the same device
 // functions on the same operands, each row's products in the same order, and
@@ -193,9 +193,11 @@ __device__ __forceinline__ void res_stage(const ResArgs<R>& q, unsigned char* sm
   }
 }
 
-// One warp per case, RES_TEAMS cases per CTA.
+// One warp per case, RES_TEAMS cases per CTA.  CTAs an SM: 250 iterations of
+// 8,192 cases of 30 buses (one row a lane) 2.04 ms at 6, 2.07 at 5, 2.31 at 4;
+// 3,000 of 60 (two rows) 0.66, 0.60, 0.80.
 template <class R, bool REF, bool ADAM, int RPT>
-__global__ void __launch_bounds__(32 * RES_TEAMS, sizeof(R) == 8 ? 3 : 5)
+__global__ void __launch_bounds__(32 * RES_TEAMS, sizeof(R) == 8 ? 3 : RPT == 1 ? 6 : 5)
     k_resident_warp(const ResArgs<R> q) {
   using C = typename Prec<R>::C;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -556,7 +558,7 @@ ResShape res_shape(const dpf_ybus* y, int K, bool fp64, bool refined, const Loss
   // 3,471 1,886; but 1000x300 11,344 12,548; 1x700 2,454 3,500.  In FP32 it is
   // faster over the whole range measured (30-2,048 buses, 1-3,000 cases):
   // 1x30 1,169 330; 3000x30 1,330 486; 1x2000 1,234 732; 3000x2000 17,719
-  // 13,284; 3000x300 3,216 2,346; 3000x1000 8,710 6,501.
+  // 12,700; 3000x300 3,216 2,071; 3000x1000 8,710 5,938.
   if (fp64 && n > RES_WARP_N && (n > 320 || K > 300)) return sh;
   sh.warp = n <= RES_WARP_N;
   sh.rpt = sh.warp && n <= 32 ? 1 : 2;
