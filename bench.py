@@ -523,6 +523,9 @@ def run_ours(args):
                 "fwd_adj_combined_frac": (fwd_b + adj_b) / ((fwd_avg + adj_avg) / 1e3) / 1e9 / peak,
                 "timed_launches": n_adj,
                 "l2_peak": l2,
+                "note": "the two passes larger grids iterate with, timed apart; the timed solve keeps a case "
+                        "of this size on chip (k_resident_cta) and is bound by instruction issue",
+                "step_us_per_iteration": 1e3 * t_max / args.steps / t_done if t_done else None,
             },
             "gpu_launches": int(launches),
             "clocks": clk,
@@ -665,8 +668,7 @@ def run_flat_fp32(dpf, torch, job, args, peak, l2):
                              "frac_of_l2_peak": fg / l2["gbs"], "traffic": _ncu_traffic("k_fwd_n1_2kbus")},
                      "fwd_adj_combined_gbs": (fwd_b + adj_b) / ((fa + aa) / 1e3) / 1e9,
                      "fwd_adj_combined_frac": (fwd_b + adj_b) / ((fa + aa) / 1e3) / 1e9 / peak,
-                     "fwd_adj_per_iteration_gbs": (fwd_b + adj_b) / (ms / n_it / 1e3) / 1e9,
-                     "fwd_adj_per_iteration_frac": (fwd_b + adj_b) / (ms / n_it / 1e3) / 1e9 / peak},
+                     "note": "the two passes, timed apart; the timed iterations run on chip"},
         "launch_shape": {"lanes": opts.lanes, "warps": opts.warps, "row_blocks": opts.row_blocks,
                          "pair_cases": opts.pair_cases, "stage_v": opts.stage_v},
         "after_table2_budget": {"iterations": ITERS_PER_SOLVE, "converged": int((st == 0).sum()),
@@ -1272,19 +1274,19 @@ def run_dc(args):
     print(json.dumps({
         "workload": "dc",
         "config": {"grid": "c3_n1_2kbus", "n_bus": int(g.n_bus), "cases": int(K), "tol_rel_residual": 1e-10,
-                   "solver": "Jacobi-preconditioned CG, double-float vectors (FP32 pairs), FP64 scalars, "
-                             "all cases batched"},
+                   "solver": "Jacobi-preconditioned CG on chip, one CTA per case, double-float vectors and "
+                             "scalars (FP32 pairs)"},
         "wall_ms": 1e3 * wall,
         "cg_iterations_max": iters_max, "cg_iterations_p50": float(np.median(it)),
         "us_per_cg_iteration": 1e6 * wall / max(iters_max, 1),
-        "roofline": {"bound": "hbm", "unit": "GB/s", "peak": peak, "peak_source": src,
-                     "achieved": b * iters_max / wall / 1e9, "frac": b * iters_max / wall / 1e9 / peak,
-                     "algorithmic_bytes_per_iteration": b,
+        "roofline": {"bound": "instruction issue",
+                     "two_launch_form": {"bytes_per_iteration": b, "floor_us_per_iteration": b / peak / 1e3,
+                                         "peak_gbs": peak, "peak_source": src},
                      "flops": {"unit": "TFLOP/s", "achieved": fl * iters_max / wall / 1e12,
                                "algorithmic_flops_per_iteration": fl,
                                "note": "double-float arithmetic on the FP32 pipes (nominal FP64 rate "
                                        f"{FP64_NOMINAL_TFLOPS} TFLOP/s for comparison)"},
-                     "note": "all cases run until the slowest converges (host polls every 16 iterations)"},
+                     "note": "vectors and matrix stay on chip; each case stops by itself"},
         "max_rel_error_vs_oracle_sampled": err,
         "alg1_after_1000_iterations": mm,
     }), flush=True)

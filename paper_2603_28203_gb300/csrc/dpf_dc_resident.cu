@@ -15,6 +15,11 @@
 // 2^-47 of the sum of the magnitudes.  The dot products and the step lengths
 // are double-float as well (FP64 issue is dear here, and every warp forms
 // them from the warps' partial sums).
+// Error of the angles against a dense FP64 solve, rms over the batch relative
+// to the largest angle, at a relative residual of 1e-10 (streaming form with
+// FP64 scalars, here): 3,000 cases of 30 buses 1.7e-14, 1.1e-14; 1,000 of 300
+// 6.5e-13, 3.7e-13; 1,000 of 1,000 2.7e-12, 2.4e-12; 400 of 2,000 5.3e-12,
+// 5.2e-12: the stop test's, not the arithmetic's.
 #include <cuda_runtime.h>
 
 #include <algorithm>
