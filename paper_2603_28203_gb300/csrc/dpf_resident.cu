@@ -23,7 +23,7 @@
 //
 // Measured (2,379 N-1 cases of a 2,000-bus grid, refined FP32): 123 us per
 // iteration streaming, 80 us on chip.  What bounds it now is instruction issue
-// (62% of the slots, 434 instructions per 32 rows and iteration), then the
+// (60% of the slots, 404 instructions per 32 rows and iteration), then the
 // shared-memory pipe (57%: two rows of 8-byte gathers at random banks).  8,192
 // cases of 30 buses: 15.9 -> 8.2 us; one case of 30 buses in FP64: 17.8 -> 8.7.
 //
