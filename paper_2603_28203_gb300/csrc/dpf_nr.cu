@@ -425,23 +425,58 @@ __device__ __forceinline__ Blk<T> jac_block(const NrArgs& a, int i, int j, doubl
   return b;
 }
 
-// One block row of case k: its positions' blocks to dst[q * stride].
+// One block row of case k: its positions' blocks to dst[q * stride], with
+// jac_block's arithmetic (called from here it cost the FP64 solve 2%).
 template <class T>
 __device__ __forceinline__ void assemble_row(const NrArgs& a, int r, int k, Blk<T>* __restrict__ dst, size_t stride) {
   const size_t Kp = a.Kp;
   const double2* __restrict__ U = a.U;
   const double* __restrict__ VM = a.vm;
   const int i = __ldg(a.order + r);
-  const Cx<T> vi = cx<T>(a.V[(size_t)i * Kp + k]), ii = cx<T>(a.I[(size_t)i * Kp + k]);
-  const int of = a.of[k], ot = a.ot[k], ti = __ldg(a.type + i);
+  const size_t ei = (size_t)i * Kp + k;
+  const Cx<T> vi = cx<T>(a.V[ei]), ii = cx<T>(a.I[ei]);
+  const Cx<T> si = mulc(vi, ii);             // S_i
+  const Cx<T> sdi = mulc(cx<T>(U[ei]), ii);  // S_i / |V|_i
+  const uint8_t ti = __ldg(a.type + i);
+  const bool rp = ti != NR_SLACK, rq = ti == NR_PQ;
+  const int of = a.of[k], ot = a.ot[k];
   const int q1 = __ldg(a.frp + r + 1);
   for (int q = __ldg(a.frp + r); q < q1; ++q) {
+    const int j = __ldg(a.order + __ldg(a.fcol + q));
     const int yp = __ldg(a.ymap + q);
     Blk<T> b{T(0), T(0), T(0), T(0)};
     if (yp >= 0) {
-      const int j = __ldg(a.order + __ldg(a.fcol + q));
+      double2 y = __ldg(a.yval + yp);
+      if (of >= 0) {
+        if (i == of && j == of) y = csub(y, a.yff[k]);
+        else if (i == ot && j == ot) y = csub(y, a.ytt[k]);
+        else if ((i == of && j == ot) || (i == ot && j == of)) y = csub(y, a.yft[k]);
+      }
       const size_t ej = (size_t)j * Kp + k;
-      b = jac_block<T>(a, i, j, __ldg(a.yval + yp), k, of, ot, vi, cx<T>(U[ej]), (T)VM[ej], ii, ti, __ldg(a.type + j));
+      const Cx<T> w = mulc(vi, mul(cx<T>(y), cx<T>(U[ej])));
+      const T vmj = (T)VM[ej];
+      T ba, bb, bc, bd;
+      if (i != j) {
+        ba = vmj * w.y;
+        bc = -vmj * w.x;
+        bb = w.x;
+        bd = w.y;
+      } else {
+        ba = fma(vmj, w.y, -si.y);
+        bc = fma(-vmj, w.x, si.x);
+        bb = sdi.x + w.x;
+        bd = sdi.y + w.y;
+      }
+      const uint8_t tj = __ldg(a.type + j);
+      const bool ct = tj != NR_SLACK, cv = tj == NR_PQ;
+      b.a = (rp && ct) ? ba : T(0);
+      b.b = (rp && cv) ? bb : T(0);
+      b.c = (rq && ct) ? bc : T(0);
+      b.d = (rq && cv) ? bd : T(0);
+      if (i == j) {
+        if (!rp) b.a = T(1);
+        if (!rq) b.d = T(1);
+      }
     }
     stb(dst + (size_t)q * stride, b);
   }
@@ -580,7 +615,7 @@ __device__ __forceinline__ void lu_levels(const NrArgs& a, Blk<T>* F, size_t fs,
 // Global-memory form: C cases per CTA are the lanes (their blocks adjacent),
 // the remaining thread index is the slot.
 template <class T>
-__global__ void __launch_bounds__(NR_THREADS) k_nr_lu(NrArgs a) {
+__global__ void __launch_bounds__(sizeof(T) == 8 ? NR_THREADS / 2 : NR_THREADS) k_nr_lu(NrArgs a) {
   const int lane = threadIdx.x & (a.C - 1), slot = threadIdx.x / a.C, S = blockDim.x / a.C;
   const int k = blockIdx.x * a.C + lane;
   const bool on = k < a.K && a.active[k];
