@@ -1460,7 +1460,8 @@ static int dc_run_t(dpf_workspace* w, const int32_t* outage_dev, double tol, int
     else
       k_dc_flow<float><<<cb, 256, 0, s>>>((const float4*)w->ms, a.of, a.ot, a.ob, c + 8 * (size_t)Kp, w->K, Kp);
   }
-  if (d.res_rord) {  // (every grid up to RES_MAX_N buses)
+  const DcShape on_chip = dc_res_shape(y, w->K, sizeof(T) == 4);
+  if (on_chip.ok) {
     DcRes c;
     c.K = w->K;
     c.Kp = Kp;
@@ -1476,7 +1477,7 @@ static int dc_run_t(dpf_workspace* w, const int32_t* outage_dev, double tol, int
     c.x = w->tmp_a;
     c.res = a.res;
     c.iters = a.iters;
-    CK((cudaError_t)dc_res_launch(y, c, sizeof(T) == 4, s));
+    CK((cudaError_t)dc_res_launch(y, c, on_chip, sizeof(T) == 4, s));
     w->launches += shift ? 3 : 2;
     return DPF_OK;
   }

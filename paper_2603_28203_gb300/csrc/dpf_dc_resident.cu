@@ -29,6 +29,8 @@
 
 namespace dpf {
 
+constexpr size_t DC_STATIC_SMEM = 1024;  // of k_dc_resident, at most
+
 template <class T> struct DcResArgs {
   int N, K, Kp, T_, n_pair, n_slice, max_iter;
   const int32_t* rord;
@@ -124,6 +126,7 @@ __global__ void __launch_bounds__(2048 / RPT, RPT == 8 ? 2 : 1) k_dc_resident(co
     double rr0;
     int pf, pt;
   } cs;
+  static_assert(sizeof part + sizeof cs <= DC_STATIC_SMEM, "static shared memory");
   const int k = blockIdx.x;
   const size_t Kp = (size_t)q.Kp;
   for (int t = tid; t < q.n_pair * 32; t += nt) {
@@ -303,8 +306,31 @@ __global__ void __launch_bounds__(2048 / RPT, RPT == 8 ? 2 : 1) k_dc_resident(co
   }
 }
 
+// Rows per thread where cases outnumber SMs (the best of each type, see the kernel).
+template <class T> constexpr int dc_many() { return sizeof(T) == 8 ? 4 : 8; }
+
+DcShape dc_res_shape(const dpf_ybus* y, int K, bool f32) {
+  DcShape sh;
+  const DeviceYbus& d = y->dev;
+  if (!d.res_rord) return sh;
+  int dev = 0, sms = 1, lim = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  // more cases than SMs: many rows per thread; else two, the shorter iteration
+  // (one case of 2,000 buses to 1e-10: 27.4 ms streaming, 3.9 ms)
+  sh.rpt = K > sms ? (f32 ? dc_many<float>() : dc_many<float2>()) : 2;
+  sh.T = std::max(32, ((y->n + sh.rpt - 1) / sh.rpt + 31) / 32 * 32);
+  const size_t v = f32 ? sizeof(float) : sizeof(float2);
+  sh.smem = (size_t)d.res_pairs * 32 * (2 * v + 4) + (size_t)sh.T * sh.rpt * v;
+  // B as sliced ELL is what may not fit: its slices are as long as their
+  // longest row (a star of 700 buses takes 243 KB, a dense grid of 150 240 KB)
+  sh.ok = sh.smem + DC_STATIC_SMEM <= (size_t)lim;
+  return sh;
+}
+
 template <class T>
-static int dc_res_t(const dpf_ybus* y, const DcRes& c, cudaStream_t s) {
+static int dc_res_t(const dpf_ybus* y, const DcRes& c, const DcShape& sh, cudaStream_t s) {
   const DeviceYbus& d = y->dev;
   DcResArgs<T> q;
   q.N = y->n;
@@ -333,25 +359,17 @@ static int dc_res_t(const dpf_ybus* y, const DcRes& c, cudaStream_t s) {
   q.res = c.res;
   q.iters = c.iters;
   q.tol2 = c.tol * c.tol;
-  int dev = 0, sms = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // more cases than SMs: many rows per thread (the best of each type, see the
-  // kernel); else two, the shorter iteration (one case of 2,000 buses to 1e-10:
-  // 27.4 ms streaming, 3.9 ms)
-  constexpr int many = sizeof(T) == 8 ? 4 : 8;
-  const int rpt = c.K > sms ? many : 2;
-  q.T_ = std::max(32, ((q.N + rpt - 1) / rpt + 31) / 32 * 32);
-  const size_t smem = (size_t)q.n_pair * 32 * (2 * sizeof(T) + 4) + (size_t)q.T_ * rpt * sizeof(T);
-  auto kern = rpt == many ? k_dc_resident<T, many> : k_dc_resident<T, 2>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int many = dc_many<T>();
+  q.T_ = sh.T;
+  auto kern = sh.rpt == many ? k_dc_resident<T, many> : k_dc_resident<T, 2>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
   if (e != cudaSuccess) return e;
-  kern<<<c.K, q.T_, smem, s>>>(q);
+  kern<<<c.K, q.T_, sh.smem, s>>>(q);
   return cudaGetLastError();
 }
 
-int dc_res_launch(const dpf_ybus* y, const DcRes& c, bool f32, void* stream) {
-  return f32 ? dc_res_t<float>(y, c, (cudaStream_t)stream) : dc_res_t<float2>(y, c, (cudaStream_t)stream);
+int dc_res_launch(const dpf_ybus* y, const DcRes& c, const DcShape& sh, bool f32, void* stream) {
+  return f32 ? dc_res_t<float>(y, c, sh, (cudaStream_t)stream) : dc_res_t<float2>(y, c, sh, (cudaStream_t)stream);
 }
 
 }  // namespace dpf

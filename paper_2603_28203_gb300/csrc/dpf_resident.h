@@ -65,8 +65,17 @@ struct DcRes {
   double *x, *res;       // [N][Kp] FP64 solution; |r| / |r0| per case
   int32_t* iters;
 };
-// f32: FP32 vectors, else double-float.  Returns a cudaError_t.
-int dc_res_launch(const dpf_ybus* y, const DcRes& c, bool f32, void* stream);
+// Launch shape for K cases (f32: FP32 vectors, else double-float); ok: the
+// grid has the sliced form and one case fits the shared memory of an SM.
+struct DcShape {
+  bool ok = false;
+  int rpt = 2;  // rows per thread
+  int T = 32;   // threads
+  size_t smem = 0;
+};
+DcShape dc_res_shape(const dpf_ybus* y, int K, bool f32);
+// Returns a cudaError_t.
+int dc_res_launch(const dpf_ybus* y, const DcRes& c, const DcShape& sh, bool f32, void* stream);
 
 // Evaluation of whole cases on chip (dpf_eval.cu), one CTA per case: S_calc,
 // or the loss and its adjoint.  Inputs and outputs are the caller's case-major

@@ -1,0 +1,82 @@
+"""Grids with long rows (stars, dense and randomly meshed networks): their sliced
+form of Y_bus may not fit shared memory, or is mostly padding."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import gridgen
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2603_28203_gb300 as dpf  # noqa: E402
+
+DEV = torch.device("cuda:0")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import os
+    from paper_2603_28203_gb300.build import LIB, build
+    if not os.path.exists(LIB):
+        build()
+    dpf.lib()
+
+
+def _star(n):
+    g = gridgen.make_grid(n, 3, load_scale=0.05)
+    hub = int(np.flatnonzero(g.bus_type == gridgen.SLACK)[0])
+    rng, m = np.random.default_rng(1), n - 1
+    r = rng.uniform(0.002, 0.02, m)
+    return dataclasses.replace(g, f_bus=np.full(m, hub, np.int32), t_bus=np.delete(np.arange(n), hub).astype(np.int32),
+                               r=r, x=10 * r, b_ch=np.zeros(m), tap=np.ones(m), shift=np.zeros(m))
+
+
+def _grid(name):
+    if name.startswith("star"):
+        return _star(int(name[4:]))
+    n, extra = (int(v) for v in name.split("+"))
+    return gridgen.add_random_branches(gridgen.make_grid(n, 3, load_scale=0.05), extra, 1)
+
+
+def _residual(g, va, p):
+    """|B theta - P| / |P| over the non-slack rows in FP64."""
+    flow = (va[g.f_bus] - va[g.t_bus]) / (g.x * np.where(g.tap == 0, 1.0, g.tap))
+    r = -p.copy()
+    np.add.at(r, g.f_bus, flow)
+    np.add.at(r, g.t_bus, -flow)
+    u = g.bus_type != gridgen.SLACK
+    return np.linalg.norm(r[u]) / np.linalg.norm(p[u])
+
+
+# sliced form of B: 243 KB (double-float), 712 / 427 KB, 249 KB, 232 KB; the
+# last one just fits
+@pytest.mark.parametrize("name", ["star700", "star2048", "150+10500", "300+10000", "300+9000"])
+@pytest.mark.parametrize("tol", [1e-10, 1e-4])
+@pytest.mark.parametrize("K", [2, 160])
+def test_dc_of_a_dense_grid(name, tol, K):
+    """A grid whose sliced B doesn't fit shared memory takes the streaming CG;
+    bars as for the on-chip solve (test_dc_on_chip_residual): 2 tol in
+    double-float, 10 tol in FP32."""
+    g = _grid(name)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    P = g.p_spec * (1 + 0.1 * np.random.default_rng(2).uniform(-1, 1, (K, 1)))
+    Pt = torch.tensor(P, device=DEV)
+    out = dpf.dpf_dc_solve(y, ws, K, p_spec=Pt, tol=tol)
+    assert (out["rel_residual"].cpu().numpy() <= tol).all() and (out["iters"].cpu().numpy() >= 1).all()
+    bar = (2 if tol < 1e-5 else 10) * tol
+    va = out["va"].cpu().numpy()
+    for k in range(0, K, max(1, K // 5)):
+        assert _residual(g, va[k], P[k]) <= bar, k
+    # the same start inside a solve
+    res = dict(va=torch.zeros((K, g.n_bus), dtype=torch.float64, device=DEV),
+               vm=torch.zeros((K, g.n_bus), dtype=torch.float64, device=DEV))
+    dpf.dpf_solve_batch(y, ws, dpf.SolveOpts(precision=dpf.FP32R, max_iter=0, dc_start=1, dc_tol=tol), n_case=K,
+                        p_spec=Pt, q_spec=torch.zeros_like(Pt), **res)
+    for k in range(0, K, max(1, K // 5)):
+        assert _residual(g, res["va"][k].cpu().numpy(), P[k]) <= bar, k
