@@ -279,6 +279,12 @@ int dpf_solve_iterate(dpf_workspace* ws, int32_t n_iter, void* stream);
  * are those of the two-pass kernels (FP32, FP32R: to the bit; lanes, warps,
  * row_blocks and pair_cases then only set the order of the loss sum). */
 int dpf_solve_end(dpf_workspace* ws, const dpf_batch* b, void* stream);
+/* The kernel over the whole GPU waits at barriers between its CTAs.  A wait
+ * gives up after `polls` polls (0: the default, about a second); the solve then
+ * ends with DPF_E_CUDA from dpf_active_count, dpf_solve_end or dpf_solve_batch
+ * and no outputs.  dpf_solve_end therefore synchronises `stream` for such
+ * solves (unless it is being captured). */
+int dpf_wait_limit(dpf_workspace* ws, int64_t polls);
 /* Autotuner.  Times candidate launch shapes of the solve loop on this batch
  * -- cases per row group (`lanes`, i.e. rows per warp = 32/lanes), warps per
  * CTA, row blocks, the two-cases-per-thread variants and shared-memory V

@@ -19,5 +19,5 @@ from .dpf import (DPFError, SolveOpts, Workspace, Ybus, dpf_active_count, dpf_ad
                   dpf_nr_solve, dpf_paramid_begin, dpf_paramid_step, dpf_power,
                   dpf_power_noalloc,
                   dpf_solve_batch, dpf_solve_begin, dpf_solve_end,
-                  dpf_solve_iterate, dpf_status_str, dpf_workspace_create, dpf_ybus_bridges,
+                  dpf_solve_iterate, dpf_status_str, dpf_wait_limit, dpf_workspace_create, dpf_ybus_bridges,
                   dpf_ybus_export, dpf_ybus_upload, lib)

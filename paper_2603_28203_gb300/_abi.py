@@ -82,6 +82,7 @@ SIGNATURES = {
     "dpf_solve_end": (C.c_int, [VP, C.POINTER(DpfBatch), VP]),
     "dpf_active_count": (C.c_int, [VP, p_i32, VP]),
     "dpf_autotune": (C.c_int, [VP, VP, C.POINTER(DpfBatch), C.POINTER(DpfSolveOpts), I32, VP]),
+    "dpf_wait_limit": (C.c_int, [VP, C.c_int64]),
     "dpf_iterations_done": (C.c_int, [VP, p_i32]),
     "dpf_power": (C.c_int, [VP, VP, I32, VP, VP, VP, I32, VP, VP, VP]),
     "dpf_loss_backward": (C.c_int, [VP, VP, I32, VP, VP, VP, VP, VP, VP, VP, I32,

@@ -397,6 +397,7 @@ struct dpf_workspace {
   float* grid_terms = nullptr;
   unsigned* grid_sus = nullptr;
   unsigned* grid_bar = nullptr;
+  int64_t grid_polls = GRID_POLLS;
   bool pid_ready = false;  // operating points staged by dpf_paramid_begin
   std::vector<std::pair<std::vector<long long>, std::vector<int>>> tune_cache;  // key -> (lanes, warps, rb, pairs)
   bool spec_per_case = false, has_outage = false;
@@ -880,7 +881,7 @@ static int launch_span(dpf_workspace* w, cudaStream_t s, int n, bool with_check)
     if (with_check) TRY(launch_check_any(w, s, false));
     CK((cudaError_t)grid_launch(make_plan<float>(w).it, w->grid, w->res_lo, w->lanes, w->K, n,
                                 w->precision == DPF_FP32R, w->grid_terms, w->grid_sus, w->grid_bar, w->n_active + 1,
-                                s));
+                                w->grid_polls, s));
     w->launches++;
     return DPF_OK;
   }
@@ -1674,6 +1675,13 @@ extern "C" int dpf_active_count(dpf_workspace* w, int32_t* n_active, void* strea
   return barrier_error(w);
 }
 
+extern "C" int dpf_wait_limit(dpf_workspace* w, int64_t polls) {
+  if (!w) return fail(DPF_E_INVALID, "dpf_wait_limit: NULL workspace");
+  if (polls < 0) return fail(DPF_E_INVALID, "dpf_wait_limit: polls must be >= 0");
+  w->grid_polls = polls ? polls : GRID_POLLS;
+  return DPF_OK;
+}
+
 extern "C" int dpf_profile_enable(dpf_workspace* w, int32_t on) {
   if (!w) return fail(DPF_E_INVALID, "dpf_profile_enable: NULL workspace");
   w->profile = on != 0;
@@ -1824,6 +1832,18 @@ extern "C" int dpf_solve_end(dpf_workspace* w, const dpf_batch* b, void* stream)
   cudaStream_t s = (cudaStream_t)stream;
   const dpf_ybus* y = w->y;
   const bool hio = b->host_io != 0;
+  if (w->grid.ok) {  // a barrier that gave up leaves no state to return (a stream being captured cannot be waited for)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(s, &cap));
+    if (cap == cudaStreamCaptureStatusNone) {
+      int32_t act;
+      const int rc = dpf_active_count(w, &act, s);
+      if (rc != DPF_OK) {
+        w->begun = false;
+        return rc;
+      }
+    }
+  }
   TRY(launch_check_any(w, s, true));
   const size_t E = (size_t)y->n * w->Kp;
   const int nb = (int)std::min<size_t>((E + 255) / 256, (size_t)num_sms() * 16);
@@ -1862,7 +1882,7 @@ static int solve_batched(const dpf_ybus* y, dpf_workspace* w, const dpf_batch* b
     // non-blocking poll of the active count, one interval behind
     if (pending && cudaEventQuery(ev) == cudaSuccess) {
       pending = false;
-      if (*w->h_n_active == 0) break;
+      if (w->h_n_active[0] == 0 || w->h_n_active[1]) break;
     }
     if (!pending) {
       cudaMemcpyAsync(w->h_n_active, w->n_active, 8, cudaMemcpyDeviceToHost, s);
@@ -1872,10 +1892,6 @@ static int solve_batched(const dpf_ybus* y, dpf_workspace* w, const dpf_batch* b
   }
   if (pending) cudaEventSynchronize(ev);
   cudaEventDestroy(ev);
-  if (rc == DPF_OK && w->grid.ok) {
-    int32_t act;
-    rc = dpf_active_count(w, &act, s);
-  }
   if (rc != DPF_OK) return rc;
   return dpf_solve_end(w, b, s);
 }

@@ -21,7 +21,8 @@
 //
 // The barrier needs every CTA resident (a cooperative launch: the driver
 // refuses what does not fit), and its wait gives up after a limit, sets an
-// error flag that the host reads with the active count, and the CTA returns.
+// error flag and the CTA returns, as later launches of the solve do at once; the
+// host reads the flag with the active count and at the solve's end.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,15 +41,15 @@ struct GridArgs {
   float* terms;           // [2][2][Kp] step and 1 / sqrt(1 - beta2^t), by iteration parity
   unsigned* suspect;      // [Kp]
   unsigned* bar;          // arrivals of this launch, whether a case is suspect (both zeroed)
-  int32_t* err;
+  int32_t* err;           // a barrier gave up (sticky for the solve)
+  long long polls;        // of a barrier before it gives up
 };
 
 constexpr int GRID_WARPS = 32;  // of a CTA at most
-constexpr long long GRID_SPIN = 1ll << 24;  // polls before a barrier gives up (seconds)
 
 // Grid barrier number `gen` (1, 2, ...): 0 if it gave up, else 1 + the word
 // beside the counter (whether any case is suspect).
-__device__ __forceinline__ int grid_barrier(unsigned* bar, unsigned gen, int32_t* err) {
+__device__ __forceinline__ int grid_barrier(unsigned* bar, unsigned gen, int32_t* err, long long polls) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -59,7 +60,7 @@ __device__ __forceinline__ int grid_barrier(unsigned* bar, unsigned gen, int32_t
     unsigned v;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-    } while (v < want && ++n < GRID_SPIN);
+    } while (v < want && ++n < polls);
     ok = v >= want ? 1 + (int)__ldcg(bar + 1) : 0;
     if (!ok) *err = 1;
     __threadfence();
@@ -145,6 +146,8 @@ __global__ void __launch_bounds__(GRID_WARPS * 32, 1) k_grid_resident(const Grid
   const unsigned Kp = (unsigned)a.Kp;
   const int kl = lane & (q.lanes - 1), rsub = lane / q.lanes, step = q.wpb * q.rpw;
   if (__ldcg(a.n_active) == 0) return;  // (the same for every CTA: nothing changes it before the first barrier)
+  // an earlier interval, or another CTA of this one, gave up: the state is lost
+  if (__syncthreads_or(threadIdx.x == 0 && __ldcg(q.err))) return;  // (one read: the whole CTA or none of it)
   const int tasks = q.vb_per_cta * q.wpb;
   // task -> its case, rows i0, i0 + step, ... < r1, and the cell of row 0
   struct Task {
@@ -256,7 +259,7 @@ __global__ void __launch_bounds__(GRID_WARPS * 32, 1) k_grid_resident(const Grid
         atomicOr(q.bar + 1, 1u);
       }
     }
-    const int passed = grid_barrier(q.bar, ++gen, q.err);
+    const int passed = grid_barrier(q.bar, ++gen, q.err, q.polls);
     if (!passed) return;
     const int par = it & 1;
     for (int t = warp, j = 0; work && t < tasks; t += nw, ++j) {  // ---- adjoint
@@ -325,7 +328,7 @@ __global__ void __launch_bounds__(GRID_WARPS * 32, 1) k_grid_resident(const Grid
       }
       sc.store(a.sc, k, lane);
     });
-    if (!grid_barrier(q.bar, ++gen, q.err)) return;
+    if (!grid_barrier(q.bar, ++gen, q.err, q.polls)) return;
   }
   for (int t = warp, j = 0; work && t < tasks; t += nw, ++j) {  // state out
     if (!((act0 >> j) & 1)) continue;
@@ -372,7 +375,8 @@ GridShape grid_shape(const dpf_ybus* y, int K, const LossOrder& lo, int lanes, s
 }
 
 int grid_launch(const IterArgs<float>& a, const GridShape& g, const LossOrder& lo, int lanes, int K, int n_it,
-                bool refined, float* terms, unsigned* suspect, unsigned* bar, int32_t* err, void* stream) {
+                bool refined, float* terms, unsigned* suspect, unsigned* bar, int32_t* err, int64_t polls,
+                void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   GridArgs q;
   q.a = a;
@@ -392,6 +396,7 @@ int grid_launch(const IterArgs<float>& a, const GridShape& g, const LossOrder& l
   q.suspect = suspect;
   q.bar = bar;
   q.err = err;
+  q.polls = polls;
   const bool adam = a.opt == OPT_ADAM;
   auto kern = refined ? (adam ? k_grid_resident<true, true> : k_grid_resident<true, false>)
                       : (adam ? k_grid_resident<false, true> : k_grid_resident<false, false>);

@@ -50,9 +50,11 @@ struct GridShape {
 };
 GridShape grid_shape(const dpf_ybus* y, int K, const LossOrder& lo, int lanes, size_t smem_limit);
 // terms: 4 Kp floats; suspect: Kp words, zero between launches; bar: two words;
-// err: set to 1 if a barrier gave up.  Returns a cudaError_t.
+// err: set to 1 if a barrier gave up after `polls`.  Returns a cudaError_t.
+constexpr int64_t GRID_POLLS = 1 << 20;  // of some 0.7 us: about a second
 int grid_launch(const IterArgs<float>& a, const GridShape& g, const LossOrder& lo, int lanes, int K, int n_it,
-                bool refined, float* terms, unsigned* suspect, unsigned* bar, int32_t* err, void* stream);
+                bool refined, float* terms, unsigned* suspect, unsigned* bar, int32_t* err, int64_t polls,
+                void* stream);
 
 // On-chip form of the DC solve (dpf_dc_resident.cu): every case of the batch
 // to its tolerance in one launch.

@@ -318,6 +318,11 @@ def dpf_grid_barrier_cost(ctas_per_sm: int = 4, reps: int = 1000, stream=None) -
     return us.value
 
 
+def dpf_wait_limit(ws: Workspace, polls: int = 0):
+    """Polls of a grid barrier before it gives up (0: the default)."""
+    _check(lib().dpf_wait_limit(ws.handle, int(polls)))
+
+
 def dpf_iterations_done(ws: Workspace) -> int:
     n = C.c_int32()
     _check(lib().dpf_iterations_done(ws.handle, C.byref(n)))
