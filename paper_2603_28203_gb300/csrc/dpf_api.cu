@@ -693,6 +693,7 @@ static Plan<R> make_plan(dpf_workspace* w) {
   s.beta2 = w->opts.beta2;
   s.factor = w->opts.factor;
   s.threshold = w->opts.threshold;
+  s.keep = (float)(1.0 - w->opts.threshold);
   s.min_lr = w->opts.min_lr;
   s.gamma = w->opts.gamma;
   s.lr0 = w->opts.lr;

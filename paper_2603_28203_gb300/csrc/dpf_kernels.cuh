@@ -519,6 +519,7 @@ template <class R> struct SchedArgs {
   R* isbc2;
   int32_t* n_active;
   double inv_m, beta1, beta2, factor, threshold, min_lr, gamma, lr0;
+  float keep;  // 1 - threshold
   int sched, patience, cooldown, step_every, opt;
 };
 

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "dpf_kernels.cuh"
+#include "dpf_plateau.h"
 
 namespace dpf {
 
@@ -10,12 +11,11 @@ namespace dpf {
 // same decisions and values as sched_case).  FP64 issue is dear on GB300, so
 // in FP32 solves a step takes two FP64 operations: lane 0 carries beta1^t,
 // lane 1 beta2^t; the plateau test compares the FP32 loss sums and falls back
-// to the FP64 comparison only where they are within 1e-6 of the threshold;
-// the step schedule's power is taken when its exponent changes.
+// to the FP64 comparison only near the threshold (dpf_plateau.h); the step schedule's power is taken when its exponent changes.
 template <class R> struct ResSched {
   double lr, best, bt;    // bt: lane 0 beta1^t, lane 1 beta2^t
   float bsum;             // FP32: the loss sum behind `best` (< 0: best as loaded)
-  float tsum;             // FP32: bsum (1 - threshold), approximately (< 0: not usable)
+  float tsum;             // FP32: the bar of the next improvement (plateau_bar)
   R lrw;                  // lr in working precision
   int bad, cool, it;
   R step, isb;            // of the update numbered it + 1
@@ -44,10 +44,8 @@ template <class R> struct ResSched {
   // the decision of sched_case on this iterate's loss
   __device__ __forceinline__ bool improved(const SchedArgs<R>& s, R lsum) {
     if constexpr (sizeof(R) == 4) {
-      if (tsum > 1e-30f) {
-        if (lsum < tsum * (1.f - 1e-6f)) return true;
-        if (lsum > tsum * (1.f + 1e-6f)) return false;
-      }
+      const int side = plateau_side(lsum, tsum);
+      if (side) return side > 0;
       if (bsum >= 0.f) best = (double)bsum * s.inv_m;
     }
     return (double)lsum * s.inv_m < best * (1.0 - s.threshold);
@@ -58,8 +56,7 @@ template <class R> struct ResSched {
       if (improved(s, lsum)) {
         if constexpr (sizeof(R) == 4) {
           bsum = lsum;
-          const float f = 1.f - (float)s.threshold;
-          tsum = f > 1e-3f ? lsum * f : -1.f;
+          tsum = plateau_bar(lsum, s.keep);
         } else {
           best = (double)lsum * s.inv_m;
         }
