@@ -878,16 +878,30 @@ static int launch_span(dpf_workspace* w, cudaStream_t s, int n, bool with_check)
     if (with_check) TRY(launch_check_any(w, s, false));
     return launch_resident(w, s, n);
   }
-  if (w->grid.ok && !w->profile) {
-    if (with_check) TRY(launch_check_any(w, s, false));
-    CK((cudaError_t)grid_launch(make_plan<float>(w).it, w->grid, w->res_lo, w->lanes, w->K, n,
-                                w->precision == DPF_FP32R, w->grid_terms, w->grid_sus, w->grid_bar, w->n_active + 1,
-                                w->grid_polls, s));
-    w->launches++;
-    return DPF_OK;
+  int rc = DPF_OK;
+  auto streaming = [&] {
+    for (int i = 0; i < n && rc == DPF_OK; ++i) rc = launch_iteration_any(w, s, with_check && i == 0);
+    return cudaSuccess;
+  };
+  if (!w->grid.ok || w->profile) {
+    streaming();
+    return rc;
   }
-  for (int i = 0; i < n; ++i) TRY(launch_iteration_any(w, s, with_check && i == 0));
-  return DPF_OK;
+  if (with_check) TRY(launch_check_any(w, s, false));
+  with_check = false;
+  CK((cudaError_t)whole_or_streaming(
+      w->grid,
+      [&] {
+        w->launches++;
+        return grid_launch(make_plan<float>(w).it, w->grid, w->res_lo, w->lanes, w->K, n, w->precision == DPF_FP32R,
+                           w->grid_terms, w->grid_sus, w->grid_bar, w->n_active + 1, w->grid_polls, s);
+      },
+      [&] {
+        w->launches--;
+        cudaGetLastError();
+      },
+      streaming));
+  return rc;
 }
 
 // Capture one check interval (FP64 test + check_every iterations) as a graph.

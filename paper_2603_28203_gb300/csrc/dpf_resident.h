@@ -56,6 +56,25 @@ int grid_launch(const IterArgs<float>& a, const GridShape& g, const LossOrder& l
                 bool refined, float* terms, unsigned* suspect, unsigned* bar, int32_t* err, int64_t polls,
                 void* stream);
 
+// One interval of a solve with a whole-GPU shape: by `whole`, or by `streaming`
+// (for good) where the driver refuses the cooperative launch.  grid_shape
+// counts the device's SMs, of which a context or stream may have fewer (MPS, a
+// green context); nothing of the interval has run when it is refused.  Both
+// return a cudaError_t, `refused` clears the runtime's last error.
+inline bool launch_refused(int e) {
+  return e == 720 || e == 701 || e == 801;  // too large to be resident, out of resources, not supported
+}
+template <class Whole, class Cleared, class Streaming>
+int whole_or_streaming(GridShape& g, Whole whole, Cleared refused, Streaming streaming) {
+  if (g.ok) {
+    const int e = whole();
+    if (!launch_refused(e)) return e;
+    refused();
+    g = GridShape();
+  }
+  return streaming();
+}
+
 // On-chip form of the DC solve (dpf_dc_resident.cu): every case of the batch
 // to its tolerance in one launch.
 struct DcRes {
