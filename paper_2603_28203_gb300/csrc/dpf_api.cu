@@ -14,6 +14,7 @@
 #include "dpf_kernels.cuh"
 #include "dpf_dc.cuh"
 #include "dpf_resident.h"
+#include "dpf_smem.h"
 
 using namespace dpf;
 
@@ -1149,19 +1150,17 @@ static int upload_windows(dpf_workspace* w, cudaStream_t s) {
 
 template <class R>
 static int set_smem_attr(int bytes) {
-  if (bytes > 48 * 1024) {
-    CK(cudaFuncSetAttribute(k_fwd<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    CK(cudaFuncSetAttribute(k_adj<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    if constexpr (sizeof(R) == 4) {
-      CK(cudaFuncSetAttribute(k_fwd2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-      CK(cudaFuncSetAttribute(k_adj2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-      CK(cudaFuncSetAttribute(k_fwd2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-      CK(cudaFuncSetAttribute(k_adj2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-      CK(cudaFuncSetAttribute(k_fwd<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-      CK(cudaFuncSetAttribute(k_adj<float, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-      CK(cudaFuncSetAttribute(k_fwd_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-      CK(cudaFuncSetAttribute(k_adj<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    }
+  CK(allow_smem(k_fwd<R>, bytes));
+  CK(allow_smem(k_adj<R>, bytes));
+  if constexpr (sizeof(R) == 4) {
+    CK(allow_smem(k_fwd2<false>, bytes));
+    CK(allow_smem(k_adj2<false>, bytes));
+    CK(allow_smem(k_fwd2<true>, bytes));
+    CK(allow_smem(k_adj2<true>, bytes));
+    CK(allow_smem(k_fwd<float, true>, bytes));
+    CK(allow_smem(k_adj<float, false, true>, bytes));
+    CK(allow_smem(k_fwd_mixed, bytes));
+    CK(allow_smem(k_adj<float, true>, bytes));
   }
   return DPF_OK;
 }

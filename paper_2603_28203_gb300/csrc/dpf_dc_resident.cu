@@ -26,6 +26,7 @@
 
 #include "dpf_dc.cuh"
 #include "dpf_resident.h"
+#include "dpf_smem.h"
 
 namespace dpf {
 
@@ -362,7 +363,7 @@ static int dc_res_t(const dpf_ybus* y, const DcRes& c, const DcShape& sh, cudaSt
   constexpr int many = dc_many<T>();
   q.T_ = sh.T;
   auto kern = sh.rpt == many ? k_dc_resident<T, many> : k_dc_resident<T, 2>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
+  cudaError_t e = allow_smem(kern, sh.smem);
   if (e != cudaSuccess) return e;
   kern<<<c.K, q.T_, sh.smem, s>>>(q);
   return cudaGetLastError();

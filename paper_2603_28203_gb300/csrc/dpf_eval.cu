@@ -24,6 +24,7 @@
 #include "dpf_kernels.cuh"
 #include "dpf_resident.h"
 #include "dpf_sell.cuh"
+#include "dpf_smem.h"
 
 namespace dpf {
 
@@ -307,7 +308,7 @@ static int eval_t(const dpf_ybus* y, const EvalCall& c, cudaStream_t s) {
   q.v64 = q.m + (bwd ? np * (unsigned)sizeof(R) : 0u);
   const size_t smem = q.v64 + (loss && sizeof(R) == 4 ? np * 16u : 0u);
   auto kern = !bwd ? k_eval_case<R, false, false> : loss ? k_eval_case<R, true, true> : k_eval_case<R, true, false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);

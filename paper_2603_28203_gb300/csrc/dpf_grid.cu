@@ -30,6 +30,7 @@
 #include "dpf_kernels.cuh"
 #include "dpf_resident.h"
 #include "dpf_sched.cuh"
+#include "dpf_smem.h"
 
 namespace dpf {
 
@@ -400,7 +401,7 @@ int grid_launch(const IterArgs<float>& a, const GridShape& g, const LossOrder& l
   const bool adam = a.opt == OPT_ADAM;
   auto kern = refined ? (adam ? k_grid_resident<true, true> : k_grid_resident<true, false>)
                       : (adam ? k_grid_resident<false, true> : k_grid_resident<false, false>);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+  cudaError_t e = allow_smem(kern, g.smem);
   if (e == cudaSuccess) e = cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};

@@ -33,6 +33,7 @@
 
 #include "dpf_internal.h"
 #include "dpf_nr.h"
+#include "dpf_smem.h"
 
 using namespace dpf;
 
@@ -1259,7 +1260,7 @@ extern "C" int dpf_nr_stats(const dpf_nr* h, int64_t* n_pos, int64_t* n_pairs, i
 // CTAs of the shared-memory form an SM holds.
 template <class T>
 static int smem_ctas(int threads, size_t bytes, int* n) {
-  CK(cudaFuncSetAttribute(k_nr_lu_smem<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  CK(allow_smem(k_nr_lu_smem<T>, bytes));
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_nr_lu_smem<T>, threads, bytes));
   return DPF_OK;
 }

@@ -39,6 +39,7 @@
 #include "dpf_resident.h"
 #include "dpf_sched.cuh"
 #include "dpf_sell.cuh"
+#include "dpf_smem.h"
 
 namespace dpf {
 
@@ -571,7 +572,7 @@ ResShape res_shape(const dpf_ybus* y, int K, bool fp64, bool refined, const Loss
 template <class R>
 static cudaError_t res_go(void (*kern)(const ResArgs<R>), const ResArgs<R>& q, const ResShape& sh, bool pdl,
                           cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
+  cudaError_t e = allow_smem(kern, sh.smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(sh.warp ? (q.K + RES_TEAMS - 1) / RES_TEAMS : q.K);
