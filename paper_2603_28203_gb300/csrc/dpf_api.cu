@@ -872,10 +872,15 @@ static int launch_check_any(dpf_workspace* w, cudaStream_t s, bool final_pass) {
                                   : launch_check<float>(w, s, final_pass);
 }
 
-// n iterations, the FP64 test first if with_check; on chip where the grid fits
-// (not while the forward and adjoint passes are timed one by one).
+// Whether a launch of n iterations runs on chip, or on the whole GPU (not while
+// the forward and adjoint passes are timed one by one).
+static bool span_on_chip(const dpf_workspace* w, int n) { return w->res.ok && !w->profile && n >= w->res.min_span; }
+static bool span_whole_gpu(const dpf_workspace* w, int n) { return w->grid.ok && !w->profile && n >= w->grid.min_span; }
+
+// n iterations, the FP64 test first if with_check.  The forms keep the same
+// state between launches, so a solve may go from one to the other.
 static int launch_span(dpf_workspace* w, cudaStream_t s, int n, bool with_check) {
-  if (w->res.ok && !w->profile) {
+  if (span_on_chip(w, n)) {
     if (with_check) TRY(launch_check_any(w, s, false));
     return launch_resident(w, s, n);
   }
@@ -884,7 +889,7 @@ static int launch_span(dpf_workspace* w, cudaStream_t s, int n, bool with_check)
     for (int i = 0; i < n && rc == DPF_OK; ++i) rc = launch_iteration_any(w, s, with_check && i == 0);
     return cudaSuccess;
   };
-  if (!w->grid.ok || w->profile) {
+  if (!span_whole_gpu(w, n)) {
     streaming();
     return rc;
   }
@@ -1659,7 +1664,7 @@ extern "C" int dpf_solve_iterate(dpf_workspace* w, int32_t n_iter, void* stream)
   n_iter = std::min(n_iter, w->opts.max_iter - w->t_done);
   const int ce = w->opts.check_every;
   while (n_iter > 0) {
-    if (w->opts.use_graph && !w->profile && !w->grid.ok && w->t_done % ce == 0 && n_iter >= ce) {
+    if (w->opts.use_graph && !w->profile && !span_whole_gpu(w, ce) && w->t_done % ce == 0 && n_iter >= ce) {
       if (!w->gexec) TRY(build_graph(w));
       CK(cudaGraphLaunch(w->gexec, s));
       w->launches += w->graph_kernels;
@@ -2037,7 +2042,7 @@ extern "C" int dpf_autotune(const dpf_ybus* y, dpf_workspace* w, const dpf_batch
   // a grid whose iterations run on chip has one shape (the options below only
   // give the order of its loss sum): nothing to time
   TRY(dpf_solve_begin(y, w, b, &base, s));
-  if (w->res.ok) {
+  if (w->res.ok && base.check_every >= w->res.min_span) {
     w->begun = false;
     o->lanes = auto_lanes;
     o->warps = 8;

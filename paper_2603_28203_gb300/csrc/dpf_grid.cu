@@ -371,6 +371,7 @@ GridShape grid_shape(const dpf_ybus* y, int K, const LossOrder& lo, int lanes, s
   const long long bytes = (long long)g.vb * lanes * ((long long)lo.rpb * 32 + lo.wpb * 4);
   if (bytes > (long long)smem_limit - 1024) return g;  // (the barrier's flag)
   g.smem = (size_t)bytes;
+  g.min_span = grid_min_span(K);
   g.ok = true;
   return g;
 }

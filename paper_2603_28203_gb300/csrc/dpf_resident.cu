@@ -561,6 +561,7 @@ ResShape res_shape(const dpf_ybus* y, int K, bool fp64, bool refined, const Loss
   // 1x30 1,169 330; 3000x30 1,330 486; 1x2000 1,234 732; 3000x2000 17,719
   // 12,700; 3000x300 3,216 2,071; 3000x1000 8,710 5,938.
   if (fp64 && n > RES_WARP_N && (n > 320 || K > 300)) return sh;
+  sh.min_span = res_min_span(n, K, fp64, refined);
   sh.warp = n <= RES_WARP_N;
   sh.rpt = sh.warp && n <= 32 ? 1 : 2;
   sh.T = sh.warp ? 32 : ((n + 1) / 2 + 31) / 32 * 32;

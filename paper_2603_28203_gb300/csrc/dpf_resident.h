@@ -20,8 +20,30 @@ struct ResShape {
   bool warp = false;  // one warp per case
   int rpt = 1;        // rows per thread
   int T = 32;         // compute threads per case
+  int min_span = 1;   // fewest iterations of a launch that pay
   size_t smem = 0;
 };
+
+// A launch loads and stores every case's state in strided 8- and 16-byte
+// pieces, which the iterations between have to earn: with tests (or the
+// caller's steps) closer than this the streaming kernels are faster.  Time of
+// 48 iterations, streaming / on chip, by the iterations per launch:
+//   FP32R  2,000 x 2,379  2: 8.1 / 18.7 ms  6: 7.9 / 9.6   10: 7.9 / 7.8
+//          2,000 x 600    2: 2.6 / 5.0      6: 2.4 / 2.6    8: 2.4 / 2.3
+//          300 x 3,000    2: 2.1 / 2.8      4: 2.0 / 1.9
+//          2,000 x 1      2: 0.87 / 0.91
+//   FP32   2,000 x 2,379  2: 7.7 / 11.4     4: 7.6 / 8.1    6: faster
+//          2,000 x 600    2: 2.5 / 3.1      4: 2.3 / 2.3
+//          100 x 2,000    2: 1.08 / 1.20    3: 0.98 / 0.97
+//          30 x 8,192     1: 1.6 / 1.8 ms
+inline int res_min_span(int n, int K, bool fp64, bool refined) {
+  const long long e = (long long)n * K;
+  if (fp64) return n > 256 && K > 100 ? 3 : 1;  // 300 x 152, 2: 4.0 / 4.2 ms
+  if (n <= RES_WARP_N) return e > 100000 ? 2 : 1;
+  if (K <= 300 && n <= 512) return 1;
+  if (refined) return e <= 250000 ? 3 : e <= 1000000 ? 4 : e <= 1300000 ? 8 : 10;
+  return K <= 300 ? 2 : e <= 250000 ? 3 : e <= 1300000 ? 4 : 6;
+}
 
 // The order in which the streaming kernels of the same options sum a case's
 // loss (row blocks, warps, rows per warp), which the on-chip form repeats.
@@ -46,8 +68,14 @@ struct GridShape {
   int ctas = 0, warps = 0, workers = 0;
   int gx = 0;   // case tiles that hold cases
   int vb = 0;   // virtual blocks (case tile x row block) per CTA
+  int min_span = 1;  // fewest iterations of a launch that pay
   size_t smem = 0;
 };
+// The same for the whole-GPU form: a launch costs some 2.6 us plus 0.2 us per
+// case (the schedulers' state) more than an iteration streaming.  48
+// iterations, FP32: 2,500 x 64, 4: 1.09 / 1.29 ms, 12: 1.06 / 1.08; 2,500 x 20,
+// 4: 0.94 / 1.03, 8: 0.89 / 0.91; 10,000 x 16, 1: 1.51 / 1.72, 2: 1.28 / 1.26.
+inline int grid_min_span(int K) { return 2 + K / 5; }
 GridShape grid_shape(const dpf_ybus* y, int K, const LossOrder& lo, int lanes, size_t smem_limit);
 // terms: 4 Kp floats; suspect: Kp words, zero between launches; bar: two words;
 // err: set to 1 if a barrier gave up after `polls`.  Returns a cudaError_t.
