@@ -275,7 +275,8 @@ int dpf_solve_iterate(dpf_workspace* ws, int32_t n_iter, void* stream);
 /* Grids of up to 2,048 buses iterate on chip (a case's state stays in one SM
  * for a whole check interval), a few cases of a larger grid in one kernel over
  * the whole GPU, unless plain, stage_v or stage_y is set or the precision is
- * DPF_MIXED; FP64 only up to 64 buses, or 320 buses and 300 cases.  A few
+ * DPF_MIXED; FP64 only up to 320 buses and a few hundred to a few thousand
+ * cases.  A few
  * iterations between two tests (or a short dpf_solve_iterate) run in the
  * two-pass kernels where that is faster.  Results
  * are those of the two-pass kernels (FP32, FP32R: to the bit; lanes, warps,

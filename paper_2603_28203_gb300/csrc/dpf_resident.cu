@@ -552,15 +552,10 @@ ResShape res_shape(const dpf_ybus* y, int K, bool fp64, bool refined, const Loss
   const DeviceYbus& d = y->dev;
   const int n = y->n;
   if (!d.res_rord || n > RES_MAX_N || y->m_loss <= 0) return sh;
-  // FP64 is bound by the FP64 pipe: the streaming kernels spread a case over
-  // many SMs, so the on-chip form pays only where an iteration is mostly
-  // latency.  Microseconds per 100 iterations (streaming, on chip), cases x
-  // buses: 1x30 1,920 982; 3000x30 4,256 4,017; 1x300 2,316 1,883; 150x300
-  // 3,471 1,886; but 1000x300 11,344 12,548; 1x700 2,454 3,500.  In FP32 it is
-  // faster over the whole range measured (30-2,048 buses, 1-3,000 cases):
-  // 1x30 1,169 330; 3000x30 1,330 486; 1x2000 1,234 732; 3000x2000 17,719
-  // 12,700; 3000x300 3,216 2,071; 3000x1000 8,710 5,938.
-  if (fp64 && n > RES_WARP_N && (n > 320 || K > 300)) return sh;
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (!res_pays(n, K, fp64, sms)) return sh;
   sh.min_span = res_min_span(n, K, fp64, refined);
   sh.warp = n <= RES_WARP_N;
   sh.rpt = sh.warp && n <= 32 ? 1 : 2;

@@ -24,6 +24,34 @@ struct ResShape {
   size_t smem = 0;
 };
 
+// Whether K cases of n buses are few (or wide) enough for the on-chip form.
+// FP64 is bound by the FP64 pipe, which the streaming kernels keep busy with
+// live rows only, while here a warp of 32 or 64 rows costs the same whatever it
+// holds: the form pays where an iteration is mostly latency.  100 iterations,
+// tests every 25, streaming / on chip in ms (152 SMs: 4 cases per CTA, 3 CTAs
+// per SM, so 608 cases are one CTA per SM and 1,824 a full wave):
+//   one row per lane    9 x 3,000 2.8 / 4.1  14 x 1,824 2.8 / 3.3  24 x 3,000
+//     4.0 / 4.1; but 30 x 1,500 3.1 / 2.4, 30 x 5,000 7.3 / 7.0, 30 x 8,000 9.1 / 10.7
+//   two rows            33 x 600 2.5 / 1.6, 33 x 1,216 3.1 / 3.8, 33 x 8,000 10.4 /
+//     16.9; 64 x 900 3.8 / 2.9, 64 x 1,216 3.9 / 4.3, 64 x 1,824 5.6 / 4.4, 64 x
+//     2,400 6.3 / 7.1, 64 x 3,000 7.9 / 7.1, 64 x 4,000 9.8 / 11.2
+//   one CTA per case    1 x 30 1.9 / 1.0, 1 x 300 2.3 / 1.9, 150 x 300 3.5 / 1.9,
+//     300 x 320 5.4 / 3.3; but 1,000 x 300 11.3 / 12.5, 1 x 700 2.5 / 3.5
+// FP32 pays over the whole range (1 x 30 1.2 / 0.33, 3,000 x 2,000 17.7 / 12.7)
+// but for very many cases of a grid that half fills its rows: 50 iterations,
+// 14 x 100,000 3.3 / 4.1, 33 x 50,000 3.2 / 3.4, 65 x 20,000 2.7 / 2.8.
+inline bool res_pays(int n, long long K, bool fp64, int sms) {
+  if (!fp64) {
+    const int rows = n <= 32 ? 32 : n <= RES_WARP_N ? 64 : (n + 63) / 64 * 64;
+    return 100 * n >= 55 * rows || K <= (n <= RES_WARP_N ? 32768 : 16384);
+  }
+  if (n > RES_WARP_N) return n <= 320 && K <= 300;
+  const long long wave = 12ll * sms;
+  if (n <= 32) return K <= 8 * sms || (n >= 28 && K <= 3 * wave);
+  return K <= 4 * sms || (n >= 48 && K <= 7 * sms) ||
+         (K <= 2 * wave && 100 * n * K >= 78 * 64 * wave * ((K + wave - 1) / wave));
+}
+
 // A launch loads and stores every case's state in strided 8- and 16-byte
 // pieces, which the iterations between have to earn: with tests (or the
 // caller's steps) closer than this the streaming kernels are faster.  Time of

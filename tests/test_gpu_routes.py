@@ -92,3 +92,18 @@ def test_few_cases_keep_the_on_chip_form_for_single_steps():
     y = dpf.dpf_build_ybus(_grid(300))
     _, launches = _solve(y, 20, dpf.FP32, 20, [20, 1, 1, 1])
     assert launches[2:] == [1, 1]
+
+
+# the ends of the ranges in which whole warps of FP64 rows pay on 152 SMs, and
+# FP32 batches that half fill their rows
+@pytest.mark.parametrize("n,K,precision,chip", [
+    (14, 1216, "FP64", True), (14, 1217, "FP64", False), (30, 5000, "FP64", True), (30, 8000, "FP64", False),
+    (33, 608, "FP64", True), (33, 609, "FP64", False), (64, 1000, "FP64", True), (64, 1216, "FP64", False),
+    (64, 1824, "FP64", True), (64, 2400, "FP64", False), (300, 300, "FP64", True), (300, 301, "FP64", False),
+    (14, 32768, "FP32", True), (14, 32769, "FP32", False), (30, 40000, "FP32", True), (65, 16385, "FP32R", False)])
+def test_many_cases_of_narrow_grids_run_streaming(n, K, precision, chip):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the limits count 152 SMs")
+    y = dpf.dpf_build_ybus(_grid(n))
+    _, launches = _solve(y, K, getattr(dpf, precision), 20, [20, 20])
+    assert all((k <= 6) == chip for k in launches), launches
