@@ -1345,15 +1345,8 @@ extern "C" int dpf_nr_solve(dpf_nr* h, const dpf_batch* b, const dpf_nr_opts* o,
   a.C = lanes_for(K);
   // The shared-memory form where one case's factor fits and the cases still
   // iterating are few: it takes a case in the least time, the global form the
-  // most cases at a time (it hides one case's latency behind others).  Both
-  // give the same bits; o->lanes > 0 forces the global form.  Whole solve in
-  // ms by waves of CTAs, shared-memory and global form: FP32, 2,000 buses, 1
-  // case 1.0 / 1.9, 300 (2 waves) 2.3 / 4.3, 850 (6) 6.2 / 7.5, 2,379 (16)
-  // 17.1 / 12.8; 1,000 buses, 300 (2) 1.6 / 3.1, 2,000 (14) 8.8 / 7.0; 300
-  // buses, 300 (1) 1.1 / 2.0, 3,000 (7) 4.0 / 4.0; 118, 3,000 (4) 1.35 /
-  // 1.52.  FP64, one wave: 30 buses, 1 case 1.2 / 1.4; 118, 500 1.0 / 1.3; 300,
-  // 300 2.3 / 3.7; 1,000, 120 2.9 / 5.0; but 30 buses, 1,500 (10 CTAs an SM) 2.1
-  // / 1.7 and 118, 3,000 3.5 / 2.7: a few CTAs keep the FP64 pipe busy.
+  // most cases at a time (it hides one case's latency behind others; nr_smem_cases).
+  // Both give the same bits; o->lanes > 0 forces the global form.
   const size_t need = precision == DPF_FP64 ? lu_smem_bytes<double>(sym.row_ptr[sym.n], y->n, h->chunk_units, h->n_chunk)
                                             : lu_smem_bytes<float>(sym.row_ptr[sym.n], y->n, h->chunk_units, h->n_chunk);
   const bool fits = o->lanes == 0 && h->sstream && need <= smem_optin();
@@ -1362,7 +1355,7 @@ extern "C" int dpf_nr_solve(dpf_nr* h, const dpf_batch* b, const dpf_nr_opts* o,
     int per_sm = 0;
     if (precision == DPF_FP64) TRY(smem_ctas<double>(h->smem_threads, need, &per_sm));
     else TRY(smem_ctas<float>(h->smem_threads, need, &per_sm));
-    smem_cases = num_sms_nr() * (precision == DPF_FP64 ? std::min(per_sm, 4) : per_sm * 6);
+    smem_cases = nr_smem_cases(y->n, precision == DPF_FP64, num_sms_nr(), per_sm);
   }
   a.va_slack = y->va_slack;
   a.tol = tol;

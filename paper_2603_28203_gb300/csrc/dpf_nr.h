@@ -54,4 +54,28 @@ struct NrSymbolic {
 // DPF_E_UNSUPPORTED when the update lists would exceed `max_pairs`.
 int nr_symbolic(const dpf_ybus* y, int64_t max_pairs, NrSymbolic* s);
 
+// Most cases the shared-memory form of the factor takes (per_sm: its CTAs an SM
+// holds).  Its time grows by waves of CTAs, each about one case's latency; the
+// global form's hardly grows until it fills the GPU, the sooner the smaller the
+// grid's factor.  Whole N-1 solve in us, shared-memory / global, by cases:
+//   FP32   30 buses (10 an SM)  1,216 482 / 548    2,432 634 / 599
+//          64 (9)      1,216 538 / 702    2,432 738 / 751
+//          118 (5)     1,216 753 / 793    1,824 962 / 871    2,432 1172 / 938
+//          200 (4)     1,216 1187 / 1386  1,824 1566 / 1508
+//          256 (4)     1,824 1675 / 1850  2,432 2051 / 2072
+//          300 (2)     912 1227 / 1281    1,216 1514 / 1341  1,824 2133 / 1604
+//          450 (2)     912 2118 / 2110    1,216 2711 / 2327
+//          600 (2)     1,216 2570 / 2642  1,520 3130 / 2981
+//          800 (2)     1,520 5182 / 6275  1,824 6036 / 6663
+//          2,000 (1)   300 2300 / 4300    850 6200 / 7500    2,379 17100 / 12800
+//   FP64   one wave of a few CTAs keeps its pipe busy: 30 buses, 1 case 1.2 / 1.4
+//          ms; 118, 500 1.0 / 1.3; 300, 300 2.3 / 3.7; 1,000, 120 2.9 / 5.0; but
+//          30, 1,500 (10 CTAs an SM) 2.1 / 1.7 and 118, 3,000 3.5 / 2.7
+inline int nr_smem_cases(int n, bool fp64, int sms, int per_sm) {
+  if (fp64) return sms * (per_sm < 4 ? per_sm : 4);
+  if (per_sm >= 9) return sms * per_sm * 27 / 20;
+  const int waves = per_sm >= 3 ? (n < 240 ? 2 : 3) : per_sm == 1 ? 6 : n < 500 ? 3 : n < 750 ? 4 : 5;
+  return sms * per_sm * waves;
+}
+
 }  // namespace dpf

@@ -107,3 +107,26 @@ def test_many_cases_of_narrow_grids_run_streaming(n, K, precision, chip):
     y = dpf.dpf_build_ybus(_grid(n))
     _, launches = _solve(y, K, getattr(dpf, precision), 20, [20, 20])
     assert all((k <= 6) == chip for k in launches), launches
+
+
+# Newton, FP32: CTAs of the shared-memory factor on 152 SMs (10, 5, 4, 4, 2, 2 an SM)
+# in as many waves as pay; one case more goes to the global form
+@pytest.mark.parametrize("n,most", [(30, 152 * 10 * 27 // 20), (118, 152 * 5 * 2), (200, 152 * 4 * 2),
+                                    (256, 152 * 4 * 3), (300, 152 * 2 * 3), (600, 152 * 2 * 4)])
+def test_newton_factor_leaves_shared_memory_with_many_cases(n, most):
+    """A step in shared memory is two launches shorter than the global form
+    (assembly and update are part of it)."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the limits count 152 SMs")
+    y = dpf.dpf_build_ybus(_grid(n))
+    for K, chip in ((most, True), (most + 1, False)):
+        nr = dpf.dpf_nr_create(y, K)
+        out = {k: torch.ones((K, n), dtype=torch.float64, device=DEV) for k in ("va", "vm")}
+        count, va = [], []
+        for lanes in (0, 8):
+            before = nr.stats()["launches"]
+            dpf.dpf_nr_solve(nr, precision=dpf.FP32, tol=1e-9, max_iter=1, n_case=K, lanes=lanes, **out)
+            count.append(nr.stats()["launches"] - before)
+            va.append(out["va"].clone())
+        assert count[1] - count[0] == (2 if chip else 0)
+        assert torch.equal(va[0], va[1])
