@@ -266,6 +266,7 @@ extern "C" int dpf_ybus_upload(dpf_ybus* y, void* stream) {
     add(&d.res_slot, sell.slot);
     d.res_slices = (int)sell.soff.size() - 1;
     d.res_pairs = sell.soff.back();
+    d.res_longest = sell.soff[1];
   }
   add(&d.ent32, ent);
   add(&d.row_ptr, y->irow_ptr);

@@ -507,6 +507,12 @@ __global__ void __launch_bounds__(res_threads<R>(), 1) k_resident_cta(const ResA
 }
 
 // ---- host ---------------------------------------------------------------------
+// Threads of a CTA for T compute threads: a warp of its own for the scheduler,
+// unless that would leave room for one CTA per SM instead of two.
+template <class R> static int res_cta_threads(int T) {
+  return T <= 512 && T + 32 > 512 ? T : std::min(T + 32, res_threads<R>());
+}
+
 static LossGeo loss_geo(const LossOrder& lo) {
   LossGeo g;
   g.gy = lo.gy;
@@ -561,7 +567,15 @@ ResShape res_shape(const dpf_ybus* y, int K, bool fp64, bool refined, const Loss
   sh.rpt = sh.warp && n <= 32 ? 1 : 2;
   sh.T = sh.warp ? 32 : ((n + 1) / 2 + 31) / 32 * 32;
   sh.smem = fp64 ? res_layout<double>(y, sh, refined, lo).total : res_layout<float>(y, sh, refined, lo).total;
-  sh.ok = sh.smem <= smem_limit;
+  if (sh.smem > smem_limit) return sh;
+  int ctas = 1, ctas_free = 1;
+  if (!sh.warp && !fp64) {  // CTAs an SM holds by shared memory, and by its 65,536 registers (64 a thread)
+    int most = 0;
+    cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    ctas = std::max(1, most / (int)(sh.smem + 1024));
+    ctas_free = 1024 / res_cta_threads<float>(sh.T);
+  }
+  sh.ok = res_pays_dense(n, K, fp64, sms, d.res_pairs, d.res_longest, ctas, ctas_free);
   return sh;
 }
 
@@ -572,10 +586,7 @@ static cudaError_t res_go(void (*kern)(const ResArgs<R>), const ResArgs<R>& q, c
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(sh.warp ? (q.K + RES_TEAMS - 1) / RES_TEAMS : q.K);
-  // a warp of its own for the scheduler, unless that would leave room for one
-  // CTA per SM instead of two
-  const int threads = sh.T <= 512 && sh.T + 32 > 512 ? sh.T : std::min(sh.T + 32, res_threads<R>());
-  cfg.blockDim = dim3(sh.warp ? 32 * RES_TEAMS : threads);
+  cfg.blockDim = dim3(sh.warp ? 32 * RES_TEAMS : res_cta_threads<R>(sh.T));
   cfg.dynamicSmemBytes = sh.smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];

@@ -52,6 +52,26 @@ inline bool res_pays(int n, long long K, bool fp64, int sms) {
          (K <= 2 * wave && 100 * n * K >= 78 * 64 * wave * ((K + wave - 1) / wave));
 }
 
+// Whether K cases of a grid with long rows pay, from its sliced form (entry
+// pairs in all slices, in the longest one).  FP32: where the staged matrix, not
+// the threads, limits the CTAs of an SM (ctas < ctas_free), by the padded
+// entries per row times the waves of CTAs (beyond some 16 both forms grow
+// alike).  50 iterations, streaming / on chip in ms: 1,000 buses + 2,000
+// branches x 2,400 (134) 4.5 / 4.4, 300 + 4,800 x 600 (156) 1.5 / 1.4, x 1,000
+// (260) 1.8 / 2.2, 150 + 2,400 x 1,000 (133) 1.26 / 1.21, x 2,400 (316) 2.2 / 2.4,
+// 1,000 with a bus of 160 branches x 2,400 (150) 5.2 / 6.4; 100 iterations, 150
+// + 5,000 x 1,000 (507) 2.7 / 5.0, a star of 300 x 1,000 (224) 5.2 / 7.2.
+// FP64: a CTA's longest slice is one warp's chain, and padding costs the FP64
+// pipe: a star of 300 x 1 8.0 / 10.5, 60 + 1,400 x 1 4.0 / 4.4; but 300 with a bus
+// of 160 branches x 1 3.6 / 3.3, 150 + 2,400 x 1 2.1 / 1.9.
+inline bool res_pays_dense(int n, long long K, bool fp64, int sms, int pairs, int longest, int ctas, int ctas_free) {
+  const long long padded = 64ll * pairs;  // entries
+  if (fp64) return longest <= 100 && padded <= 50ll * n;
+  if (ctas >= ctas_free) return true;
+  const long long per_wave = (long long)sms * ctas;
+  return padded * (K < 16 * per_wave ? K : 16 * per_wave) <= 145 * per_wave * n;
+}
+
 // A launch loads and stores every case's state in strided 8- and 16-byte
 // pieces, which the iterations between have to earn: with tests (or the
 // caller's steps) closer than this the streaming kernels are faster.  Time of

@@ -80,3 +80,46 @@ def test_dc_of_a_dense_grid(name, tol, K):
                         p_spec=Pt, q_spec=torch.zeros_like(Pt), **res)
     for k in range(0, K, max(1, K // 5)):
         assert _residual(g, res["va"][k].cpu().numpy(), P[k]) <= bar, k
+
+
+def _hub(n, degree):
+    """make_grid with `degree` more branches at bus n // 2."""
+    g = gridgen.make_grid(n, 3, load_scale=0.05)
+    h = n // 2
+    near = {h, *g.t_bus[g.f_bus == h], *g.f_bus[g.t_bus == h]}
+    to = np.random.default_rng(0).permutation([i for i in range(n) if i not in near])[:degree]
+    new = dict(f_bus=np.full(degree, h), t_bus=to, r=np.full(degree, 0.05), x=np.full(degree, 0.3),
+               b_ch=np.zeros(degree), tap=np.ones(degree), shift=np.zeros(degree))
+    return dataclasses.replace(g, **{k: np.concatenate([getattr(g, k), v.astype(getattr(g, k).dtype)])
+                                     for k, v in new.items()})
+
+
+@pytest.mark.parametrize("name,K,precision,chip", [("300+4800", 500, "FP32", True), ("300+4800", 1000, "FP32", False),
+                                                   ("150+5000", 100, "FP32R", True), ("150+5000", 1000, "FP32R", False),
+                                                   ("star300", 1000, "FP32", False), ("hub", 2400, "FP32", False),
+                                                   ("hub", 1000, "FP32", True), ("star300", 1, "FP64", False),
+                                                   ("60+1400", 1, "FP64", False), ("60+1400", 1000, "FP32", True)])
+def test_iterations_of_dense_grids_run_where_they_are_faster(name, K, precision, chip):
+    """A span of 20 iterations is one launch on chip, 40 streaming; FP32 gives
+    the same bits either way."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the limits count 152 SMs")
+    g = _hub(1000, 160) if name == "hub" else _grid(name)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    opts = dpf.SolveOpts(precision=getattr(dpf, precision), max_iter=40, check_every=20, lr=1e-3, use_graph=0)
+    va = []
+    for streaming in (False, True):
+        out = dict(n_case=K, va=torch.zeros((K, g.n_bus), dtype=torch.float64, device=DEV),
+                   vm=torch.ones((K, g.n_bus), dtype=torch.float64, device=DEV))
+        dpf.dpf_profile_enable(ws, streaming)
+        dpf.dpf_solve_begin(y, ws, opts, **out)
+        before = dpf.dpf_kernel_launches(ws)
+        dpf.dpf_solve_iterate(ws, 20)
+        launches = dpf.dpf_kernel_launches(ws) - before
+        assert (launches <= 6) == (chip and not streaming), launches
+        dpf.dpf_solve_iterate(ws, 20)
+        dpf.dpf_solve_end(ws, **out)
+        va.append(out["va"])
+    if precision != "FP64":
+        assert torch.equal(va[0], va[1])
