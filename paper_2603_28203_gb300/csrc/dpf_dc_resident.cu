@@ -319,14 +319,20 @@ DcShape dc_res_shape(const dpf_ybus* y, int K, bool f32) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   // more cases than SMs: many rows per thread; else two, the shorter iteration
-  // (one case of 2,000 buses to 1e-10: 27.4 ms streaming, 3.9 ms)
-  sh.rpt = K > sms ? (f32 ? dc_many<float>() : dc_many<float2>()) : 2;
+  // (one case of 2,000 buses to 1e-10: 27.4 ms streaming, 3.9 ms), and for what
+  // one warp holds
+  sh.rpt = K > sms && y->n > 64 ? (f32 ? dc_many<float>() : dc_many<float2>()) : 2;
   sh.T = std::max(32, ((y->n + sh.rpt - 1) / sh.rpt + 31) / 32 * 32);
   const size_t v = f32 ? sizeof(float) : sizeof(float2);
   sh.smem = (size_t)d.res_pairs * 32 * (2 * v + 4) + (size_t)sh.T * sh.rpt * v;
   // B as sliced ELL is what may not fit: its slices are as long as their
   // longest row (a star of 700 buses takes 243 KB, a dense grid of 150 240 KB)
-  sh.ok = sh.smem + DC_STATIC_SMEM <= (size_t)lim;
+  if (sh.smem + DC_STATIC_SMEM > (size_t)lim) return sh;
+  int most = 0;
+  cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  const int ctas = std::max(1, most / (int)(sh.smem + DC_STATIC_SMEM + 1024));
+  const int ctas_free = std::max(1, std::min(32, (sh.rpt > 2 ? 512 : 1024) / sh.T));  // (128 or 64 registers a thread)
+  sh.ok = dc_pays(y->n, K, f32, sms, d.res_pairs, ctas, ctas_free);
   return sh;
 }
 

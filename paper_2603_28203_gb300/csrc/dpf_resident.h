@@ -163,7 +163,8 @@ struct DcRes {
   int32_t* iters;
 };
 // Launch shape for K cases (f32: FP32 vectors, else double-float); ok: the
-// grid has the sliced form and one case fits the shared memory of an SM.
+// grid has the sliced form, one case fits the shared memory of an SM and the
+// batch is faster on chip.
 struct DcShape {
   bool ok = false;
   int rpt = 2;  // rows per thread
@@ -171,6 +172,17 @@ struct DcShape {
   size_t smem = 0;
 };
 DcShape dc_res_shape(const dpf_ybus* y, int K, bool f32);
+// The same question as res_pays_dense for the DC solve (ms, streaming / on
+// chip).  To 1e-4, FP32: 1,000 buses + 8,000 branches x 1,000 (137) 0.81 / 0.71, x
+// 2,400 (329) 1.2 / 1.5, 1,000 + 16,000 x 600 (147) 0.69 / 0.51, x 1,000 (245) 0.83 /
+// 0.86, 300 + 10,000 x 1,000 (504) 0.57 / 0.64.  To 1e-10, double-float: 300 + 4,800
+// x 1,000 (260) 1.30 / 0.83, x 2,400 (623) 1.70 / 1.79, 150 + 5,000 x 1,000 (507)
+// 0.73 / 0.80, 1,000 + 8,000 x 2,400 (329) 3.4 / 2.3.
+inline bool dc_pays(int n, long long K, bool f32, int sms, int pairs, int ctas, int ctas_free) {
+  if (ctas >= ctas_free) return true;
+  const long long per_wave = (long long)sms * ctas;
+  return 64ll * pairs * (K < 16 * per_wave ? K : 16 * per_wave) <= (f32 ? 225 : 450) * per_wave * n;
+}
 // Returns a cudaError_t.
 int dc_res_launch(const dpf_ybus* y, const DcRes& c, const DcShape& sh, bool f32, void* stream);
 

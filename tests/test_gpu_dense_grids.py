@@ -123,3 +123,39 @@ def test_iterations_of_dense_grids_run_where_they_are_faster(name, K, precision,
         va.append(out["va"])
     if precision != "FP64":
         assert torch.equal(va[0], va[1])
+
+
+@pytest.mark.parametrize("name,K,tol,chip", [("1000+8000", 1000, 1e-4, True), ("1000+8000", 2400, 1e-4, False),
+                                             ("300+4800", 1000, 1e-10, True), ("300+4800", 2400, 1e-10, False)])
+def test_dc_of_dense_grids_runs_where_it_is_faster(name, K, tol, chip):
+    """On chip a DC solve is one launch beside its set-up, streaming two per
+    iteration; the residual bars are those of test_dc_of_a_dense_grid."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the limits count 152 SMs")
+    g = _grid(name)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    P = g.p_spec * (1 + 0.1 * np.random.default_rng(2).uniform(-1, 1, (K, 1)))
+    before = dpf.dpf_kernel_launches(ws)
+    out = dpf.dpf_dc_solve(y, ws, K, p_spec=torch.tensor(P, device=DEV), tol=tol)
+    assert (dpf.dpf_kernel_launches(ws) - before < 12) == chip
+    assert (out["rel_residual"].cpu().numpy() <= tol).all()
+    for k in range(0, K, K // 4):
+        assert _residual(g, out["va"][k].cpu().numpy(), P[k]) <= (2 if tol < 1e-5 else 10) * tol, k
+
+
+# more cases than SMs of grids that one warp holds: two rows per thread
+@pytest.mark.parametrize("n", [5, 30, 33, 64])
+@pytest.mark.parametrize("tol", [1e-10, 1e-4])
+def test_dc_of_many_small_grids(n, tol):
+    K = 700
+    g = gridgen.make_grid(n, 3, load_scale=0.1)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    P = g.p_spec * (1 + 0.1 * np.random.default_rng(n).uniform(-1, 1, (K, 1)))
+    P[K - 1] = P[0]
+    out = dpf.dpf_dc_solve(y, ws, K, p_spec=torch.tensor(P, device=DEV), tol=tol)
+    va = out["va"].cpu().numpy()
+    assert (out["rel_residual"].cpu().numpy() <= tol).all() and np.array_equal(va[0], va[K - 1])
+    for k in range(0, K, 50):
+        assert _residual(g, va[k], P[k]) <= (2 if tol < 1e-5 else 10) * tol, k
