@@ -159,3 +159,25 @@ def test_dc_of_many_small_grids(n, tol):
     assert (out["rel_residual"].cpu().numpy() <= tol).all() and np.array_equal(va[0], va[K - 1])
     for k in range(0, K, 50):
         assert _residual(g, va[k], P[k]) <= (2 if tol < 1e-5 else 10) * tol, k
+
+
+# rows of the hub staged in 20 to 75 KB beside the passes' static arrays
+@pytest.mark.parametrize("n", [700, 1200, 1500, 1700, 2048, 3000])
+@pytest.mark.parametrize("K", [1, 40])
+def test_fp64_passes_of_a_star(n, K):
+    """The streaming FP64 passes on a bus of n - 1 branches: one step of a solve
+    from the flat start, against the oracle's S_calc through the mismatch."""
+    import oracle
+    from oracle.ybus import grid_ybus
+    g = _star(n)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    out = dict(n_case=K, va=torch.zeros((K, n), dtype=torch.float64, device=DEV),
+               vm=torch.ones((K, n), dtype=torch.float64, device=DEV),
+               loss=torch.zeros(K, dtype=torch.float64, device=DEV))
+    dpf.dpf_solve_batch(y, ws, dpf.SolveOpts(precision=dpf.FP64, max_iter=3, check_every=2, lr=1e-4), **out)
+    Y = grid_ybus(g)
+    for k in (0, K - 1):
+        va, vm = out["va"][k].cpu().numpy(), out["vm"][k].cpu().numpy()
+        loss = oracle.loss_grad(Y, va, vm, g.p_spec, g.q_spec, g.bus_type)[0]
+        assert abs(out["loss"][k].item() - loss) <= 1e-10 * loss
