@@ -2134,7 +2134,14 @@ static int eval_chip_begin(const dpf_ybus* y, dpf_workspace* w, int K, int preci
   return DPF_OK;
 }
 
-// State of an evaluation of grids above RES_MAX_N buses: the caller's state and
+// Whether an evaluation runs on chip: grids up to RES_MAX_N buses, unless the
+// streaming kernels are faster and the workspace has room for their state.
+static bool eval_on_chip(const dpf_ybus* y, const dpf_workspace* w, int K, int precision, bool backward) {
+  if (!y || !y->dev.res_rord) return false;
+  return !w || w->cap_cases < K || eval_pays(y->n, K, precision == DPF_FP64, backward, y->dev.res_longest);
+}
+
+// State of an evaluation by the streaming kernels: the caller's state and
 // injections into the workspace layout (one kernel), outages and the case
 // flags.  No host synchronisation (but for an outage list's check).
 template <class R>
@@ -2240,7 +2247,7 @@ extern "C" int dpf_power(const dpf_ybus* y, dpf_workspace* w, int32_t n_case, co
   dpf::Range nvtx_range("dpf_power");
   clear_error();
   cudaStream_t s = (cudaStream_t)stream;
-  if (y && y->dev.res_rord) {  // (every grid up to RES_MAX_N buses)
+  if (eval_on_chip(y, w, n_case, precision, false)) {
     TRY(eval_chip_begin(y, w, n_case, precision, va, vm, nullptr, nullptr, outage, s));
     EvalCall c = {};
     c.K = n_case;
@@ -2370,7 +2377,7 @@ extern "C" int dpf_loss_backward(const dpf_ybus* y, dpf_workspace* w, int32_t n_
   cudaStream_t s = (cudaStream_t)stream;
   if ((g_series == nullptr) != (b_series == nullptr))
     return fail(DPF_E_INVALID, "g_series and b_series must be given together");
-  if (y && y->dev.res_rord) {  // (every grid up to RES_MAX_N buses)
+  if (eval_on_chip(y, w, n_case, precision, true)) {
     TRY(eval_chip_begin(y, w, n_case, precision, va, vm, p_spec, q_spec, outage, s));
     EvalCall c = {};
     c.K = n_case;

@@ -186,6 +186,23 @@ inline bool dc_pays(int n, long long K, bool f32, int sms, int pairs, int ctas, 
 // Returns a cudaError_t.
 int dc_res_launch(const dpf_ybus* y, const DcRes& c, const DcShape& sh, bool f32, void* stream);
 
+// Whether an evaluation of K cases pays on chip.  A CTA waits for its longest
+// row's warp, and FP64 warps cost the same however few rows they hold; with many
+// cases the streaming kernels hide both.  us, streaming / on chip, gradient
+// FP32, FP64 and (last) S_calc FP64: 300 buses, one of 160 branches x 1,000 224 /
+// 179, 299 / 260, 160 / 134, x 2,400 309 / 327, 432 / 498, 218 / 245; a star of
+// 300 x 1,000 261 / 264, 319 / 400, 183 / 208; of 700 x 100 365 / 206, 452 / 287,
+// 243 / 157, x 1,000 479 / 735, 627 / 1100, 328 / 555; 14 buses x 100,000 461 /
+// 479, 601 / 803, 287 / 344, 33 x 50,000 480 / 447, 673 / 735, 326 / 323; FP64
+// gradients of 2,000 buses, one of 160 branches x 1,000 785 / 865, one of 300 x
+// 600 642 / 697.  S_calc in FP32 is faster on chip throughout.
+inline bool eval_pays(int n, long long K, bool fp64, bool backward, int longest) {
+  if (!fp64 && !backward) return true;
+  const int rows = (n + 31) / 32 * 32;
+  const int most = fp64 && backward && n > 1500 ? 80000 : 120000;
+  return (longest <= 64 || longest * K <= most) && (100 * n >= 55 * rows || K <= 32768);
+}
+
 // Evaluation of whole cases on chip (dpf_eval.cu), one CTA per case: S_calc,
 // or the loss and its adjoint.  Inputs and outputs are the caller's case-major
 // arrays; outputs may be NULL.

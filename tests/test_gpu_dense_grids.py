@@ -181,3 +181,35 @@ def test_fp64_passes_of_a_star(n, K):
         va, vm = out["va"][k].cpu().numpy(), out["vm"][k].cpu().numpy()
         loss = oracle.loss_grad(Y, va, vm, g.p_spec, g.q_spec, g.bus_type)[0]
         assert abs(out["loss"][k].item() - loss) <= 1e-10 * loss
+
+
+@pytest.mark.parametrize("name,K,precision,chip", [("star700", 342, "FP32", True), ("star700", 343, "FP32", False),
+                                                   ("star700", 343, "FP64", False), ("14", 32768, "FP64", True),
+                                                   ("14", 32769, "FP64", False), ("14", 32769, "FP32", False)])
+def test_evaluations_run_where_they_are_faster(name, K, precision, chip):
+    """Gradients by either route against the oracle; an evaluation on chip is
+    one launch, streaming is more.  FP32 bars as in
+    test_evaluation_on_chip_against_oracle, for |Y_ii| of a hub (700 x 100) by
+    the sum's 350 pairs: 1e-3; without room in the workspace it stays on chip."""
+    import oracle
+    from oracle.ybus import grid_ybus
+    g = _grid(name) if name != "14" else gridgen.make_grid(14, 3, load_scale=0.1)
+    Y = grid_ybus(g)
+    y = dpf.dpf_build_ybus(g)
+    rng = np.random.default_rng(5)
+    n, distinct = g.n_bus, 7
+    va, vm = 0.05 * rng.standard_normal((distinct, n)), 1 + 0.02 * rng.standard_normal((distinct, n))
+    at = np.arange(K) % distinct
+    t = lambda a: torch.tensor(a[at], device=DEV)  # noqa: E731
+    for room, on_chip in ((K, chip), (1, True)):
+        ws = dpf.dpf_workspace_create(y, room)
+        before = dpf.dpf_kernel_launches(ws)
+        out = dpf.dpf_loss_backward(y, ws, t(va), t(vm), precision=getattr(dpf, precision))
+        assert (dpf.dpf_kernel_launches(ws) - before == 1) == on_chip
+        tol = 1e-3 if precision == "FP32" else 1e-10
+        for k in (*range(distinct), K - 1):
+            L, ga, gm = oracle.loss_grad(Y, va[at[k]], vm[at[k]], g.p_spec, g.q_spec, g.bus_type)
+            assert abs(out["loss"][k].item() - L) <= 1e-10 * L
+            scale = max(np.abs(ga).max(), np.abs(gm).max())
+            assert np.abs(out["d_va"][k].cpu().numpy() - ga).max() <= tol * scale
+            assert np.abs(out["d_vm"][k].cpu().numpy() - gm).max() <= tol * scale
