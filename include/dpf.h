@@ -296,9 +296,10 @@ int dpf_wait_limit(dpf_workspace* ws, int64_t polls);
  * into o->lanes, o->warps, o->row_blocks, o->pair_cases and o->stage_v.  The batch's
  * inputs are read (as in dpf_solve_begin) but no output is written; a later
  * dpf_solve_begin starts from scratch.  Results are cached in the workspace
- * per (n_case, precision, grid, outage/injection layout).  Synchronises
- * `stream`.  Returns at once, options unchanged, for batches that iterate on
- * chip (see dpf_solve_iterate): the two passes' launch shape isn't used. */
+ * per (n_case, precision, grid, outage/injection layout, check interval).
+ * Synchronises `stream`.  Batches that iterate on chip (see dpf_solve_iterate)
+ * are not timed: they get the automatic shape, with nothing staged, which only
+ * sets the order of their loss sum. */
 int dpf_autotune(const dpf_ybus* y, dpf_workspace* ws, const dpf_batch* b, dpf_solve_opts* o,
                  int32_t iters, void* stream);
 

@@ -2014,7 +2014,7 @@ extern "C" int dpf_autotune(const dpf_ybus* y, dpf_workspace* w, const dpf_batch
   if (iters < 1) return fail(DPF_E_INVALID, "iters must be >= 1");
   cudaStream_t s = (cudaStream_t)stream;
   const std::vector<long long> key = {b->n_case, o->precision, (long long)y->n, y->nnz, b->outage != nullptr,
-                                      b->p_spec != nullptr};
+                                      b->p_spec != nullptr, o->check_every};
   for (auto& kv : w->tune_cache)
     if (kv.first == key) {
       o->lanes = kv.second[0];
