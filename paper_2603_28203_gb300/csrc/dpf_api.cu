@@ -241,6 +241,7 @@ extern "C" int dpf_ybus_upload(dpf_ybus* y, void* stream) {
     const double dii = dcval[y->idpos[i]];
     dcinv2[i] = pair(dii != 0.0 ? 1.0 / dii : 0.0);
   }
+  for (int i = 0; i < n; ++i) d.longest = std::max(d.longest, (y->irow_ptr[i + 1] - y->irow_ptr[i] + 1) / 2);
   SellY sell;
   if (n <= RES_MAX_N) build_sell(y, dcval2, dcinv2, sell);
   // one allocation and one copy for all of them
@@ -266,7 +267,6 @@ extern "C" int dpf_ybus_upload(dpf_ybus* y, void* stream) {
     add(&d.res_slot, sell.slot);
     d.res_slices = (int)sell.soff.size() - 1;
     d.res_pairs = sell.soff.back();
-    d.res_longest = sell.soff[1];
   }
   add(&d.ent32, ent);
   add(&d.row_ptr, y->irow_ptr);
@@ -2138,7 +2138,7 @@ static int eval_chip_begin(const dpf_ybus* y, dpf_workspace* w, int K, int preci
 // streaming kernels are faster and the workspace has room for their state.
 static bool eval_on_chip(const dpf_ybus* y, const dpf_workspace* w, int K, int precision, bool backward) {
   if (!y || !y->dev.res_rord) return false;
-  return !w || w->cap_cases < K || eval_pays(y->n, K, precision == DPF_FP64, backward, y->dev.res_longest);
+  return !w || w->cap_cases < K || eval_pays(y->n, K, precision == DPF_FP64, backward, y->dev.longest);
 }
 
 // State of an evaluation by the streaming kernels: the caller's state and

@@ -359,6 +359,13 @@ GridShape grid_shape(const dpf_ybus* y, int K, const LossOrder& lo, int lanes, s
   // thread the gathers, which miss L1, and issue bound both forms: 2 x 100,000
   // 23.3 and 25.2, 96 x 10,000 39.4 and 39.3.
   if ((long long)y->n * K * 16 > (long long)sms * 1024 * 17) return g;
+  // A long row is one lane's chain of reads past L1, with the whole GPU at the
+  // barrier; the streaming kernels stage it in shared memory (one case: read it
+  // through L1).  us per iteration, streaming and here, a bus of 160 and of 320
+  // branches: 2 x 5,000 34.6 / 40.3, 55.5 / 71.6; 4 x 10,000 37.7 / 40.4, 61.0 / 83.7; 1 x
+  // 2,500 35.2 / 36.9, 60.9 / 65.0; but 1 x 10,000 39.3 / 37.5, 67.0 / 63.6, and of 80
+  // 12 x 10,000 28.4 / 25.3, 4 x 2,500 25.1 / 26.5.
+  if (y->dev.longest > 64 && (K > 1 || y->n <= 5000)) return g;
   g.gx = (K + lanes - 1) / lanes;
   const long long nvb = (long long)g.gx * lo.gy;
   g.ctas = (int)std::min<long long>(sms, nvb);

@@ -71,7 +71,7 @@ struct DeviceYbus {
   uint16_t* res_puser = nullptr;
   int32_t* res_slot = nullptr;  // [nnz] CSR entry -> its value's index in res_val32 / res_val64
   int res_pairs = 0, res_slices = 0;
-  int res_longest = 0;          // entry pairs of the longest slice (half the longest row)
+  int longest = 0;              // entry pairs of the longest row (any grid)
 };
 
 }  // namespace dpf

@@ -575,7 +575,7 @@ ResShape res_shape(const dpf_ybus* y, int K, bool fp64, bool refined, const Loss
     ctas = std::max(1, most / (int)(sh.smem + 1024));
     ctas_free = 1024 / res_cta_threads<float>(sh.T);
   }
-  sh.ok = res_pays_dense(n, K, fp64, sms, d.res_pairs, d.res_longest, ctas, ctas_free);
+  sh.ok = res_pays_dense(n, K, fp64, sms, d.res_pairs, d.longest, ctas, ctas_free);
   return sh;
 }
 

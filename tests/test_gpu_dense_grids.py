@@ -213,3 +213,26 @@ def test_evaluations_run_where_they_are_faster(name, K, precision, chip):
             scale = max(np.abs(ga).max(), np.abs(gm).max())
             assert np.abs(out["d_va"][k].cpu().numpy() - ga).max() <= tol * scale
             assert np.abs(out["d_vm"][k].cpu().numpy() - gm).max() <= tol * scale
+
+
+@pytest.mark.parametrize("n,degree,K,whole", [(3000, 100, 4, True), (3000, 160, 4, False), (3000, 160, 1, False),
+                                              (6000, 160, 1, True), (6000, 160, 2, False)])
+def test_whole_gpu_iterations_of_a_hub(n, degree, K, whole):
+    """A bus of more than about 128 branches runs streaming, with the same bits."""
+    g = _hub(n, degree)
+    y = dpf.dpf_build_ybus(g)
+    ws = dpf.dpf_workspace_create(y, K)
+    opts = dpf.SolveOpts(precision=dpf.FP32, max_iter=40, check_every=20, lr=1e-3, use_graph=0)
+    va = []
+    for streaming in (False, True):
+        out = dict(n_case=K, va=torch.zeros((K, n), dtype=torch.float64, device=DEV),
+                   vm=torch.ones((K, n), dtype=torch.float64, device=DEV))
+        dpf.dpf_profile_enable(ws, streaming)
+        dpf.dpf_solve_begin(y, ws, opts, **out)
+        before = dpf.dpf_kernel_launches(ws)
+        dpf.dpf_solve_iterate(ws, 20)
+        assert (dpf.dpf_kernel_launches(ws) - before <= 6) == (whole and not streaming)
+        dpf.dpf_solve_iterate(ws, 20)
+        dpf.dpf_solve_end(ws, **out)
+        va.append(out["va"])
+    assert torch.equal(va[0], va[1])
