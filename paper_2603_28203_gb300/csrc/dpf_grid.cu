@@ -146,9 +146,11 @@ __global__ void __launch_bounds__(GRID_WARPS * 32, 1) k_grid_resident(const Grid
   float* red = reinterpret_cast<float*>(OS + (size_t)q.vb_per_cta * cells);  // [vb][wpb][lanes]
   const unsigned Kp = (unsigned)a.Kp;
   const int kl = lane & (q.lanes - 1), rsub = lane / q.lanes, step = q.wpb * q.rpw;
-  if (__ldcg(a.n_active) == 0) return;  // (the same for every CTA: nothing changes it before the first barrier)
-  // an earlier interval, or another CTA of this one, gave up: the state is lost
-  if (__syncthreads_or(threadIdx.x == 0 && __ldcg(q.err))) return;  // (one read: the whole CTA or none of it)
+  // no case runs (the same for every CTA: nothing changes it before the first
+  // barrier), or an earlier interval or another CTA of this one gave up (the
+  // state is lost); one thread reads, so that the whole CTA leaves or none of it
+  const int gone = threadIdx.x == 0 ? (__ldcg(a.n_active) == 0) | (__ldcg(q.err) != 0) : 0;
+  if (__syncthreads_or(gone)) return;
   const int tasks = q.vb_per_cta * q.wpb;
   // task -> its case, rows i0, i0 + step, ... < r1, and the cell of row 0
   struct Task {
