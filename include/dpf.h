@@ -275,12 +275,12 @@ int dpf_solve_iterate(dpf_workspace* ws, int32_t n_iter, void* stream);
 /* Grids of up to 2,048 buses iterate on chip (a case's state stays in one SM
  * for a whole check interval), a few cases of a larger grid in one kernel over
  * the whole GPU, unless plain, stage_v or stage_y is set or the precision is
- * DPF_MIXED; FP64 only up to 320 buses and a few hundred to a few thousand
- * cases.  A few
- * iterations between two tests (or a short dpf_solve_iterate) run in the
- * two-pass kernels where that is faster.  Results
- * are those of the two-pass kernels (FP32, FP32R: to the bit; lanes, warps,
- * row_blocks and pair_cases then only set the order of the loss sum). */
+ * DPF_MIXED.  The two-pass kernels run what they are faster at: FP64 beyond
+ * 320 buses or a few hundred to a few thousand cases, batches of grids with
+ * long rows, a few iterations between two tests (or a short
+ * dpf_solve_iterate).  Results are those of the two-pass kernels (FP32, FP32R:
+ * to the bit; lanes, warps, row_blocks and pair_cases then only set the order
+ * of the loss sum). */
 int dpf_solve_end(dpf_workspace* ws, const dpf_batch* b, void* stream);
 /* The kernel over the whole GPU waits at barriers between its CTAs.  A wait
  * gives up after `polls` polls (0: the default, about a second); the solve then
@@ -412,9 +412,11 @@ int dpf_loss_backward(const dpf_ybus* y, dpf_workspace* ws, int32_t n_case,
  * bridge is DPF_E_ISLANDED) as for dpf_solve_batch.  Conjugate gradients
  * with the Jacobi preconditioner on the GPU, per case until |r| <= tol |r0|
  * or max_iter iterations; the vectors are double-float pairs (~48 bits)
- * for tol < 1e-5 and FP32 for tol >= 1e-5, the per-case scalars FP64
- * (grids above 2,048 buses) or double-float (up to there, where one CTA runs
- * a case's whole solve on chip).  Outputs (caller-owned device
+ * for tol < 1e-5 and FP32 for tol >= 1e-5.  Up to 2,048 buses one CTA runs a
+ * case's whole solve on chip with double-float per-case scalars; larger grids,
+ * and those whose matrix does not fit an SM's shared memory, take two launches
+ * per iteration with FP64 scalars (angles no closer to an FP64 solve, see
+ * csrc/dpf_dc_resident.cu).  Outputs (caller-owned device
  * arrays): va [n_case][n_bus] (required), iters [n_case] and rel_residual
  * [n_case] (|r| / |r0| at the stop; either may be NULL).  Uses (and
  * resets) the workspace like the other calls. */

@@ -16,10 +16,16 @@
 // are double-float as well (FP64 issue is dear here, and every warp forms
 // them from the warps' partial sums).
 // Error of the angles against a dense FP64 solve, rms over the batch relative
-// to the largest angle, at a relative residual of 1e-10 (streaming form with
-// FP64 scalars, here): 3,000 cases of 30 buses 1.7e-14, 1.1e-14; 1,000 of 300
-// 6.5e-13, 3.7e-13; 1,000 of 1,000 2.7e-12, 2.4e-12; 400 of 2,000 5.3e-12,
-// 5.2e-12: the stop test's, not the arithmetic's.
+// to the largest angle, by the relative residual asked for (streaming form with
+// FP64 scalars and q as a recurrence / here; cases x buses):
+//             1e-4             1e-10              1e-14
+//   3,000 x 30    1.3e-6 / 1.3e-6  1.8e-14 / 1.0e-14  1.8e-14 / 1.0e-14
+//   1,000 x 300   1.3e-5 / 9.8e-6  6.8e-13 / 3.7e-13  6.2e-13 / 2.6e-13
+//   1,000 x 1,000 3.5e-5 / 2.8e-5  2.6e-12 / 2.3e-12  1.3e-12 / 3.7e-13
+//   400 x 2,000   1.3e-5 / 8.0e-6  3.8e-12 / 3.8e-12  6.6e-13 / 2.4e-13
+// so the double-float scalars cost nothing (at 1e-10 and above the error is the
+// stop test's); what the recurrence lost, the direct product keeps.  Totals in
+// three floats took 20-39% longer, in fixed point 50-100%, with the same errors.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -105,8 +111,9 @@ template <> __device__ __forceinline__ float4 pair_to<float2>(float4 v) { return
 template <> __device__ __forceinline__ float2 pair_to<float>(float4 v) { return make_float2(v.x, v.z); }
 
 // Every thread's rows are the positions tid + s * T.  What bounds it is issue
-// of the (emulated) arithmetic, about 330 instructions per row and iteration
-// in double-float, a quarter of them the two reductions.  Milliseconds for
+// of the (emulated) arithmetic, 286 instructions per 32 rows and iteration in
+// double-float (issue 68%, FMA pipe 48%, shared memory 51%), 121 in FP32 (48%,
+// 20%, 49%), a quarter of them the two reductions.  Milliseconds for
 // 2,379 outages of a 2,000-bus grid to 1e-10 (double-float) and 1e-4 (FP32):
 // streaming 119.5 and 48; four rows per thread and one CTA per SM 47.8 and
 // 20.7; eight rows and two CTAs 57.7 (spills) and 15.8; two rows of 1,024

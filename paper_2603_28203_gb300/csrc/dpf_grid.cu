@@ -3,12 +3,13 @@
 // launch per test interval.
 //
 // The streaming kernels spend two launches per iteration on such batches, most
-// of it launch and drain latency (one case of 100,000 buses: 18.7 us for 6 MB
+// of it launch and drain latency (one case of 100,000 buses: 17.3 us for 6 MB
 // of state).  Here every SM runs one CTA that keeps its rows' master values
 // and moments in shared memory for the whole interval; only V and w, which
 // other SMs gather, live in L2 (read past L1, which is not coherent).  Two
-// grid barriers (about 1.6 us each) separate the passes: 14.9 us.  What bounds
-// it is the chain of L2 reads of a pass and the barriers.
+// grid barriers (about 1.6 us each) separate the passes: 11.3 us.  What bounds
+// it is the barriers and the chain of L2 reads of a pass (of 28 warp cycles per
+// issue 15 are spent at a barrier, 7 on a load; issue 22%, L2 13%).
 //
 // Work is split as the streaming forward pass splits it: virtual blocks (case
 // tile x row block) of `wpb` warps, dealt to the CTAs, a warp per virtual
@@ -355,11 +356,13 @@ GridShape grid_shape(const dpf_ybus* y, int K, const LossOrder& lo, int lanes, s
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // About one element per thread of the GPU: there an iteration is launch and
-  // drain latency.  us per iteration, streaming and here: 1 x 100,000 buses
-  // 20.7 and 14.9, 1 x 20,000 16.0 and 12.4, 8 x 10,000 17.4 and 14.4, 60 x
-  // 2,500 18.5 and 16.3, 4 x 40,000 20.0 and 19.8.  With more elements per
-  // thread the gathers, which miss L1, and issue bound both forms: 2 x 100,000
-  // 23.3 and 25.2, 96 x 10,000 39.4 and 39.3.
+  // drain latency.  us per iteration without the tests, streaming and here:
+  // 1 x 100,000 buses 17.3 and 11.3, 1 x 20,000 13.2 and 9.5, 8 x 10,000 13.6
+  // and 11.5, 16 x 10,000 15.6 and 13.0, 60 x 2,500 15.3 and 12.5, 4 x 40,000
+  // 15.8 and 13.8.  With more elements per thread the gathers, which miss L1,
+  // and issue bound both forms, and the gain shrinks: 2 x 100,000 18.9 and 17.7,
+  // 96 x 10,000 32.5 and 29.5 with the limit lifted (it was set when this form
+  // took 25.2 and 39.3 there; where it should lie now is not measured).
   if ((long long)y->n * K * 16 > (long long)sms * 1024 * 17) return g;
   // A long row is one lane's chain of reads past L1, with the whole GPU at the
   // barrier; the streaming kernels stage it in shared memory (one case: read it

@@ -25,7 +25,11 @@
 // iteration streaming, 80 us on chip.  What bounds it now is instruction issue
 // (60% of the slots, 404 instructions per 32 rows and iteration), then the
 // shared-memory pipe (57%: two rows of 8-byte gathers at random banks).  8,192
-// cases of 30 buses: 15.9 -> 8.2 us; one case of 30 buses in FP64: 17.8 -> 8.7.
+// cases of 30 buses: 15.9 -> 8.1 us (issue 64%, 612 instructions per case and
+// iteration, 31% of the warps); one case of 30 buses in FP64: 17.8 -> 8.7 (a
+// dependent chain: 9 of 13 warp cycles per issue wait for a fixed latency).
+// Batches, grids and spans for which the streaming kernels are faster are
+// given to them (res_pays, res_pays_dense, res_min_span).
 //
 // The results are those of the streaming kernels to the bit: the same device
 // functions on the same operands, each row's products in the same order, and
