@@ -285,8 +285,8 @@ int dpf_solve_end(dpf_workspace* ws, const dpf_batch* b, void* stream);
 /* The kernel over the whole GPU waits at barriers between its CTAs.  A wait
  * gives up after `polls` polls (0: the default, about a second); the solve then
  * ends with DPF_E_CUDA from dpf_active_count, dpf_solve_end or dpf_solve_batch
- * and no outputs.  dpf_solve_end therefore synchronises `stream` for such
- * solves (unless it is being captured). */
+ * and no outputs.  dpf_solve_end therefore synchronises `stream` where
+ * that kernel ran (unless the stream is being captured). */
 int dpf_wait_limit(dpf_workspace* ws, int64_t polls);
 /* Autotuner.  Times candidate launch shapes of the solve loop on this batch
  * -- cases per row group (`lanes`, i.e. rows per warp = 32/lanes), warps per

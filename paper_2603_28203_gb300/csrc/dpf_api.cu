@@ -400,6 +400,7 @@ struct dpf_workspace {
   unsigned* grid_sus = nullptr;
   unsigned* grid_bar = nullptr;
   int64_t grid_polls = GRID_POLLS;
+  bool grid_used = false;   // this solve launched it (its error word counts)
   bool pid_ready = false;  // operating points staged by dpf_paramid_begin
   std::vector<std::pair<std::vector<long long>, std::vector<int>>> tune_cache;  // key -> (lanes, warps, rb, pairs)
   bool spec_per_case = false, has_outage = false;
@@ -899,15 +900,16 @@ static int launch_span(dpf_workspace* w, cudaStream_t s, int n, bool with_check)
   CK((cudaError_t)whole_or_streaming(
       w->grid,
       [&] {
-        w->launches++;
-        return grid_launch(make_plan<float>(w).it, w->grid, w->res_lo, w->lanes, w->K, n, w->precision == DPF_FP32R,
-                           w->grid_terms, w->grid_sus, w->grid_bar, w->n_active + 1, w->grid_polls, s);
+        const int e = grid_launch(make_plan<float>(w).it, w->grid, w->res_lo, w->lanes, w->K, n,
+                                  w->precision == DPF_FP32R, w->grid_terms, w->grid_sus, w->grid_bar, w->n_active + 1,
+                                  w->grid_polls, s);
+        if (e == cudaSuccess) {
+          w->launches++;
+          w->grid_used = true;
+        }
+        return e;
       },
-      [&] {
-        w->launches--;
-        cudaGetLastError();
-      },
-      streaming));
+      [&] { cudaGetLastError(); }, streaming));
   return rc;
 }
 
@@ -1652,6 +1654,7 @@ extern "C" int dpf_solve_begin(const dpf_ybus* y, dpf_workspace* w, const dpf_ba
     w->launches++;
   }
   w->t_done = 0;
+  w->grid_used = false;
   w->begun = true;
   return DPF_OK;
 }
@@ -1852,7 +1855,7 @@ extern "C" int dpf_solve_end(dpf_workspace* w, const dpf_batch* b, void* stream)
   cudaStream_t s = (cudaStream_t)stream;
   const dpf_ybus* y = w->y;
   const bool hio = b->host_io != 0;
-  if (w->grid.ok) {  // a barrier that gave up leaves no state to return (a stream being captured cannot be waited for)
+  if (w->grid_used) {  // a barrier that gave up leaves no state to return (a stream being captured cannot be waited for)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     CK(cudaStreamIsCapturing(s, &cap));
     if (cap == cudaStreamCaptureStatusNone) {
