@@ -44,21 +44,21 @@ struct GridArgs {
   unsigned* suspect;      // [Kp]
   unsigned* bar;          // arrivals of this launch, whether a case is suspect (both zeroed)
   int32_t* err;           // a barrier gave up (sticky for the solve)
-  long long polls;        // of a barrier before it gives up
+  int polls;              // of a barrier before it gives up
 };
 
 constexpr int GRID_WARPS = 32;  // of a CTA at most
 
 // Grid barrier number `gen` (1, 2, ...): 0 if it gave up, else 1 + the word
 // beside the counter (whether any case is suspect).
-__device__ __forceinline__ int grid_barrier(unsigned* bar, unsigned gen, int32_t* err, long long polls) {
+__device__ __forceinline__ int grid_barrier(unsigned* bar, unsigned gen, int32_t* err, int polls) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     const unsigned want = gen * gridDim.x;
     __threadfence();
     atomicAdd(bar, 1u);
-    long long n = 0;
+    int n = 0;
     unsigned v;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
@@ -410,7 +410,7 @@ int grid_launch(const IterArgs<float>& a, const GridShape& g, const LossOrder& l
   q.suspect = suspect;
   q.bar = bar;
   q.err = err;
-  q.polls = polls;
+  q.polls = (int)std::min<int64_t>(polls, 1 << 30);
   const bool adam = a.opt == OPT_ADAM;
   auto kern = refined ? (adam ? k_grid_resident<true, true> : k_grid_resident<true, false>)
                       : (adam ? k_grid_resident<false, true> : k_grid_resident<false, false>);
